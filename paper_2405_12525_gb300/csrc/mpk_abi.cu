@@ -187,6 +187,15 @@ KArgs mpk::base_args(Plan &P, int32_t p) {
         a.w_chunk_nsl = P.w_chunk_nsl;
         a.ngroups = P.num_groups;
     }
+    if (P.wave) {
+        a.v_cell = P.v_cell + P.v_cell_off[p];
+        a.v_ncells = P.v_cell_off[p + 1] - P.v_cell_off[p];
+        a.slice_row = P.slice_row;
+        a.v_gsl = P.v_gsl;
+        a.v_count = P.v_count;
+        a.v_ngroups = P.v_ngroups;
+        a.v_maxsl = P.v_maxsl;
+    }
     return a;
 }
 

@@ -286,7 +286,17 @@ struct KArgs {
     const int32_t *w_chunk_nsl;    // slices of every chunk
     int32_t ngroups;
     int32_t p_launch;              // powers of this launch (local 1..p_launch)
+    // wave kernel (static schedule): the cells of this launch in line order as (first slice,
+    // slices, g << 5 | k, 0), the rows of every slice, the slices of every group and the finished
+    // slices per (power, group); zero when the launch starts
+    const int4 *v_cell;
+    const int32_t *slice_row;  // slices + 1
+    const int32_t *v_gsl;
+    int32_t *v_count;          // (p + 1) x v_ngroups
+    int32_t v_ncells, v_ngroups;
+    int32_t v_maxsl;           // slices of the largest group
 };
+constexpr int kWaveMaxCells = 1 << 20;  // cells of a wave launch (a descriptor holds 21 bits)
 // warp-ticketed engine: slices per item, claim queues (one per warp of a block)
 constexpr int kWarpSlices = 1;
 constexpr int kWarpQueues = 16;
@@ -341,6 +351,12 @@ struct Plan {
     int32_t *w_cnt = nullptr;           // (p_max+1) x nchunks counters, then kWarpQueues claim counters
     int32_t *w_slice_chunk = nullptr;   // chunk of every slice (device)
     int32_t *w_chunk_nsl = nullptr;     // slices of every chunk (device)
+    // wave kernel (single plans of the staged engine at the planner's own block shape)
+    bool wave = false;
+    int32_t v_ngroups = 0, v_maxsl = 0;
+    int4 *v_cell = nullptr;             // cells of every p, concatenated
+    std::vector<int32_t> v_cell_off;    // pmax + 2: the cells of p start at v_cell_off[p]
+    int32_t *slice_row = nullptr, *v_gsl = nullptr, *v_count = nullptr;
     int32_t drop_unit = -1;  // armed by mpk_debug_drop_release for the next launch
     unsigned long long *trace = nullptr;  // counters when built with opts.trace
     int grid_mpk[4] = {0, 0, 0, 0};  // persistent grid size per mode

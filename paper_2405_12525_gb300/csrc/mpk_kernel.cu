@@ -12,6 +12,7 @@
 // a row are issued before its FMAs.  The result equals the oracle's fma-per-term row sums
 // bit for bit.
 #include "mpk_kernel_dev.cuh"
+#include "mpk_wave.cuh"
 
 #include <type_traits>
 
@@ -505,8 +506,31 @@ static int occupancy_grid_w(int mode, int m, int vtype) {
     return c;
 }
 
+// The wave kernel for (mode, width, value type, accumulator), ready to launch, and its shared memory
+static void *select_wave(int mode, int m, int vtype, bool a32, int *smem) {
+    static bool ready[3][3][5][2] = {};  // width index: log2 of m
+    if (vtype < 0 || vtype > 2 || mode < 0 || mode > 2) fail(MPK_ERR_UNSUPPORTED, "value type %d, mode %d", vtype, mode);
+    void *fn = vtype == MPK_F64 ? select_wave_f64(mode, m, a32, smem)
+                                : (vtype == MPK_F32 ? select_wave_f32(mode, m, a32, smem)
+                                                    : select_wave_bf16(mode, m, a32, smem));
+    bool &r = ready[vtype][mode][__builtin_ctz((unsigned)m)][a32 ? 1 : 0];
+    if (!r) {
+        MPK_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, *smem));
+        r = true;
+    }
+    return fn;
+}
+
 void launch_mpk(const Plan &P, KArgs &a, int mode, cudaStream_t s) {
     const bool a32 = P.accum == MPK_F32;
+    if (P.wave && a.v_cell != nullptr && a.drop_unit < 0) {
+        const int grid = std::min(device_sms(), a.v_maxsl);
+        int smem = 0;
+        void *fn = select_wave(mode, P.m, P.val_type, a32, &smem);
+        void *args[] = {&a};
+        MPK_CUDA(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kWaveBS), args, (size_t)smem, s));
+        return;
+    }
     if (P.engine == MPK_ENGINE_SWEEP && a.trace == nullptr && a.drop_unit < 0 && a.w_item == nullptr) {
         if (P.num_chunks <= 0) return;
         void *fn = select_sweep(mode, P.m, P.val_type, a32);

@@ -331,6 +331,84 @@ void export_csr(const Plan &P, int32_t *rp, int32_t *ci, double *va, cudaStream_
     MPK_CUDA(cudaStreamSynchronize(s));
 }
 
+// Tables of the wave kernel.  A matrix within the cache budget beside four of its vectors is one group
+// (each power is one cell); others keep the plan's groups.  The plan goes without (and runs k_mpk)
+// when a chunk reads rows outside its own group and the two beside it, which the kernel's
+// dependency rule does not cover (levels of another matrix), when there are too many cells, or
+// when the tables do not fit the memory budget.
+static void plan_wave(Plan &P, const std::vector<int32_t> &g_slice, const std::vector<int32_t> &c_slice,
+                      const std::vector<int64_t> &sptr, const std::vector<int2> &hull, const int32_t *slice_row,
+                      bool default_budget, std::vector<int32_t> &host, cudaStream_t s) {
+    const int32_t G = P.num_groups, NS = P.num_slices, pmax = P.p_max;
+    if (P.padded / 32 >= INT32_MAX) return;
+    // groups as runs of the plan's: the kernel's cells pay for a larger budget than k_mpk's, since a
+    // block's share of a cell is what hides the cell's hand-over to the next power
+    const int64_t wave_cache = default_budget ? device_l2_bytes() / 4 * 5 : P.cache_bytes;
+    const int64_t mat = (P.val_bytes + 4) * P.padded, vec = (int64_t)8 * P.n * P.m;
+    const bool one = P.identity || mat + 4 * vec <= P.cache_bytes;
+    std::vector<int32_t> vs(1, 0);  // first slice of every group, and the end
+    const int64_t most = wave_cache / P.window;
+    int64_t bytes = 0;
+    for (int32_t g = 0; g < G && !one; ++g) {
+        const int64_t b = (P.val_bytes + 4) * (sptr[g_slice[g + 1]] - sptr[g_slice[g]]) +
+                          (4 + 16 * (int64_t)P.m) * 32 * (g_slice[g + 1] - g_slice[g]);
+        if (g > 0 && bytes + b > most) {
+            vs.push_back(g_slice[g]);
+            bytes = 0;
+        }
+        bytes += b;
+    }
+    vs.push_back(NS);
+    const int32_t VG = (int32_t)vs.size() - 1;
+    const int64_t ncell = (int64_t)VG * pmax * (pmax + 1) / 2;
+    if ((int64_t)VG * pmax >= kWaveMaxCells || ncell > (1 << 22)) return;
+    if (!one) {
+        if ((int32_t)hull.size() != P.num_chunks) return;
+        // (c_slice ascends: chunk c starts at slice c_slice[c])
+        std::vector<int32_t> vc0((size_t)VG + 1);  // first chunk of every group
+        for (int32_t g = 0; g <= VG; ++g)
+            vc0[g] = (int32_t)(std::lower_bound(c_slice.begin(), c_slice.end(), vs[g]) - c_slice.begin());
+        for (int32_t g = 0; g < VG; ++g) {
+            const int32_t lo = vc0[std::max(g - 1, 0)], hi = vc0[std::min(g + 2, VG)];
+            for (int32_t c = vc0[g]; c < vc0[g + 1]; ++c)
+                if (hull[c].x < lo || hull[c].y >= hi) return;
+        }
+    }
+    // one block of device memory: cells, rows of the slices, slices of the groups, counters (zero)
+    const int64_t ncount = (int64_t)(pmax + 1) * VG;
+    const int64_t words = 4 * ncell + ((int64_t)NS + 1) + VG + ncount;
+    if (P.arena.budget > 0 && P.arena.bytes + 4 * words > P.arena.budget) return;
+    host.assign((size_t)(4 * ncell + VG), 0);  // the caller keeps it until the copies are done
+    int32_t *vc = host.data(), *gsl = host.data() + 4 * ncell;
+    for (int32_t g = 0; g < VG; ++g) gsl[g] = vs[g + 1] - vs[g];
+    P.v_maxsl = *std::max_element(gsl, gsl + VG);
+    P.v_cell_off.assign((size_t)pmax + 2, 0);
+    int32_t c = 0;
+    for (int32_t p = 1; p <= pmax; ++p) {  // lines g + kSlotSkew * k ascending, k ascending inside a line
+        P.v_cell_off[p] = c;
+        for (int32_t d = kSlotSkew; d <= VG - 1 + kSlotSkew * p; ++d)
+            for (int32_t k = 1; k <= p; ++k) {
+                const int32_t g = d - kSlotSkew * k;
+                if (g < 0 || g >= VG) continue;
+                vc[4 * (int64_t)c] = vs[g];
+                vc[4 * (int64_t)c + 1] = gsl[g];
+                vc[4 * (int64_t)c + 2] = (g << 5) | k;
+                ++c;
+            }
+    }
+    P.v_cell_off[pmax + 1] = c;
+    P.v_ngroups = VG;
+    int32_t *dev = P.arena.alloc_n<int32_t>(words);
+    P.v_cell = reinterpret_cast<int4 *>(dev);
+    P.v_gsl = dev + 4 * ncell;
+    P.v_count = P.v_gsl + VG;
+    P.slice_row = P.v_count + ncount;
+    MPK_CUDA(cudaMemcpyAsync(dev, host.data(), sizeof(int32_t) * host.size(), cudaMemcpyHostToDevice, s));
+    MPK_CUDA(cudaMemsetAsync(P.v_count, 0, sizeof(int32_t) * (size_t)ncount, s));
+    MPK_CUDA(cudaMemcpyAsync(P.slice_row, slice_row, sizeof(int32_t) * ((size_t)NS + 1), cudaMemcpyDeviceToDevice, s));
+    P.wave = true;
+}
+
 Plan *build_plan(const mpk_csr *A, const Levels *L, const mpk_plan_opts *o, cudaStream_t s,
                  const std::vector<int32_t> *inst_row, const std::vector<int32_t> *inst_p) {
     if (!o) fail(MPK_ERR_INVALID, "options are NULL");
@@ -596,6 +674,7 @@ Plan *build_plan(const mpk_csr *A, const Levels *L, const mpk_plan_opts *o, cuda
         MPK_CUDA(cudaMemsetAsync(P->col, 0xff, sizeof(int32_t) * (size_t)(P->padded + 32), s));  // padding: col = -1
 
         std::vector<int32_t> c_row, c_slice, g_chunk;
+        std::vector<int2> chunk_hull;  // first and last chunk of each chunk's dependencies
         std::vector<int32_t> h_win;  // shape 3: kXWin (first row, rows, position) per chunk
         int32_t NC = 0, stage_entries = 0;
         for (int attempt = 0;; ++attempt) {
@@ -668,7 +747,8 @@ Plan *build_plan(const mpk_csr *A, const Levels *L, const mpk_plan_opts *o, cuda
             // ---- dependency ranges: exact chunk sets as bitmaps over each hull, compressed
             P->dep_ranges = P->arena.alloc_n<int4>(2 * (int64_t)(NC > 0 ? NC : 1));
             if (NC > 0) {
-                std::vector<int2> hull((size_t)NC);
+                std::vector<int2> &hull = chunk_hull;
+                hull.resize((size_t)NC);
                 MPK_CUDA(cudaMemcpyAsync(hull.data(), P->dep, sizeof(int2) * (size_t)NC, cudaMemcpyDeviceToHost, s));
                 MPK_CUDA(cudaStreamSynchronize(s));
                 std::vector<int64_t> woff((size_t)NC + 1, 0);
@@ -1011,6 +1091,11 @@ Plan *build_plan(const mpk_csr *A, const Levels *L, const mpk_plan_opts *o, cuda
         P->work_slots = std::max(pmax + 1, 4);  // all powers (original order) or ring of 3 + accumulator
         P->work = P->arena.alloc_n<double>((int64_t)P->work_slots * n * m + 1);
         if (P->accum == MPK_F32) P->shadow = P->arena.alloc_n<float>(2 * (int64_t)n * m + 1);
+        std::vector<int32_t> wave_host;
+        // ---- wave kernel: single plans of the staged engine whose block shape the planner chose
+        if (o->engine == MPK_ENGINE_STAGED && o->shape == 0 && !batch && !P->level_capped && !P->split_levels &&
+            !o->trace && o->shuffle_seed == 0 && n > 0)
+            plan_wave(*P, g_slice, c_slice, sptr, chunk_hull, d_srow.p, o->cache_bytes == 0, wave_host, s);
         MPK_CUDA(cudaStreamSynchronize(s));  // host vectors above must outlive their copies
     } catch (...) {
         P->arena.release();

@@ -1,0 +1,623 @@
+// The wave kernel: level-blocked powers on a static schedule (device code; instantiated per
+// value type in mpk_wave_f64.cu, mpk_wave_f32.cu and mpk_wave_bf16.cu).
+#pragma once
+#include "mpk_kernel_dev.cuh"
+
+namespace mpk {
+
+// What bounds it.  An FP64 FMA holds an SM quarter's pipe for 67 cycles (0.594 T FMA/s measured on
+// all SMs), so 256^3, p = 8 needs 1.58 ms of it; k_mpk's units (claimed through a ticket, handed
+// over block-wide, 8 FMA slots for a row of 7 entries) took 2.08 ms.  Here nothing is claimed and
+// nothing handed over block-wide, a row takes exactly its slice's width of FMAs, and 28 warps
+// work on as many slices: 1.99 ms; binary32 sums, bound by instruction issue and the latency of the
+// gathers: 1.45 -> 1.33 ms.  Blocks of right-hand sides, where k_mpk's gathers of one column at a
+// time made L1 the bound: 100^3 27-point stencil, 8 columns, p = 8: 4.21 -> 3.42 ms.
+//
+// One cooperative launch, one block per SM.  The Lp-diagram cells (group g, power k) are walked
+// in line order, as k_mpk does; every cell's 32-row slices are divided evenly over the blocks,
+// so nothing is claimed at run time and a slice is the unit of work: a compute warp waits for
+// nothing but its own entries and the cell's dependencies.
+//
+// Warp roles of a block:
+//  - warp 0 (dispatcher) lists the block's slices of every cell in schedule order in a ring of
+//    descriptors in shared memory, 32 a step;
+//  - warp 1 (loader) copies the entries of the listed slices into a circular buffer in shared
+//    memory, a tile of up to 32 slices on one mbarrier, with one pair of bulk copies per run of
+//    neighbouring slices.  The copies need no dependency and run ahead of the cells by the
+//    buffer's size;
+//  - warp 2 (poller) reads the completion counters of the cells that the next 32 cells depend on
+//    (relaxed loads, then one acquire fence for all that became ready) and stores how many
+//    cells may run in s_ready;
+//  - warp 3 (publisher) sees from the warps' progress words which cells the block has finished,
+//    issues one fence at GPU scope for all of them and adds the block's slices to the cells'
+//    counters;
+//  - the others compute.  A lane owns one (row, right-hand side) pair, so a slice is M units of
+//    32 / M rows, and warp w takes the units w, w + W, ...: it waits for the slice's tile and
+//    cell, gathers x and runs the row sums.
+// A cell (g, k) is ready when the cells (g-1 .. g+1, k-1) are complete: groups are whole levels,
+// and a row reads its own level and the two beside it.  The same wait covers what the cell
+// overwrites in the rings of the recurrence (three blocks) and of the binary32 copy (two).
+//
+// With lanes along the right-hand sides a gather reads whole rows of x (8 M consecutive bytes)
+// instead of one column of 32 rows, which would touch 32 lines an instruction and make L1 the
+// bound from M = 4 on.
+//
+// Deadlock freedom: every block is resident (cooperative launch); cells are dispatched, polled,
+// computed and published in one order, and a cell depends on earlier cells only, so the first
+// unfinished cell can always run.  Every wait is bounded by a.wait_ns (globaltimer); on expiry
+// the launch's epoch and MPK_ERR_TIMEOUT are recorded in a.err, all blocks leave, and no block
+// leaves with a bulk copy of its own in flight.
+//
+// The counters start at zero: the last block whose poller and publisher are done (nothing is
+// polled or published after that) clears them for the next launch, and stores the epoch, while
+// the compute warps still finish the last power, whose cells nothing waits for.
+constexpr int kWaveAux = 4;     // dispatcher, loader, poller, publisher
+constexpr int kWaveWarps = 28;  // compute warps: 16 / 20 / 24 / 28 took 2.34 / 2.15 / 2.03 / 1.99 ms at 256^3, p = 8
+constexpr int kWaveBS = 32 * (kWaveWarps + kWaveAux);
+constexpr int kBatch = 8;       // entries of a row whose x values are gathered together
+constexpr int kDescRing = 512;  // slice descriptors in shared memory
+constexpr int kWaveTiles = 32;  // tiles in shared memory or in flight
+// Entries of the circular buffer, of the widest slice it takes (a wider one is read from global
+// memory) and of a tile.  A slice that starts near the end of the buffer runs on past it, into
+// room for one slice.
+template <class VT> struct WaveBuf {
+    static constexpr int ENTRY = (int)sizeof(typename VT::T) + 4;
+    static constexpr int SLICE = 32 * 64;
+    static constexpr int CAP = (200 * 1024 / ENTRY - SLICE) / 256 * 256;
+    static constexpr int TILE = CAP / 3;
+    static constexpr int ALL = CAP + SLICE + 32 * kBatch;  // a batch may read past its slice
+    static_assert(TILE >= SLICE, "a slice fits a tile");
+};
+
+struct __align__(16) WaveDesc {
+    int32_t e32;    // first entry of the slice / 32
+    int32_t width;  // entries a row; top bit: first of a run of neighbouring slices
+    int32_t row0;
+    uint32_t ckr;   // cell << 11 | power << 6 | rows
+};
+
+__device__ __forceinline__ int ld_acquire_cta_shared(const int *p) {
+    int v;
+    asm volatile("ld.acquire.cta.shared.b32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release_cta_shared(int *p, int v) {
+    asm volatile("st.release.cta.shared.b32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
+}
+
+// Bound of a wait, for use in its spin loop only: the first call starts the clock, and the clock
+// (slow to read) is looked at every 64 calls.
+struct Deadline {
+    uint64_t t0 = 0;
+    int calls = 0;
+    __device__ __forceinline__ bool expired(int64_t limit_ns) {
+        if (calls++ & 63) return false;
+        const uint64_t t = globaltimer();
+        if (t0 == 0) t0 = t;
+        return t - t0 > (uint64_t)limit_ns;
+    }
+};
+
+// the block's share of a cell of nsl slices: [x, y)
+__device__ __forceinline__ int2 wave_share(int nsl, int block, int blocks) {
+    return make_int2((int)((int64_t)nsl * block / blocks), (int)((int64_t)nsl * (block + 1) / blocks));
+}
+
+// Epilogue of one (row, column) of step j at local power k: w is its row sum.  own / back: its
+// values of the two previous steps and old the accumulator (recurrence), or own is x0's value
+// copied to Y[0] (power 1).
+template <int M, int MODE, class AT>
+__device__ __forceinline__ void wave_epilogue(const KArgs &a, int k, int64_t at, bool valid, int lane, AT wa, double own,
+                                              double back, double old) {
+    constexpr bool A32 = sizeof(AT) == 4;
+    const int j = a.k_offset + k;
+    const double w = to_f64(wa);
+    double *y = a.ybase + (int64_t)ring_slot(a, j) * a.ystride + at;
+    if constexpr (MODE == MODE_CHEB) {
+        const double vn = j == 1 ? fma(a.halpha, w, a.hbeta * own) : fma(a.alpha, w, fma(a.beta, own, -back));
+        // complex coefficients act on column pairs, which sit in neighbouring lanes
+        const double other = (M > 1 && a.complex_coeff) ? __shfl_xor_sync(0xffffffffu, vn, 1) : 0.0;
+        if (valid) {
+            *y = vn;
+            if constexpr (A32) a.shadow[(int64_t)(j & 1) * a.ystride + at] = __double2float_rn(vn);
+            double acc = fma(a.cre[k], vn, old);
+            if (M > 1 && a.complex_coeff) acc = fma((lane & 1) ? a.cim[k] : -a.cim[k], other, acc);
+            a.acc[at] = acc;
+        }
+    } else if (valid) {
+        if (!A32 && k == a.p_launch && a.v_ngroups > 1)
+            __stcs(y, w);  // not read again here: see row_epilogue_loaded
+        else
+            *y = w;
+        if constexpr (A32) a.shadow[(int64_t)(j & 1) * a.ystride + at] = (float)wa;
+        if constexpr (MODE == MODE_HOST) __stcs(a.yhost + (int64_t)j * a.ystride + at, w);
+        if (k == 1 && a.y0copy) a.y0copy[at] = own;
+    }
+}
+
+// N entries of the rows of a warp (entry t of a lane's row 32 t places on): their x values are
+// gathered together, then summed in order.  N is exact: an FP64 FMA takes its 64 cycles of the
+// pipe even when no lane of the warp runs it, so sums are never padded to a batch.
+template <int N, int M, class VT, class AT, class VP, class CP>
+__device__ __forceinline__ void wave_batch(VP sv, CP sc, const AT *x, AT &acc) {
+    int c[N];
+    AT xv[N];
+#pragma unroll
+    for (int t = 0; t < N; ++t) {
+        c[t] = sc[32 * t];
+        xv[t] = AT(0);
+        if (c[t] >= 0) xv[t] = x[(int64_t)c[t] * M];
+    }
+#pragma unroll
+    for (int t = 0; t < N; ++t) {
+        const AT v = sv[32 * t];
+        if (c[t] >= 0) acc = afma(v, xv[t], acc);
+    }
+}
+
+template <int M, int MODE, class VT, bool A32>
+__global__ void __launch_bounds__(kWaveBS, 1) k_wave(const KArgs a) {
+    using AT = typename std::conditional<A32, float, double>::type;
+    using T = typename VT::T;
+    constexpr int G = 32 / M;  // rows of a unit
+    using Buf = WaveBuf<VT>;
+    extern __shared__ __align__(128) unsigned char smem[];  // values, then columns
+    T *const sval = reinterpret_cast<T *>(smem);
+    int32_t *const scol = reinterpret_cast<int32_t *>(smem + Buf::ALL * sizeof(T));
+    __shared__ WaveDesc desc[kDescRing];
+    __shared__ uint32_t vpos[kDescRing];  // entries of the buffer's slices before this one, all in all
+    __shared__ int loc[kDescRing];  // where a slice's entries are: offset / 32, tile << 16, phase << 24; -1: global memory
+    __shared__ __align__(8) uint64_t full[kWaveTiles];
+    __shared__ int s_ready, s_pushed, s_loaded, s_total, s_abort, s_left;
+    __shared__ int s_prog[32];  // units finished by each compute warp
+    __shared__ int32_t s_epoch;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int block = blockIdx.x, blocks = gridDim.x;
+    if (tid < 32) s_prog[tid] = 0;
+    if (tid == 0) {
+        s_epoch = (int32_t)ld_relaxed(reinterpret_cast<const int32_t *>(a.epoch_word)) + 1;
+        s_ready = 0;
+        s_pushed = 0;
+        s_loaded = 0;
+        s_total = -1;
+        s_abort = 0;
+        s_left = 0;
+        for (int q = 0; q < kWaveTiles; ++q) mbar_init(&full[q], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    const int32_t epoch = s_epoch;
+    const int4 *cells = a.v_cell;  // (first slice, slices, g << 5 | k, unused)
+    const int ncells = a.v_ncells;
+
+    auto give_up = [&]() {  // a wait expired: tell this block and the others
+        if (atomicExch(a.err, epoch) != epoch) st_relaxed(a.err + 1, (int)MPK_ERR_TIMEOUT);
+        *(volatile int *)&s_abort = 1;
+    };
+    auto aborted = [&]() -> bool { return *(volatile int *)&s_abort != 0; };
+    // smallest descriptor that is not finished (every lane of an auxiliary warp)
+    auto frontier = [&]() -> int {
+        const int v = lane < kWaveWarps ? ld_acquire_cta_shared(&s_prog[lane]) * kWaveWarps + lane : INT_MAX;
+        return __reduce_min_sync(0xffffffffu, v) / M;
+    };
+
+    if (warp == 0) {
+        // ------------------------------------------------------------------ dispatcher
+        int pushed = 0, room = kDescRing;  // descriptors below `room` may be written
+        uint32_t vnext = 0;
+        bool stop = false;
+        for (int c0 = 0; c0 < ncells && !stop; c0 += 32) {
+            const int4 ce = c0 + lane < ncells ? __ldg(cells + c0 + lane) : make_int4(0, 0, 0, 0);
+            const int2 sh = wave_share(ce.y, block, blocks);
+            int end = sh.y - sh.x;  // inclusive prefix sum over the 32 cells
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, end, o);
+                if (lane >= o) end += v;
+            }
+            const int total = __shfl_sync(0xffffffffu, end, 31);
+            for (int t0 = 0; t0 < total && !stop; t0 += 32) {
+                const int t = t0 + lane;
+                int q = 0;  // the cell of item t: the number of cells that end at or before it
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const int v = __shfl_sync(0xffffffffu, end, q + o - 1);
+                    if (v <= t) q += o;
+                }
+                const int qc = min(q, 31);
+                const int first = __shfl_sync(0xffffffffu, ce.x + sh.x, qc);
+                const int csize = __shfl_sync(0xffffffffu, sh.y - sh.x, qc);
+                const int qend = __shfl_sync(0xffffffffu, end, qc);
+                const int gk = __shfl_sync(0xffffffffu, ce.z, qc);
+                WaveDesc d{0, 0, 0, 0};
+                if (t < total) {
+                    const int s = first + (t - (qend - csize));
+                    const int64_t e0 = __ldg(a.slice_ptr + s), e1 = __ldg(a.slice_ptr + s + 1);
+                    const int r0 = __ldg(a.slice_row + s), r1 = __ldg(a.slice_row + s + 1);
+                    d.e32 = (int32_t)(e0 >> 5);
+                    d.width = (int32_t)((e1 - e0) >> 5);
+                    d.row0 = r0;
+                    d.ckr = (uint32_t)(c0 + qc) << 11 | (uint32_t)(gk & 31) << 6 | (uint32_t)(r1 - r0);
+                }
+                const int cnt = min(32, total - t0);
+                // where the entries go, and where runs start: at a cell's first slice, after a slice
+                // that is not copied, and where the buffer starts over
+                const int size = d.width <= Buf::SLICE / 32 ? 32 * d.width : 0;
+                uint32_t vp = (uint32_t)size;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t v = __shfl_up_sync(0xffffffffu, vp, o);
+                    if (lane >= o) vp += v;
+                }
+                const uint32_t vend = vnext + __shfl_sync(0xffffffffu, vp, 31);
+                vp += vnext - (uint32_t)size;
+                vnext = vend;
+                const uint32_t prev = __shfl_up_sync(0xffffffffu, vp, 1);
+                const int psize = __shfl_up_sync(0xffffffffu, size, 1);
+                if (lane == 0 || t == qend - csize || psize == 0 || prev / Buf::CAP != vp / Buf::CAP)
+                    d.width |= (int)0x80000000;
+                if (pushed + cnt > room) {
+                    Deadline w0;
+                    for (;;) {
+                        room = frontier() + kDescRing;
+                        if (pushed + cnt <= room) break;
+                        const bool late = aborted() || w0.expired(2 * a.wait_ns + 100000000LL);
+                        if (__any_sync(0xffffffffu, late)) {
+                            if (lane == 0) give_up();
+                            stop = true;
+                            break;
+                        }
+                        __nanosleep(100);
+                    }
+                    if (stop) break;
+                }
+                if (lane < cnt) {
+                    desc[(pushed + lane) & (kDescRing - 1)] = d;
+                    vpos[(pushed + lane) & (kDescRing - 1)] = vp;
+                }
+                pushed += cnt;
+                __syncwarp();
+                if (lane == 0) st_release_cta_shared(&s_pushed, pushed);
+            }
+        }
+        if (lane == 0) st_release_cta_shared(&s_total, pushed);
+    } else if (warp == 1) {
+        // ------------------------------------------------------------------ loader
+        int next = 0, tile = 0, old = 0;  // next descriptor, next tile, oldest tile in use
+        uint32_t tail = 0;                // position of the oldest slice in use
+        int t_desc = 0;                   // descriptors before the end of the tile with number lane (mod 32)
+        Deadline w0;
+        bool stop = false;
+        while (!stop) {
+            const int total_desc = ld_acquire_cta_shared(&s_total);  // before s_pushed: it is final then
+            const int have = __shfl_sync(0xffffffffu, ld_acquire_cta_shared(&s_pushed), 0) - next;
+            if (have <= 0) {
+                if (__any_sync(0xffffffffu, total_desc >= 0 || aborted())) {
+                    if (__any_sync(0xffffffffu, aborted())) break;
+                    if (__shfl_sync(0xffffffffu, ld_acquire_cta_shared(&s_pushed), 0) <= next) break;
+                    continue;
+                }
+                if (__any_sync(0xffffffffu, w0.expired(2 * a.wait_ns + 200000000LL))) {
+                    if (lane == 0) give_up();
+                    break;
+                }
+                __nanosleep(50);
+                continue;
+            }
+            __syncwarp();
+            WaveDesc d{0, 0, 0, 0};
+            uint32_t vp = 0;
+            if (lane < have) {
+                d = desc[(next + lane) & (kDescRing - 1)];
+                vp = vpos[(next + lane) & (kDescRing - 1)];
+            }
+            const int width = d.width & 0x7fffffff;
+            const bool staged = width <= Buf::SLICE / 32;
+            const uint32_t ve = vp + (staged ? 32u * (uint32_t)width : 0u);
+            const uint32_t v0 = __shfl_sync(0xffffffffu, vp, 0);
+            const unsigned int over = __ballot_sync(0xffffffffu, lane >= have || ve - v0 > (uint32_t)Buf::TILE);
+            const int cnt = over ? __ffs(over) - 1 : 32;  // at least 1: a slice fits a tile
+            const uint32_t vend = __shfl_sync(0xffffffffu, ve, cnt - 1);
+            while (vend - tail > (uint32_t)Buf::CAP || tile - old >= kWaveTiles) {  // room, and a free tile
+                const int done = frontier();
+                while (old < tile && __shfl_sync(0xffffffffu, t_desc, old & 31) <= done) ++old;
+                tail = done >= next ? v0 : vpos[done & (kDescRing - 1)];
+                if (vend - tail <= (uint32_t)Buf::CAP && tile - old < kWaveTiles) break;
+                if (__any_sync(0xffffffffu, aborted() || w0.expired(2 * a.wait_ns + 200000000LL))) {
+                    if (lane == 0) give_up();
+                    stop = true;
+                    break;
+                }
+            }
+            if (stop) break;
+            const int b = tile & (kWaveTiles - 1);
+            if (lane == 0) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                mbar_expect_tx(&full[b], (vend - v0) * (uint32_t)Buf::ENTRY);
+            }
+            const uint32_t o = vp % Buf::CAP;
+            if (lane < cnt)
+                loc[(next + lane) & (kDescRing - 1)] =
+                    staged ? (int)(o >> 5) | b << 16 | ((tile / kWaveTiles) & 1) << 24 : -1;
+            // a run of neighbouring slices: one pair of copies, by the run's first lane
+            const bool head = lane < cnt && staged && (lane == 0 || d.width < 0);
+            const unsigned int heads = __ballot_sync(0xffffffffu, head || lane >= cnt || !staged);
+            const unsigned int after = lane == 31 ? 0u : heads & (0xfffffffeu << lane);
+            const uint32_t run = __shfl_sync(0xffffffffu, ve, after ? __ffs(after) - 2 : 31) - vp;
+            if (head && run > 0) {
+                // the launch's last power is the last use of the entries (see k_mpk)
+                const bool last_use = a.v_ngroups > 1 && ((d.ckr >> 6) & 31u) == (uint32_t)a.p_launch;
+                bulk_g2s(sval + o, static_cast<const T *>(a.val) + 32 * (int64_t)d.e32, run * (uint32_t)sizeof(T), &full[b],
+                         last_use);
+                bulk_g2s(scol + o, a.col + 32 * (int64_t)d.e32, run * 4u, &full[b], last_use);
+            }
+            next += cnt;
+            if (lane == b) t_desc = next;
+            ++tile;
+            __syncwarp();
+            if (lane == 0) st_release_cta_shared(&s_loaded, next);
+            w0 = Deadline();
+        }
+        // the copies in flight land before the warp leaves, whatever the compute warps do
+        for (int q = old; q < tile; ++q) {
+            Deadline w1;
+            while (!mbar_try_wait(&full[q & (kWaveTiles - 1)], (q / kWaveTiles) & 1))
+                if (w1.expired(a.wait_ns)) break;
+        }
+    } else if (warp < kWaveAux) {
+        if (warp == 2) {
+            // -------------------------------------------------------------- poller
+            const int ng = a.v_ngroups;
+            bool stop = false;
+            for (int c0 = 0; c0 < ncells && !stop; c0 += 32) {
+                const int gk = c0 + lane < ncells ? __ldg(cells + c0 + lane).z : 0;
+                const int k = gk & 31, g = gk >> 5;
+                const int32_t *cnt = a.v_count + (int64_t)(k - 1) * ng;
+                int need[3];
+                bool ok = k <= 1;
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const int h = g - 1 + q;
+                    need[q] = (!ok && h >= 0 && h < ng) ? __ldg(a.v_gsl + h) : 0;
+                }
+                int known = 0;  // leading cells of the 32 already announced
+                Deadline w0;
+                while (known < 32) {
+                    const int err = ld_relaxed(a.err);
+                    if (!ok) {
+                        int got[3];
+#pragma unroll
+                        for (int q = 0; q < 3; ++q) got[q] = need[q] > 0 ? ld_relaxed(cnt + g - 1 + q) : 0;
+                        ok = got[0] >= need[0] && got[1] >= need[1] && got[2] >= need[2];
+                    }
+                    const unsigned int m = __ballot_sync(0xffffffffu, ok);
+                    const int run = m == 0xffffffffu ? 32 : __ffs(~m) - 1;
+                    if (run > known) {
+                        // acquire the counted rows before this block's reads of them: the same counters
+                        // again (a fence here waits for the SM's own stores: 1700 cycles against 900)
+#pragma unroll
+                        for (int q = 0; q < 3; ++q)
+                            if (need[q] > 0 && lane >= known && lane < run) ld_acquire(cnt + g - 1 + q);
+                        __syncwarp();
+                        if (lane == 0) st_release_cta_shared(&s_ready, c0 + run);
+                        known = run;
+                        w0 = Deadline();
+                        continue;
+                    }
+                    const bool late = err == epoch || aborted() || w0.expired(a.wait_ns);
+                    if (__any_sync(0xffffffffu, late)) {
+                        if (lane == 0) give_up();
+                        stop = true;
+                        break;
+                    }
+                }
+            }
+        } else {
+            // -------------------------------------------------------------- publisher
+            int base = 0;  // descriptors of the cells before the 32 at hand
+            bool stop = false;
+            for (int c0 = 0; c0 < ncells && !stop; c0 += 32) {
+                const int4 ce = c0 + lane < ncells ? __ldg(cells + c0 + lane) : make_int4(0, 0, 0, 0);
+                const int2 sh = wave_share(ce.y, block, blocks);
+                const int size = sh.y - sh.x, k = ce.z & 31;
+                int end = size;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(0xffffffffu, end, o);
+                    if (lane >= o) end += v;
+                }
+                const int total = __shfl_sync(0xffffffffu, end, 31);
+                end += base;
+                base += total;
+                bool todo = size > 0 && k < a.p_launch;  // nothing waits for the last power
+                Deadline w0;
+                for (;;) {
+                    const unsigned int left = __ballot_sync(0xffffffffu, todo);
+                    if (left == 0) break;
+                    const int done = frontier();
+                    const bool now = todo && end <= done;
+                    if (__any_sync(0xffffffffu, now)) {
+                        __syncwarp();         // every lane's view of the progress words
+                        fence_acq_rel_gpu();  // acquires the finished slices' rows, releases them
+                        if (now)
+                            atomicAdd(a.v_count + (int64_t)k * a.v_ngroups + (ce.z >> 5), size);
+                        todo = todo && !now;
+                        w0 = Deadline();
+                        continue;
+                    }
+                    const bool late = aborted() || w0.expired(2 * a.wait_ns + 100000000LL);
+                    if (__any_sync(0xffffffffu, late)) {
+                        if (lane == 0) give_up();
+                        stop = true;
+                        break;
+                    }
+                    __nanosleep(32);
+                }
+            }
+        }
+        // both done: this block neither polls nor publishes any more
+        __syncwarp();
+        int last = 0;
+        if (lane == 0) {
+            __threadfence();
+            if (atomicAdd(&s_left, 1) == 1) {
+                __threadfence();
+                last = atomicAdd(a.exit_count, 1u) == (unsigned int)blocks - 1;
+            }
+        }
+        if (__shfl_sync(0xffffffffu, last, 0)) {
+            __threadfence();
+            for (int64_t i = lane; i < (int64_t)a.p_launch * a.v_ngroups; i += 32) a.v_count[a.v_ngroups + i] = 0;
+            if (lane == 0) {
+                *a.exit_count = 0u;
+                *a.epoch_word = (unsigned int)epoch;
+            }
+            __threadfence();
+        }
+    } else {
+        // ------------------------------------------------------------------ compute warps
+        const int w = warp - kWaveAux;
+        const int rl = lane / M, cl = lane % M;    // this lane's row of a group, its right-hand side
+        int done = 0, ready = 0, seen = 0;
+        for (int unit = w;; unit += kWaveWarps) {
+            const int idx = unit / M, q = unit % M;
+            if (idx >= seen) {  // wait for the descriptor, or the end
+                Deadline w0;
+                bool none = false;
+                for (;;) {
+                    const int total = ld_acquire_cta_shared(&s_total);
+                    seen = ld_acquire_cta_shared(&s_loaded);
+                    if (idx < seen) break;
+                    if ((total >= 0 && idx >= total) || aborted() || w0.expired(2 * a.wait_ns + 300000000LL)) {
+                        none = true;
+                        break;
+                    }
+                    __nanosleep(20);
+                }
+                if (__any_sync(0xffffffffu, none)) break;
+                seen = __shfl_sync(0xffffffffu, seen, 0);
+                __syncwarp();  // lane 0's acquire, for every lane while `seen` holds
+            }
+            WaveDesc d = desc[idx & (kDescRing - 1)];
+            d.width &= 0x7fffffff;
+            const int lc = loc[idx & (kDescRing - 1)];
+            const int cell = (int)(d.ckr >> 11), k = (int)(d.ckr >> 6) & 31, rows = (int)(d.ckr & 63u);
+            if (cell >= ready) {  // the cell's dependencies
+                Deadline w0;
+                bool none = false;
+                for (;;) {
+                    ready = ld_acquire_cta_shared(&s_ready);
+                    if (cell < ready) break;
+                    if (aborted() || w0.expired(2 * a.wait_ns + 100000000LL)) {
+                        none = true;
+                        break;
+                    }
+                }
+                if (__any_sync(0xffffffffu, none)) break;
+                ready = __shfl_sync(0xffffffffu, ready, 0);
+                __syncwarp();  // lane 0's acquire, for every lane while `ready` holds
+            }
+            if (lc >= 0) {  // the slice's tile
+                uint64_t *const bar = &full[(lc >> 16) & 31];
+                const uint32_t phase = (uint32_t)lc >> 24;
+                if (!mbar_try_wait(bar, phase)) {
+                    Deadline w0;
+                    while (!mbar_try_wait(bar, phase))
+                        if (w0.expired(a.wait_ns)) break;
+                    if (!__all_sync(0xffffffffu, mbar_try_wait(bar, phase))) {
+                        if (lane == 0) give_up();
+                        break;
+                    }
+                }
+            }
+            const double *xin = input_block<M>(a, k);
+            const AT *xacc = InputAcc<M, AT>::get(a, k) + cl;
+            if (q * G < rows) {
+                const int r = q * G + rl;
+                const bool valid = r < rows;
+                const int64_t at = ((int64_t)d.row0 + r) * M + cl;
+                // rows of earlier steps that the epilogue reads, on their way during the sums
+                double own = 0.0, back = 0.0, old = 0.0;
+                if constexpr (MODE == MODE_CHEB) {
+                    if (valid) {
+                        own = xin[at];
+                        if (a.k_offset + k != 1)
+                            back = a.ybase[(int64_t)ring_slot(a, a.k_offset + k - 2) * a.ystride + at];
+                        old = a.acc[at];
+                    }
+                } else if (k == 1 && a.y0copy && valid) {
+                    own = a.x0[at];
+                }
+                AT acc = AT(0);
+                int left = d.width;
+                if (lc >= 0) {
+                    const int o = 32 * (lc & 0xffff) + r;
+                    SVal<VT, AT> sv{sval + o};
+                    const int32_t *sc = scol + o;
+                    for (; left >= kBatch; left -= kBatch) {
+                        wave_batch<kBatch, M, VT, AT>(sv, sc, xacc, acc);
+                        sc += 32 * kBatch;
+                        sv.p += 32 * kBatch;
+                    }
+                    switch (left) {
+                        case 1: wave_batch<1, M, VT, AT>(sv, sc, xacc, acc); break;
+                        case 2: wave_batch<2, M, VT, AT>(sv, sc, xacc, acc); break;
+                        case 3: wave_batch<3, M, VT, AT>(sv, sc, xacc, acc); break;
+                        case 4: wave_batch<4, M, VT, AT>(sv, sc, xacc, acc); break;
+                        case 5: wave_batch<5, M, VT, AT>(sv, sc, xacc, acc); break;
+                        case 6: wave_batch<6, M, VT, AT>(sv, sc, xacc, acc); break;
+                        case 7: wave_batch<7, M, VT, AT>(sv, sc, xacc, acc); break;
+                        default: break;
+                    }
+                } else {  // a slice wider than the buffer takes: entries from global memory
+                    const int64_t e = 32 * (int64_t)d.e32 + r;
+                    GVal<VT, AT> gv{static_cast<const T *>(a.val) + e};
+                    GCol gc{a.col + e};
+                    for (; left > 0; --left) {
+                        wave_batch<1, M, VT, AT>(gv, gc, xacc, acc);
+                        gc.p += 32;
+                        gv.p += 32;
+                    }
+                }
+                wave_epilogue<M, MODE, AT>(a, k, at, valid, lane, acc, own, back, old);
+            }
+            __syncwarp();
+            ++done;
+            if (lane == 0) st_release_cta_shared(&s_prog[w], done);
+        }
+    }
+}
+
+template <class VT, int M> static void *wave_fn(int mode, bool a32) {
+    if constexpr (!std::is_same<VT, ValF64>::value)
+        if (a32) {
+            if (mode == MODE_HOST) {
+                if constexpr (M == 1) return (void *)k_wave<1, MODE_HOST, VT, true>;
+            }
+            return mode == MODE_POWERS ? (void *)k_wave<M, MODE_POWERS, VT, true> : (void *)k_wave<M, MODE_CHEB, VT, true>;
+        }
+    if (mode == MODE_HOST) {
+        if constexpr (M == 1) return (void *)k_wave<1, MODE_HOST, VT, false>;
+        fail(MPK_ERR_UNSUPPORTED, "host output needs nrhs 1");
+    }
+    return mode == MODE_POWERS ? (void *)k_wave<M, MODE_POWERS, VT, false> : (void *)k_wave<M, MODE_CHEB, VT, false>;
+}
+
+template <class VT> void *select_wave_vt(int mode, int m, bool a32, int *smem) {
+    *smem = WaveBuf<VT>::ALL * WaveBuf<VT>::ENTRY;
+    switch (m) {
+        case 1: return wave_fn<VT, 1>(mode, a32);
+        case 2: return wave_fn<VT, 2>(mode, a32);
+        case 4: return wave_fn<VT, 4>(mode, a32);
+        case 8: return wave_fn<VT, 8>(mode, a32);
+        case 16: return wave_fn<VT, 16>(mode, a32);
+    }
+    fail(MPK_ERR_UNSUPPORTED, "nrhs %d", m);
+}
+
+// defined in mpk_wave_<type>.cu: the kernel for (mode, nrhs, accumulator) 
+void *select_wave_f64(int mode, int m, bool a32, int *smem);
+void *select_wave_f32(int mode, int m, bool a32, int *smem);
+void *select_wave_bf16(int mode, int m, bool a32, int *smem);
+
+}  // namespace mpk

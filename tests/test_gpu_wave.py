@@ -1,0 +1,76 @@
+"""The wave kernel (static schedule, plans at the planner's block shape) against the oracle, bit
+for bit, where it can go wrong: row widths around its batches of 8 entries and around the widest
+slice it stages (64 entries), empty rows, ragged last slices, blocks of every width, one group and
+many, and more cells than one step of its auxiliary warps (32)."""
+import numpy as np
+import pytest
+
+import gen
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mpk():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2405_12525_gb300 as m
+    m.build()
+    m.load()
+    return m
+
+
+def _widths_matrix(n, widths, stream):
+    """Row i stores widths[i % len] entries (at most its window) near the diagonal, non-symmetric."""
+    seed = gen.derive_seed(stream)
+    u = gen.splitmix64(seed, n)
+    rows, cols = [], []
+    for i in range(n):
+        w = min(widths[i % len(widths)], n)
+        lo = max(0, min(i - w // 2 - int(u[i] % np.uint64(3)), n - w))
+        rows += [i] * w
+        cols += list(range(lo, lo + w))
+    vals = gen.uniform(gen.derive_seed(stream + 1), len(rows))
+    return gen.from_coo(n, rows, cols, vals)
+
+
+def _check(mpk, A, m, p, order, sym=False, val="f64", accum=0, **opts):
+    vt = {"f64": mpk.MPK_F64, "f32": mpk.MPK_F32}[val]
+    dA = mpk.CsrMatrix.from_host(A, is_symmetric=sym, value_type=vt)
+    L = mpk.build_levels(dA, 0)
+    P = mpk.plan(dA, L, p_max=p, nrhs=m, order=order, accum=accum, **opts)
+    stored = A.with_values(A.val.astype(np.float32).astype(np.float64)) if val == "f32" else A
+    X = gen.vector(A.n, m, stream=5)
+    perm = L.perm.cpu().numpy()
+    Xin = X[perm] if order == mpk.ORDER_PLAN else X
+    Y = torch.full((p + 1, A.n, m), float("nan"), dtype=torch.float64, device="cuda")
+    for _ in range(2):  # the second launch finds the counters that the first one cleared
+        Y.fill_(float("nan"))
+        P.apply(torch.from_numpy(np.ascontiguousarray(Xin)).cuda(), p, Y=Y)
+        P.sync_status()
+        want = oracle.mpk_acc32(stored, X, p) if accum else oracle.mpk(stored, X, p)
+        got = Y.cpu().numpy()
+        if order == mpk.ORDER_PLAN:
+            want = want[:, perm]
+        assert np.array_equal(got.view(np.uint64), np.ascontiguousarray(want).view(np.uint64))
+
+
+@pytest.mark.parametrize("m", [1, 2, 4, 8, 16])
+@pytest.mark.parametrize("widths", [(0, 1, 7), (8, 9, 3, 0), (16, 17, 15), (62, 63, 64, 65, 2), (80, 1)])
+def test_row_widths(mpk, m, widths):
+    _check(mpk, _widths_matrix(1000 + 7 * m, widths, 900), m, 3, mpk.ORDER_ORIGINAL)
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 64, 4863, 4864, 4865])
+@pytest.mark.parametrize("p", [1, 2, 31])
+def test_row_counts(mpk, n, p):
+    _check(mpk, _widths_matrix(n, (3, 2), 910), 1, p, mpk.ORDER_PLAN)
+
+
+@pytest.mark.parametrize("cache_bytes", [1, 40000, 400000])
+@pytest.mark.parametrize("m,val,accum", [(1, "f64", 0), (2, "f64", 0), (8, "f32", 0), (1, "f32", 1), (4, "f32", 1)])
+def test_many_groups(mpk, cache_bytes, m, val, accum):
+    _check(mpk, gen.laplacian_3d(19, 17, 23), m, 9, mpk.ORDER_PLAN, sym=True, val=val, accum=accum,
+           cache_bytes=cache_bytes)

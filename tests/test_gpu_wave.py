@@ -69,8 +69,34 @@ def test_row_counts(mpk, n, p):
     _check(mpk, _widths_matrix(n, (3, 2), 910), 1, p, mpk.ORDER_PLAN)
 
 
+@pytest.mark.parametrize("n,p", [(60007, 31), (9000, 31)])
+def test_descriptor_ring_wraps(mpk, n, p):
+    """Slices of one entry a row: the ring of descriptors, not the entry buffer, limits the lead."""
+    _check(mpk, _widths_matrix(n, (1, 0, 1), 920), 1, p, mpk.ORDER_PLAN, cache_bytes=1 << 30)
+    _check(mpk, gen.laplacian_3d(17, 9, 6), 2, p, mpk.ORDER_PLAN, sym=True, cache_bytes=20000)
+
+
 @pytest.mark.parametrize("cache_bytes", [1, 40000, 400000])
 @pytest.mark.parametrize("m,val,accum", [(1, "f64", 0), (2, "f64", 0), (8, "f32", 0), (1, "f32", 1), (4, "f32", 1)])
 def test_many_groups(mpk, cache_bytes, m, val, accum):
     _check(mpk, gen.laplacian_3d(19, 17, 23), m, 9, mpk.ORDER_PLAN, sym=True, val=val, accum=accum,
            cache_bytes=cache_bytes)
+
+
+@pytest.mark.parametrize("m,p", [(1, 3), (2, 3), (2, 6)])
+def test_hand_over_of_small_cells(mpk, m, p):
+    """Cells of a few slices, run many times into poisoned outputs: a block must see every row that
+    a cell's counters stand for."""
+    A = gen.laplacian_3d(17, 9, 6)
+    dA = mpk.CsrMatrix.from_host(A, is_symmetric=True)
+    L = mpk.build_levels(dA, 0)
+    P = mpk.plan(dA, L, p_max=6, nrhs=m, order=mpk.ORDER_PLAN, cache_bytes=20000)
+    X = gen.vector(A.n, m, stream=81)
+    perm = L.perm.cpu().numpy()
+    want = torch.from_numpy(np.ascontiguousarray(oracle.mpk(A, X, p)[:, perm])).cuda()
+    Xd = torch.from_numpy(np.ascontiguousarray(X[perm])).cuda()
+    Y = torch.empty((p + 1, A.n, m), dtype=torch.float64, device="cuda")
+    for _ in range(300):
+        Y.fill_(float("nan"))
+        P.apply(Xd, p, Y=Y)
+        assert torch.equal(Y, want)

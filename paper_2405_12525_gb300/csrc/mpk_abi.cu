@@ -174,6 +174,7 @@ KArgs mpk::base_args(Plan &P, int32_t p) {
     a.ystride = (int64_t)P.n * P.m;
     a.shadow = P.shadow;
     a.p_launch = p;
+    a.stream_last = P.wave ? P.v_ngroups > 1 : 1;
     if (P.engine == MPK_ENGINE_WARP) {
         a.w_item = P.w_item + P.w_cell_off[p];
         a.w_gk = P.w_gk + P.w_cell_off[p];

@@ -295,6 +295,9 @@ struct KArgs {
     int32_t *v_count;          // (p + 1) x v_ngroups
     int32_t v_ncells, v_ngroups;
     int32_t v_maxsl;           // slices of the largest group
+    // 1: what the launch's last power reads and writes is the first to leave L2 (the matrix does not
+    // stay there between launches)
+    int32_t stream_last;
 };
 constexpr int kWaveMaxCells = 1 << 20;  // cells of a wave launch (a descriptor holds 21 bits)
 // warp-ticketed engine: slices per item, claim queues (one per warp of a block)

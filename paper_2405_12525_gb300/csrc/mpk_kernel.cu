@@ -43,7 +43,6 @@ constexpr int kWarpBS = 32 * kWarpQueues;
 
 template <int M, int MODE, class VT>
 __global__ void __launch_bounds__(kWarpBS, (WarpOcc<M, MODE, VT>::blocks)) k_mpkw(const KArgs a) {
-    constexpr int B = Batch<M>::B;
     const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
     __shared__ int32_t s_epoch;
     if (threadIdx.x == 0) s_epoch = ld_relaxed(reinterpret_cast<const int32_t *>(a.epoch_word)) + 1;
@@ -114,12 +113,15 @@ __global__ void __launch_bounds__(kWarpBS, (WarpOcc<M, MODE, VT>::blocks)) k_mpk
         }
         const double *xin = input_block<M>(a, k);
         for (int sl = s_first; sl < s_end; ++sl) {
-            const int64_t r = (int64_t)gr0 + 32 * (sl - gs0) + lane;
-            if (r < gr1) {
-                const int64_t e0 = __ldg(a.slice_ptr + sl), e1 = __ldg(a.slice_ptr + sl + 1);
+            const int64_t r0 = (int64_t)gr0 + 32 * (sl - gs0);
+            const int64_t e0 = __ldg(a.slice_ptr + sl), e1 = __ldg(a.slice_ptr + sl + 1);
+            if constexpr (M == 1) {
+                unit_run<M, MODE, double>(a, k, GVal<VT>{val + e0}, GCol{a.col + e0}, (int)((e1 - e0) >> 5), r0, 0, gr1, xin,
+                                          xin, lane);
+            } else if (r0 + lane < gr1) {
                 double w[M];
-                row_sum<M, B, double>(GVal<VT>{val}, GCol{a.col}, e0 + lane, (int)((e1 - e0) >> 5), xin, w);
-                row_epilogue<M, MODE, double>(a, k, r, w, xin);
+                row_sum<M, Batch<M>::B, double>(GVal<VT>{val}, GCol{a.col}, e0 + lane, (int)((e1 - e0) >> 5), xin, w);
+                row_epilogue<M, MODE, double>(a, k, r0 + lane, w, xin);
             }
         }
         __syncwarp();
@@ -148,9 +150,11 @@ __global__ void __launch_bounds__(kWarpBS, (WarpOcc<M, MODE, VT>::blocks)) k_mpk
 // One power k of the whole matrix, unblocked: blocks walk the plan's chunks, warps their
 // slices, with the level-blocked kernel's row body and epilogue (plain powers or the
 // Chebyshev recurrence), so the results are the same bits.  One launch per power; stream
-// order supplies every dependency.
+// order supplies every dependency.  Six blocks an SM with columns, eight without (8 / 6 / 5 / 4: 128^3
+// binary64 p = 8 364 / 364 / 377 / 380 us; bfloat16, binary32 sums 255 / 275 / 271 / 295 us; two
+// columns 561 / 550 / 576 / 633 us).
 template <int M, int MODE, class VT, bool A32 = false>
-__global__ void __launch_bounds__(kSpmvBS) k_sweep(const KArgs a, int k) {
+__global__ void __launch_bounds__(kSpmvBS, M == 1 ? 8 : 6) k_sweep(const KArgs a, int k) {
     using AT = typename std::conditional<A32, float, double>::type;
     const int lane = threadIdx.x & 31;
     const auto *val = static_cast<const typename VT::T *>(a.val);
@@ -159,15 +163,11 @@ __global__ void __launch_bounds__(kSpmvBS) k_sweep(const KArgs a, int k) {
     for (int c = blockIdx.x; c < a.nchunks; c += gridDim.x) {
         const int r0 = a.chunk_row[c], r1 = a.chunk_row[c + 1], sl0 = a.chunk_slice[c];
         const int nsl = (r1 - r0 + 31) >> 5;
-        for (int sl = threadIdx.x >> 5; sl < nsl; sl += kSpmvBS / 32) {
-            const int64_t r = (int64_t)r0 + 32 * sl + lane;
-            if (r < r1) {
-                const int64_t e0 = a.slice_ptr[sl0 + sl], e1 = a.slice_ptr[sl0 + sl + 1];
-                AT w[M];
-                row_sum<M, Batch<M>::B, AT>(GVal<VT, AT>{val}, GCol{a.col}, e0 + lane, (int)((e1 - e0) >> 5), xacc,
-                                            w);
-                row_epilogue<M, MODE, AT>(a, k, r, w, xin);
-            }
+        for (int it = threadIdx.x >> 5; it < nsl * M; it += kSpmvBS / 32) {
+            const int sl = it / M;
+            const int64_t e0 = a.slice_ptr[sl0 + sl], e1 = a.slice_ptr[sl0 + sl + 1];
+            unit_run<M, MODE, AT>(a, k, GVal<VT, AT>{val + e0}, GCol{a.col + e0}, (int)((e1 - e0) >> 5),
+                                  (int64_t)r0 + 32 * sl, it % M, r1, xin, xacc, lane);
         }
     }
 }
@@ -214,15 +214,13 @@ __global__ void __launch_bounds__(kSpmvBS) k_spmv_rows(const RowSegs segs) {
         const int c = g.c0 + (v - segs.first[q]);
         const int r0 = g.chunk_row[c], r1 = g.chunk_row[c + 1], sl0 = g.chunk_slice[c];
         const int nsl = (r1 - r0 + 31) >> 5;
-        for (int sl = threadIdx.x >> 5; sl < nsl; sl += kSpmvBS / 32) {
-            const int64_t r = (int64_t)r0 + 32 * sl + lane;
-            if (r < r1 && r >= g.lo && r < g.hi) {
-                const int64_t s0 = g.slice_ptr[sl0 + sl], s1 = g.slice_ptr[sl0 + sl + 1];
-                double w[M];
-                row_sum<M, Batch<M>::B, double>(GVal<VT>{val}, GCol{g.col}, s0 + lane, (int)((s1 - s0) >> 5), g.x, w);
-#pragma unroll
-                for (int i = 0; i < M; ++i) g.y[r * M + i] = w[i];
-            }
+        for (int it = threadIdx.x >> 5; it < nsl * M; it += kSpmvBS / 32) {
+            const int sl = it / M, rl = it % M * (32 / M) + lane / M;
+            const int64_t r = (int64_t)r0 + 32 * sl + rl;
+            const int64_t s0 = g.slice_ptr[sl0 + sl] + rl, s1 = g.slice_ptr[sl0 + sl + 1];
+            const double w = unit_sum<M, double>(GVal<VT>{val + s0}, GCol{g.col + s0}, (int)((s1 - s0 + rl) >> 5),
+                                                 g.x + lane % M);
+            if (r < r1 && r >= g.lo && r < g.hi) g.y[r * M + lane % M] = w;
         }
     }
 }

@@ -185,37 +185,6 @@ __device__ __forceinline__ void row_sum(VP val, CP col, int64_t off, int width, 
     }
 }
 
-// Continues a row sum from entry j0 (acc already holds entries 0..j0-1).
-template <int M, int B, class AT, class VP, class CP>
-__device__ __forceinline__ void row_sum_from(VP val, CP col, int64_t off, int j_start, int width, const AT *x,
-                                             AT (&acc)[M]) {
-    for (int j0 = j_start; j0 < width; j0 += B) {
-        AT v[B];
-        int32_t c[B];
-#pragma unroll
-        for (int b = 0; b < B; ++b) {
-            if (j0 + b < width) {
-                v[b] = val[off + 32 * (int64_t)(j0 + b)];
-                c[b] = col[off + 32 * (int64_t)(j0 + b)];
-            } else {
-                v[b] = AT(0);
-                c[b] = -1;
-            }
-        }
-        AT xv[B][M];
-#pragma unroll
-        for (int b = 0; b < B; ++b)
-#pragma unroll
-            for (int i = 0; i < M; ++i) xv[b][i] = (c[b] >= 0) ? x[(int64_t)c[b] * M + i] : AT(0);
-#pragma unroll
-        for (int b = 0; b < B; ++b)
-            if (c[b] >= 0) {
-#pragma unroll
-                for (int i = 0; i < M; ++i) acc[i] = afma(v[b], xv[b][i], acc[i]);
-            }
-    }
-}
-
 // ----------------------------------------------------------------------------- value types
 // Matrix values are stored as float64, float32 or bfloat16 and widened to float64 before
 // their FMA, exactly and with integer operations only (widen_normal32: the planner admits
@@ -393,6 +362,120 @@ __device__ __forceinline__ void row_epilogue(const KArgs &a, int k, int64_t r, c
     row_epilogue_loaded<M, MODE, AT>(a, k, r, w, e);
 }
 
+constexpr int kBatch = 8;  // entries of a row whose x values are gathered together
+// column indices staged in shared memory
+struct SCol {
+    const int32_t *p;
+    __device__ __forceinline__ int32_t operator[](int64_t i) const { return p[i]; }
+};
+
+// Epilogue of one (row, column) of step j at local power k: w is its row sum.  own / back: its
+// values of the two previous steps and old the accumulator (recurrence), or own is x0's value
+// copied to Y[0] (power 1).
+// Executed by the whole warp.
+template <int M, int MODE, class AT>
+__device__ __forceinline__ void unit_epilogue(const KArgs &a, int k, int64_t at, bool valid, int lane, AT wa, double own,
+                                              double back, double old) {
+    constexpr bool A32 = sizeof(AT) == 4;
+    const int j = a.k_offset + k;
+    const double w = to_f64(wa);
+    double *y = a.ybase + (int64_t)ring_slot(a, j) * a.ystride + at;
+    if constexpr (MODE == MODE_CHEB) {
+        const double vn = j == 1 ? fma(a.halpha, w, a.hbeta * own) : fma(a.alpha, w, fma(a.beta, own, -back));
+        // complex coefficients act on column pairs, which sit in neighbouring lanes
+        const double other = (M > 1 && a.complex_coeff) ? __shfl_xor_sync(0xffffffffu, vn, 1) : 0.0;
+        if (valid) {
+            *y = vn;
+            if constexpr (A32) a.shadow[(int64_t)(j & 1) * a.ystride + at] = __double2float_rn(vn);
+            double acc = fma(a.cre[k], vn, old);
+            if (M > 1 && a.complex_coeff) acc = fma((lane & 1) ? a.cim[k] : -a.cim[k], other, acc);
+            a.acc[at] = acc;
+        }
+    } else if (valid) {
+        if (!A32 && k == a.p_launch && a.stream_last)
+            __stcs(y, w);  // not read again here: see row_epilogue_loaded
+        else
+            *y = w;
+        if constexpr (A32) a.shadow[(int64_t)(j & 1) * a.ystride + at] = (float)wa;
+        if constexpr (MODE == MODE_HOST) __stcs(a.yhost + (int64_t)j * a.ystride + at, w);
+        if (k == 1 && a.y0copy) a.y0copy[at] = own;
+    }
+}
+
+// N entries of the rows of a warp (entry t of a lane's row 32 t places on): their x values are
+// gathered together, then summed in order.  N is exact: an FP64 FMA takes its 64 cycles of the
+// pipe even when no lane of the warp runs it, so sums are never padded to a batch (64^3 27-point,
+// p = 8, unstaged shape: 272 -> 222 us; 128^3 sweep, recurrence of 16 steps: 1331 -> 986 us).
+template <int N, int M, class AT, class VP, class CP>
+__device__ __forceinline__ void unit_batch(VP sv, CP sc, const AT *x, AT &acc) {
+    int c[N];
+    AT xv[N];
+#pragma unroll
+    for (int t = 0; t < N; ++t) {
+        c[t] = sc[32 * t];
+        xv[t] = AT(0);
+        if (c[t] >= 0) xv[t] = x[(int64_t)c[t] * M];
+    }
+#pragma unroll
+    for (int t = 0; t < N; ++t) {
+        const AT v = sv[32 * t];
+        if (c[t] >= 0) acc = afma(v, xv[t], acc);
+    }
+}
+
+// acc plus a row's `width` entries in stored order: full batches, then the exact rest.
+template <int M, class AT, class VP, class CP>
+__device__ __forceinline__ AT unit_sum(VP sv, CP sc, int width, const AT *x, AT acc = AT(0)) {
+    for (; width >= kBatch; width -= kBatch) {
+        unit_batch<kBatch, M, AT>(sv, sc, x, acc);
+        sc.p += 32 * kBatch;
+        sv.p += 32 * kBatch;
+    }
+    switch (width) {
+        case 1: unit_batch<1, M, AT>(sv, sc, x, acc); break;
+        case 2: unit_batch<2, M, AT>(sv, sc, x, acc); break;
+        case 3: unit_batch<3, M, AT>(sv, sc, x, acc); break;
+        case 4: unit_batch<4, M, AT>(sv, sc, x, acc); break;
+        case 5: unit_batch<5, M, AT>(sv, sc, x, acc); break;
+        case 6: unit_batch<6, M, AT>(sv, sc, x, acc); break;
+        case 7: unit_batch<7, M, AT>(sv, sc, x, acc); break;
+        default: break;
+    }
+    return acc;
+}
+
+// the rows of earlier steps that the epilogue of value `at` reads
+template <int MODE>
+__device__ __forceinline__ void unit_rows(const KArgs &a, int k, int64_t at, bool valid, const double *xin, double &own,
+                                          double &back, double &old) {
+    if constexpr (MODE == MODE_CHEB) {
+        if (valid) {
+            own = xin[at];
+            if (a.k_offset + k != 1) back = a.ybase[(int64_t)ring_slot(a, a.k_offset + k - 2) * a.ystride + at];
+            old = a.acc[at];
+        }
+    } else if (k == 1 && a.y0copy && valid) {
+        own = a.x0[at];
+    }
+}
+
+// One unit: the 32 / M rows from row r0 + q * 32 / M of a slice (those below `end`), every right-hand
+// side, step k: lane l owns row l / M of them and right-hand side l % M.  sv / sc: the entries of
+// the slice's first row (they advance by lane row here).
+template <int M, int MODE, class AT, class VP, class CP>
+__device__ __forceinline__ void unit_run(const KArgs &a, int k, VP sv, CP sc, int width, int64_t r0, int q, int64_t end,
+                                         const double *xin, const AT *xacc, int lane) {
+    const int rl = q * (32 / M) + lane / M, cl = lane % M;
+    const bool valid = r0 + rl < end;
+    const int64_t at = (r0 + rl) * M + cl;
+    double own = 0.0, back = 0.0, old = 0.0;
+    unit_rows<MODE>(a, k, at, valid, xin, own, back, old);  // on their way during the sums
+    sv.p += rl;
+    sc.p += rl;
+    const AT acc = unit_sum<M, AT>(sv, sc, width, xacc + cl);
+    unit_epilogue<M, MODE, AT>(a, k, at, valid, lane, acc, own, back, old);
+}
+
 // ----------------------------------------------------------------------------- K-MPK
 // Work unit = (row chunk c, local power k).  Units are claimed through one atomic ticket
 // in the order of the unit table, which lists the Lp-diagram cells (group g, power k) line
@@ -489,6 +572,7 @@ __device__ __forceinline__ void phase_a(const KArgs &a, const UnitInfo &u, int b
     pf.width = 0;
     pf.off = 0;
     pf.valid = 0;
+    if constexpr (M > 1 || !STAGING) return;  // blocks of right-hand sides gather in phase B
     if (STAGING && u.staged && cwarp < u.nsl) {  // shapes without slots never stage
         const int pre = slice_prefix<NW>(u.widths, cwarp);
         pf.width = slice_width<NW>(u.widths, cwarp);
@@ -517,12 +601,6 @@ __device__ __forceinline__ void phase_a(const KArgs &a, const UnitInfo &u, int b
 // the block modulo kDoneRing and only grow (use n of a counter completes at n times the
 // number of compute warps), so a lagging publisher never sees a counter that was reset.
 constexpr int kDoneRing = 64;
-// shapes 0-2 release the slot before their FMA chain too (1), or after their unit (0): the
-// early path holds a batch of entries in registers, more than shape 0's 40 a thread allow
-#ifndef MPK_EARLY_RELEASE_B
-#define MPK_EARLY_RELEASE_B 0
-#endif
-constexpr bool kEarlyReleaseB = MPK_EARLY_RELEASE_B != 0;
 template <int CW>
 __device__ __forceinline__ void release_slot(uint64_t *s_empty, int b, int lane) {
     __syncwarp();
@@ -597,72 +675,79 @@ __device__ __forceinline__ void phase_b(const KArgs &a, int32_t epoch, const Pre
     const SVal<VT, AT> sval{sval0 + pf.slot * Shape<SH>::SE};
     const int32_t *scol = kStageCol ? scol0 + pf.slot * Shape<SH>::SE : a.col + u.ebase;
     bool released = false;
-    if (kEarlyReleaseB && Shape<SH>::SE > 0 && u.staged && u.nsl <= kCompWarps && pf.width <= B) {
-        // the warp's one slice fits one batch: read its entries, release the slot, then compute
-        AT v[B];
-        bool on[B];
-#pragma unroll
-        for (int q = 0; q < B; ++q) {
-            on[q] = kPadMask<AT> ? ((pf.valid >> q) & 1u) != 0 : (pf.r >= 0 && q < pf.width && scol[pf.off + 32 * q] >= 0);
-            v[q] = on[q] ? sval[pf.off + 32 * q] : AT(0);
-        }
-        EpiRows<M> er;
-        if (pf.r >= 0) epilogue_load<M, MODE>(a, k, pf.r, xin, er);
-        release_slot<kCompWarps>(s_empty, pf.slot, lane);
-        released = true;
-        if (pf.r >= 0) {
-            AT w[M];
-#pragma unroll
-            for (int i = 0; i < M; ++i) w[i] = AT(0);
-#pragma unroll
-            for (int q = 0; q < B; ++q)
-                if (on[q]) {
-#pragma unroll
-                    for (int i = 0; i < M; ++i) w[i] = afma(v[q], pf.x[q][i], w[i]);
-                }
-            row_epilogue_loaded<M, MODE, AT>(a, k, pf.r, w, er);
-        }
-    } else if (Shape<SH>::SE > 0 && u.staged) {
-        if (pf.r >= 0) {  // first slice: prefetched first batch, then the rest of the row
-            AT w[M];
-#pragma unroll
-            for (int i = 0; i < M; ++i) w[i] = AT(0);
-#pragma unroll
-            for (int q = 0; q < B; ++q) {
-                if (kPadMask<AT> ? ((pf.valid >> q) & 1u) != 0 : (q < pf.width && scol[pf.off + 32 * q] >= 0)) {
-                    const AT v = sval[pf.off + 32 * q];
-#pragma unroll
-                    for (int i = 0; i < M; ++i) w[i] = afma(v, pf.x[q][i], w[i]);
-                }
-            }
-            if (pf.width > B) row_sum_from<M, 2, AT>(sval, scol, pf.off, B, pf.width, xacc, w);  // rare: wide rows
-            row_epilogue<M, MODE, AT>(a, k, pf.r, w, xin);
-        }
-        for (int sl = cwarp + kCompWarps; sl < u.nsl; sl += kCompWarps) {  // further slices (wide chunks)
+    if (M > 1 && Shape<SH>::SE > 0 && Shape<SH>::SPW > 1 && u.staged) {
+        // one block of 16 warps an SM: too few for units of 32 values, a row a lane instead (128^3,
+        // binary64, 8 columns, p = 8: 2.41 against 2.68 ms)
+        for (int sl = cwarp; sl < u.nsl; sl += kCompWarps) {
             const int64_t r = (int64_t)u.row0 + 32 * sl + lane;
             const int pre = slice_prefix<Shape<SH>::NW>(u.widths, sl);
             if (r >= u.row1) continue;
             AT w[M];
-            // a second slice of the warp (shapes of two slices a warp: all gathers of a batch at
-            // once) or, on the other shapes, the rare chunk wider than the block
-            constexpr int BS2 = Shape<SH>::SPW > 1 ? B : 2;
-            row_sum<M, BS2, AT>(sval, scol, 32 * pre + lane, slice_width<Shape<SH>::NW>(u.widths, sl), xacc, w);
+            row_sum<M, B, AT>(sval, scol, 32 * pre + lane, slice_width<Shape<SH>::NW>(u.widths, sl), xacc, w);
             row_epilogue<M, MODE, AT>(a, k, r, w, xin);
+        }
+    } else if (M > 1 && Shape<SH>::SE > 0 && u.staged) {  // units of a slice over the warps (see unit_run)
+        for (int it = cwarp; it < u.nsl * M; it += kCompWarps) {
+            const int sl = it / M, o = 32 * slice_prefix<Shape<SH>::NW>(u.widths, sl);
+            unit_run<M, MODE, AT>(a, k, SVal<VT, AT>{sval0 + pf.slot * Shape<SH>::SE + o}, SCol{scol + o},
+                                  slice_width<Shape<SH>::NW>(u.widths, sl), (int64_t)u.row0 + 32 * sl, it % M, u.row1, xin,
+                                  xacc, lane);
+        }
+    } else if (Shape<SH>::SE > 0 && u.staged) {
+        if (pf.r >= 0) {  // first slice: prefetched first batch, then the rest of the row
+            AT w[M];
+            w[0] = AT(0);
+            // as many FMAs as the slice is wide (an FP64 FMA that no lane runs costs as much)
+            auto sums = [&](auto n) {
+#pragma unroll
+                for (int q = 0; q < decltype(n)::value; ++q)
+                    if (kPadMask<AT> ? ((pf.valid >> q) & 1u) != 0 : scol[pf.off + 32 * q] >= 0)
+                        w[0] = afma(sval[pf.off + 32 * q], pf.x[q][0], w[0]);
+            };
+            static_assert(M > 1 || B == 8, "the switch covers a batch of 8");
+            if constexpr (std::is_same<AT, float>::value) {  // binary32 FMAs are cheap: no branch
+                sums(std::integral_constant<int, M == 1 ? 8 : 1>{});
+            } else switch (min(pf.width, B)) {
+                case 1: sums(std::integral_constant<int, 1>{}); break;
+                case 2: sums(std::integral_constant<int, 2>{}); break;
+                case 3: sums(std::integral_constant<int, 3>{}); break;
+                case 4: sums(std::integral_constant<int, 4>{}); break;
+                case 5: sums(std::integral_constant<int, 5>{}); break;
+                case 6: sums(std::integral_constant<int, 6>{}); break;
+                case 7: sums(std::integral_constant<int, 7>{}); break;
+                case 8: sums(std::integral_constant<int, M == 1 ? 8 : 1>{}); break;
+                default: break;
+            }
+            if (pf.width > B)  // rare: wide rows
+                w[0] = unit_sum<M, AT>(SVal<VT, AT>{sval.p + pf.off + 32 * B}, SCol{scol + pf.off + 32 * B}, pf.width - B,
+                                       xacc, w[0]);
+            row_epilogue<M, MODE, AT>(a, k, pf.r, w, xin);
+        }
+        for (int sl = cwarp + kCompWarps; sl < u.nsl; sl += kCompWarps) {  // further slices (wide chunks)
+            const int o = 32 * slice_prefix<Shape<SH>::NW>(u.widths, sl);
+            unit_run<M, MODE, AT>(a, k, SVal<VT, AT>{sval.p + o}, SCol{scol + o},
+                                  slice_width<Shape<SH>::NW>(u.widths, sl), (int64_t)u.row0 + 32 * sl, 0, u.row1, xin, xacc,
+                                  lane);
         }
     } else {  // entries in global memory (chunk too large to stage): the slot holds nothing
         release_slot<kCompWarps>(s_empty, pf.slot, lane);
         released = true;
         for (int sl = cwarp; sl < u.nsl; sl += kCompWarps) {
-            const int64_t r = (int64_t)u.row0 + 32 * sl + lane;
-            if (r >= u.row1) continue;
+            const int64_t r0 = (int64_t)u.row0 + 32 * sl;
             const int64_t s0 = __ldg(a.slice_ptr + u.slice0 + sl), s1 = __ldg(a.slice_ptr + u.slice0 + sl + 1);
-            AT w[M];
-            // entries whose x loads are issued together: the unstaged shape issues a row's
-            // loads in batches; the staged shapes keep this rare path small (registers)
-            constexpr int BU = Shape<SH>::SE == 0 ? Batch<M>::B : 1;
-            row_sum<M, BU, AT>(GVal<VT, AT>{static_cast<const typename VT::T *>(a.val) + u.ebase},
-                               GCol{a.col + u.ebase}, s0 - u.ebase + lane, (int)((s1 - s0) >> 5), xacc, w);
-            row_epilogue<M, MODE, AT>(a, k, r, w, xin);
+            const GVal<VT, AT> gv{static_cast<const typename VT::T *>(a.val) + s0};
+            const GCol gc{a.col + s0};
+            const int width = (int)((s1 - s0) >> 5);
+            if constexpr (M == 1) {
+                unit_run<M, MODE, AT>(a, k, gv, gc, width, r0, 0, u.row1, xin, xacc, lane);
+            } else if (r0 + lane < u.row1) {
+                // a row a lane, every column: the entries come from L2 here, and with lanes along the
+                // columns each would be waited for M times (64^3 27-point, 4 columns, p = 8: 923
+                // against 651 us)
+                AT w[M];
+                row_sum<M, Batch<M>::B, AT>(gv, gc, lane, width, xacc, w);
+                row_epilogue<M, MODE, AT>(a, k, r0 + lane, w, xin);
+            }
         }
     }
     if (!released) release_slot<kCompWarps>(s_empty, pf.slot, lane);
@@ -1412,8 +1497,10 @@ __global__ void __launch_bounds__(Shape<SH>::BS, (MpkOcc<M, MODE, TRACE, SH>::bl
                                                      lane, pf);
                 if (tr) {  // wait for the gathers (integer ops only) to split the unit time
                     int h = 0;
+                    if constexpr (M == 1 && kStageEntries > 0) {
 #pragma unroll
-                    for (int q = 0; q < Batch<M>::B; ++q) h ^= hi_bits(pf.x[q][0]);
+                        for (int q = 0; q < Batch<M>::B; ++q) h ^= hi_bits(pf.x[q][0]);
+                    }
                     int d;
                     asm volatile("add.u32 %0, %1, 0;" : "=r"(d) : "r"(h));
                     const long long c1 = clock64();

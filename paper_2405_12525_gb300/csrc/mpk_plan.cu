@@ -1092,8 +1092,9 @@ Plan *build_plan(const mpk_csr *A, const Levels *L, const mpk_plan_opts *o, cuda
         P->work = P->arena.alloc_n<double>((int64_t)P->work_slots * n * m + 1);
         if (P->accum == MPK_F32) P->shadow = P->arena.alloc_n<float>(2 * (int64_t)n * m + 1);
         std::vector<int32_t> wave_host;
-        // ---- wave kernel: single plans of the staged engine whose block shape the planner chose
-        if (o->engine == MPK_ENGINE_STAGED && o->shape == 0 && !batch && !P->level_capped && !P->split_levels &&
+        // ---- wave kernel: single plans of the staged engine, at the planner's block shape or the
+        //      unstaged one
+        if (o->engine == MPK_ENGINE_STAGED && (o->shape == 0 || o->shape == 3) && !batch && !P->level_capped && !P->split_levels &&
             !o->trace && o->shuffle_seed == 0 && n > 0)
             plan_wave(*P, g_slice, c_slice, sptr, chunk_hull, d_srow.p, o->cache_bytes == 0, wave_host, s);
         MPK_CUDA(cudaStreamSynchronize(s));  // host vectors above must outlive their copies

@@ -54,7 +54,6 @@ namespace mpk {
 constexpr int kWaveAux = 4;     // dispatcher, loader, poller, publisher
 constexpr int kWaveWarps = 28;  // compute warps: 16 / 20 / 24 / 28 took 2.34 / 2.15 / 2.03 / 1.99 ms at 256^3, p = 8
 constexpr int kWaveBS = 32 * (kWaveWarps + kWaveAux);
-constexpr int kBatch = 8;       // entries of a row whose x values are gathered together
 constexpr int kDescRing = 512;  // slice descriptors in shared memory
 constexpr int kWaveTiles = 32;  // tiles in shared memory or in flight
 // Entries of the circular buffer, of the widest slice it takes (a wider one is read from global
@@ -101,58 +100,6 @@ struct Deadline {
 // the block's share of a cell of nsl slices: [x, y)
 __device__ __forceinline__ int2 wave_share(int nsl, int block, int blocks) {
     return make_int2((int)((int64_t)nsl * block / blocks), (int)((int64_t)nsl * (block + 1) / blocks));
-}
-
-// Epilogue of one (row, column) of step j at local power k: w is its row sum.  own / back: its
-// values of the two previous steps and old the accumulator (recurrence), or own is x0's value
-// copied to Y[0] (power 1).
-template <int M, int MODE, class AT>
-__device__ __forceinline__ void wave_epilogue(const KArgs &a, int k, int64_t at, bool valid, int lane, AT wa, double own,
-                                              double back, double old) {
-    constexpr bool A32 = sizeof(AT) == 4;
-    const int j = a.k_offset + k;
-    const double w = to_f64(wa);
-    double *y = a.ybase + (int64_t)ring_slot(a, j) * a.ystride + at;
-    if constexpr (MODE == MODE_CHEB) {
-        const double vn = j == 1 ? fma(a.halpha, w, a.hbeta * own) : fma(a.alpha, w, fma(a.beta, own, -back));
-        // complex coefficients act on column pairs, which sit in neighbouring lanes
-        const double other = (M > 1 && a.complex_coeff) ? __shfl_xor_sync(0xffffffffu, vn, 1) : 0.0;
-        if (valid) {
-            *y = vn;
-            if constexpr (A32) a.shadow[(int64_t)(j & 1) * a.ystride + at] = __double2float_rn(vn);
-            double acc = fma(a.cre[k], vn, old);
-            if (M > 1 && a.complex_coeff) acc = fma((lane & 1) ? a.cim[k] : -a.cim[k], other, acc);
-            a.acc[at] = acc;
-        }
-    } else if (valid) {
-        if (!A32 && k == a.p_launch && a.v_ngroups > 1)
-            __stcs(y, w);  // not read again here: see row_epilogue_loaded
-        else
-            *y = w;
-        if constexpr (A32) a.shadow[(int64_t)(j & 1) * a.ystride + at] = (float)wa;
-        if constexpr (MODE == MODE_HOST) __stcs(a.yhost + (int64_t)j * a.ystride + at, w);
-        if (k == 1 && a.y0copy) a.y0copy[at] = own;
-    }
-}
-
-// N entries of the rows of a warp (entry t of a lane's row 32 t places on): their x values are
-// gathered together, then summed in order.  N is exact: an FP64 FMA takes its 64 cycles of the
-// pipe even when no lane of the warp runs it, so sums are never padded to a batch.
-template <int N, int M, class VT, class AT, class VP, class CP>
-__device__ __forceinline__ void wave_batch(VP sv, CP sc, const AT *x, AT &acc) {
-    int c[N];
-    AT xv[N];
-#pragma unroll
-    for (int t = 0; t < N; ++t) {
-        c[t] = sc[32 * t];
-        xv[t] = AT(0);
-        if (c[t] >= 0) xv[t] = x[(int64_t)c[t] * M];
-    }
-#pragma unroll
-    for (int t = 0; t < N; ++t) {
-        const AT v = sv[32 * t];
-        if (c[t] >= 0) acc = afma(v, xv[t], acc);
-    }
 }
 
 template <int M, int MODE, class VT, bool A32>
@@ -353,7 +300,7 @@ __global__ void __launch_bounds__(kWaveBS, 1) k_wave(const KArgs a) {
             const uint32_t run = __shfl_sync(0xffffffffu, ve, after ? __ffs(after) - 2 : 31) - vp;
             if (head && run > 0) {
                 // the launch's last power is the last use of the entries (see k_mpk)
-                const bool last_use = a.v_ngroups > 1 && ((d.ckr >> 6) & 31u) == (uint32_t)a.p_launch;
+                const bool last_use = a.stream_last && ((d.ckr >> 6) & 31u) == (uint32_t)a.p_launch;
                 bulk_g2s(sval + o, static_cast<const T *>(a.val) + 32 * (int64_t)d.e32, run * (uint32_t)sizeof(T), &full[b],
                          last_use);
                 bulk_g2s(scol + o, a.col + 32 * (int64_t)d.e32, run * 4u, &full[b], last_use);
@@ -483,7 +430,6 @@ __global__ void __launch_bounds__(kWaveBS, 1) k_wave(const KArgs a) {
     } else {
         // ------------------------------------------------------------------ compute warps
         const int w = warp - kWaveAux;
-        const int rl = lane / M, cl = lane % M;    // this lane's row of a group, its right-hand side
         int done = 0, ready = 0, seen = 0;
         for (int unit = w;; unit += kWaveWarps) {
             const int idx = unit / M, q = unit % M;
@@ -536,56 +482,18 @@ __global__ void __launch_bounds__(kWaveBS, 1) k_wave(const KArgs a) {
                     }
                 }
             }
-            const double *xin = input_block<M>(a, k);
-            const AT *xacc = InputAcc<M, AT>::get(a, k) + cl;
             if (q * G < rows) {
-                const int r = q * G + rl;
-                const bool valid = r < rows;
-                const int64_t at = ((int64_t)d.row0 + r) * M + cl;
-                // rows of earlier steps that the epilogue reads, on their way during the sums
-                double own = 0.0, back = 0.0, old = 0.0;
-                if constexpr (MODE == MODE_CHEB) {
-                    if (valid) {
-                        own = xin[at];
-                        if (a.k_offset + k != 1)
-                            back = a.ybase[(int64_t)ring_slot(a, a.k_offset + k - 2) * a.ystride + at];
-                        old = a.acc[at];
-                    }
-                } else if (k == 1 && a.y0copy && valid) {
-                    own = a.x0[at];
-                }
-                AT acc = AT(0);
-                int left = d.width;
+                const double *xin = input_block<M>(a, k);
+                const AT *xacc = InputAcc<M, AT>::get(a, k);
+                const int64_t r0 = d.row0, end = r0 + rows;
                 if (lc >= 0) {
-                    const int o = 32 * (lc & 0xffff) + r;
-                    SVal<VT, AT> sv{sval + o};
-                    const int32_t *sc = scol + o;
-                    for (; left >= kBatch; left -= kBatch) {
-                        wave_batch<kBatch, M, VT, AT>(sv, sc, xacc, acc);
-                        sc += 32 * kBatch;
-                        sv.p += 32 * kBatch;
-                    }
-                    switch (left) {
-                        case 1: wave_batch<1, M, VT, AT>(sv, sc, xacc, acc); break;
-                        case 2: wave_batch<2, M, VT, AT>(sv, sc, xacc, acc); break;
-                        case 3: wave_batch<3, M, VT, AT>(sv, sc, xacc, acc); break;
-                        case 4: wave_batch<4, M, VT, AT>(sv, sc, xacc, acc); break;
-                        case 5: wave_batch<5, M, VT, AT>(sv, sc, xacc, acc); break;
-                        case 6: wave_batch<6, M, VT, AT>(sv, sc, xacc, acc); break;
-                        case 7: wave_batch<7, M, VT, AT>(sv, sc, xacc, acc); break;
-                        default: break;
-                    }
+                    const int o = 32 * (lc & 0xffff);
+                    unit_run<M, MODE, AT>(a, k, SVal<VT, AT>{sval + o}, SCol{scol + o}, d.width, r0, q, end, xin, xacc, lane);
                 } else {  // a slice wider than the buffer takes: entries from global memory
-                    const int64_t e = 32 * (int64_t)d.e32 + r;
-                    GVal<VT, AT> gv{static_cast<const T *>(a.val) + e};
-                    GCol gc{a.col + e};
-                    for (; left > 0; --left) {
-                        wave_batch<1, M, VT, AT>(gv, gc, xacc, acc);
-                        gc.p += 32;
-                        gv.p += 32;
-                    }
+                    const int64_t e = 32 * (int64_t)d.e32;
+                    unit_run<M, MODE, AT>(a, k, GVal<VT, AT>{static_cast<const T *>(a.val) + e}, GCol{a.col + e}, d.width, r0,
+                                          q, end, xin, xacc, lane);
                 }
-                wave_epilogue<M, MODE, AT>(a, k, at, valid, lane, acc, own, back, old);
             }
             __syncwarp();
             ++done;

@@ -145,6 +145,25 @@ void mpk::next_epoch(Plan &P, cudaStream_t s) {
     }
 }
 
+void mpk::wave_args(const WaveSet &w, int32_t p, KArgs &a) {
+    a.v_cell = nullptr;
+    if (!w.ok) return;
+    a.v_val = w.val;
+    a.v_col = w.col;
+    a.v_slice = w.slice;
+    a.v_rowmap = w.rowmap;
+    a.v_cell = w.cell + w.cell_off[p];
+    a.v_ncells = w.cell_off[p + 1] - w.cell_off[p];
+    a.v_gsl = w.gsl;
+    a.v_count = w.count;
+    a.v_ngroups = w.ngroups;
+    a.v_maxsl = w.maxsl;
+    a.stream_last = w.ngroups > 1;  // a matrix of one group stays in L2 between launches
+}
+
+// The launch can run in A's own numbering: vectors as the caller has them, no pass before or after.
+static bool runs_natural(const Plan &P) { return P.natural.ok && P.drop_unit < 0; }
+
 KArgs mpk::base_args(Plan &P, int32_t p) {
     KArgs a;
     std::memset(&a, 0, sizeof(a));
@@ -174,7 +193,7 @@ KArgs mpk::base_args(Plan &P, int32_t p) {
     a.ystride = (int64_t)P.n * P.m;
     a.shadow = P.shadow;
     a.p_launch = p;
-    a.stream_last = P.wave ? P.v_ngroups > 1 : 1;
+    a.stream_last = 1;
     if (P.engine == MPK_ENGINE_WARP) {
         a.w_item = P.w_item + P.w_cell_off[p];
         a.w_gk = P.w_gk + P.w_cell_off[p];
@@ -188,15 +207,7 @@ KArgs mpk::base_args(Plan &P, int32_t p) {
         a.w_chunk_nsl = P.w_chunk_nsl;
         a.ngroups = P.num_groups;
     }
-    if (P.wave) {
-        a.v_cell = P.v_cell + P.v_cell_off[p];
-        a.v_ncells = P.v_cell_off[p + 1] - P.v_cell_off[p];
-        a.slice_row = P.slice_row;
-        a.v_gsl = P.v_gsl;
-        a.v_count = P.v_count;
-        a.v_ngroups = P.v_ngroups;
-        a.v_maxsl = P.v_maxsl;
-    }
+    wave_args(P.wave, p, a);
     return a;
 }
 
@@ -220,9 +231,11 @@ extern "C" mpk_status mpk_apply(const mpk_plan_t *Ph, const double *X, int32_t p
         return MPK_OK;
     }
     next_epoch(P, s);
+    const bool natural = runs_natural(P);
     KArgs a = base_args(P, p);
     a.ring = p + 1;
-    if (P.identity || P.order == MPK_ORDER_PLAN) {
+    if (natural) wave_args(P.natural, p, a);
+    if (P.identity || P.order == MPK_ORDER_PLAN || natural) {
         a.x0 = X;
         a.ybase = Y;
         a.y0copy = (Y != X) ? Y : nullptr;
@@ -267,7 +280,8 @@ extern "C" mpk_status mpk_apply_host(const mpk_plan_t *Ph, const double *X_host,
         MPK_CUDA(cudaMemcpyAsync(Y_host, X_host, xbytes, cudaMemcpyHostToHost, s));
         return MPK_OK;
     }
-    if (P.identity || P.order == MPK_ORDER_PLAN) {
+    const bool natural = runs_natural(P);
+    if (P.identity || P.order == MPK_ORDER_PLAN || natural) {
         // X into power block 0 of the workspace.  The staged engine with one right-hand side
         // runs the host-output kernel: power-1 units copy X's rows to Y_host[0] and every power's
         // rows go to Y_host as their units finish.  Other plans compute into the workspace and
@@ -279,6 +293,10 @@ extern "C" mpk_status mpk_apply_host(const mpk_plan_t *Ph, const double *X_host,
         next_epoch(P, s);
         KArgs a = base_args(P, p);
         a.ring = p + 1;
+        if (natural) wave_args(P.natural, p, a);
+        // (with many groups in plan order the output link is the bound, and k_mpk's finer units feed it
+        // evenly: 128^3, p = 8, 999 against 1004 us)
+        if (fused && !natural && P.wave.ngroups > 1) a.v_cell = nullptr;
         a.x0 = P.work;
         a.ybase = P.work;
         if (P.accum == MPK_F32) launch_round_f32(P.work, nm, P.shadow, s);
@@ -339,10 +357,11 @@ extern "C" mpk_status mpk_spmv_powers(const mpk_plan_t *Ph, const double *X, int
 // accumulator.  cheb_start: v_0 = X (gathered into plan order if the plan keeps A's order),
 // acc = c_0 v_0.  cheb_steps: steps k_begin+1 .. k_end, in launches of at most p_max steps; the
 // ring indices follow the absolute step, so any split of the steps gives the same bits.
+// natural: the state is in A's own numbering (one call's own state only; the caller's is in plan order).
 static void cheb_start(Plan &P, const double *X, double c0_re, double c0_im, bool cplx, double *ring, double *acc,
-                       cudaStream_t s) {
+                       cudaStream_t s, bool natural = false) {
     const int64_t nm = (int64_t)P.n * P.m;
-    if (P.identity || P.order == MPK_ORDER_PLAN)
+    if (P.identity || P.order == MPK_ORDER_PLAN || natural)
         MPK_CUDA(cudaMemcpyAsync(ring, X, sizeof(double) * nm, cudaMemcpyDeviceToDevice, s));
     else
         launch_gather_rows(X, P.perm, ring, P.n, P.m, s);
@@ -350,7 +369,7 @@ static void cheb_start(Plan &P, const double *X, double c0_re, double c0_im, boo
 }
 
 static void cheb_steps(Plan &P, double *ring, double *acc, int32_t k_begin, int32_t k_end, const double *coeff_re,
-                       const double *coeff_im, double scale, double shift, cudaStream_t s) {
+                       const double *coeff_im, double scale, double shift, cudaStream_t s, bool natural = false) {
     // same expressions as the recurrence's definition: 2A'v = alpha Av + beta v
     const double alpha = 2.0 / scale, beta = -2.0 * shift / scale;
     const double halpha = 1.0 / scale, hbeta = -shift / scale;
@@ -364,6 +383,7 @@ static void cheb_steps(Plan &P, double *ring, double *acc, int32_t k_begin, int3
         const int32_t pb = std::min(P.p_max, k_end - j0);
         next_epoch(P, s);
         KArgs a = base_args(P, pb);
+        if (natural) wave_args(P.natural, pb, a);
         a.x0 = ring;
         a.ybase = ring;
         a.ring = 3;
@@ -398,10 +418,11 @@ extern "C" mpk_status mpk_cheb_filter(const mpk_plan_t *Ph, const double *X, int
     if (P.n == 0) return MPK_OK;
     cudaStream_t s = as_stream(stream);
     const int64_t nm = (int64_t)P.n * P.m;
-    const bool plan_order = P.identity || P.order == MPK_ORDER_PLAN;
+    const bool natural = runs_natural(P);
+    const bool plan_order = P.identity || P.order == MPK_ORDER_PLAN || natural;
     double *acc = plan_order ? out : P.work + 3 * nm;
-    cheb_start(P, X, coeff_re[0], coeff_im ? coeff_im[0] : 0.0, coeff_im != nullptr, P.work, acc, s);
-    cheb_steps(P, P.work, acc, 0, degree, coeff_re, coeff_im, scale, shift, s);
+    cheb_start(P, X, coeff_re[0], coeff_im ? coeff_im[0] : 0.0, coeff_im != nullptr, P.work, acc, s, natural);
+    cheb_steps(P, P.work, acc, 0, degree, coeff_re, coeff_im, scale, shift, s, natural);
     if (!plan_order) launch_scatter_rows(acc, P.iperm, out, P.n, P.m, s);
     return MPK_OK;
     MPK_GUARD_END

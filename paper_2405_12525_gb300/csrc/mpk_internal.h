@@ -286,11 +286,14 @@ struct KArgs {
     const int32_t *w_chunk_nsl;    // slices of every chunk
     int32_t ngroups;
     int32_t p_launch;              // powers of this launch (local 1..p_launch)
-    // wave kernel (static schedule): the cells of this launch in line order as (first slice,
-    // slices, g << 5 | k, 0), the rows of every slice, the slices of every group and the finished
-    // slices per (power, group); zero when the launch starts
+    // wave kernel (static schedule): its sliced copy, the cells of this launch in line order as
+    // (first slice, slices, g << 5 | k, 0), the rows of every slice, the slices of every group and
+    // the finished slices per (power, group), zero when the launch starts
+    const void *v_val;
+    const int32_t *v_col;
+    const int4 *v_slice;       // slices: (first entry / 32, entries a row, first row or row map entry, rows)
+    const int32_t *v_rowmap;   // row of every lane of every slice (-1: none), or null: consecutive rows
     const int4 *v_cell;
-    const int32_t *slice_row;  // slices + 1
     const int32_t *v_gsl;
     int32_t *v_count;          // (p + 1) x v_ngroups
     int32_t v_ncells, v_ngroups;
@@ -303,6 +306,19 @@ constexpr int kWaveMaxCells = 1 << 20;  // cells of a wave launch (a descriptor 
 // warp-ticketed engine: slices per item, claim queues (one per warp of a block)
 constexpr int kWarpSlices = 1;
 constexpr int kWarpQueues = 16;
+
+// Tables of the wave kernel over one sliced copy of the matrix (device memory of the plan)
+struct WaveSet {
+    bool ok = false;
+    const void *val = nullptr;
+    const int32_t *col = nullptr;
+    const int32_t *rowmap = nullptr;  // rows of the slices' lanes when they are sorted by length
+    int32_t ngroups = 0, maxsl = 0;
+    int4 *cell = nullptr;             // cells of every p, concatenated
+    std::vector<int32_t> cell_off;    // pmax + 2: the cells of p start at cell_off[p]
+    int4 *slice = nullptr;            // records of the slices (see KArgs::v_slice)
+    int32_t *gsl = nullptr, *count = nullptr;
+};
 
 struct Plan {
     int32_t n = 0, nnz = 0, m = 1, p_max = 8, order = MPK_ORDER_ORIGINAL;
@@ -354,12 +370,9 @@ struct Plan {
     int32_t *w_cnt = nullptr;           // (p_max+1) x nchunks counters, then kWarpQueues claim counters
     int32_t *w_slice_chunk = nullptr;   // chunk of every slice (device)
     int32_t *w_chunk_nsl = nullptr;     // slices of every chunk (device)
-    // wave kernel (single plans of the staged engine at the planner's own block shape)
-    bool wave = false;
-    int32_t v_ngroups = 0, v_maxsl = 0;
-    int4 *v_cell = nullptr;             // cells of every p, concatenated
-    std::vector<int32_t> v_cell_off;    // pmax + 2: the cells of p start at v_cell_off[p]
-    int32_t *slice_row = nullptr, *v_gsl = nullptr, *v_count = nullptr;
+    // wave kernel (single plans of the staged engine at the planner's own block shape): in plan
+    // order, and, for original-order plans whose matrix has a narrow band, in the matrix's own
+    WaveSet wave, natural;
     int32_t drop_unit = -1;  // armed by mpk_debug_drop_release for the next launch
     unsigned long long *trace = nullptr;  // counters when built with opts.trace
     int grid_mpk[4] = {0, 0, 0, 0};  // persistent grid size per mode
@@ -412,7 +425,8 @@ void widen_values(int vtype, const void *src, int64_t n, double *dst, cudaStream
 // level builder (mpk_levels.cu)
 // BFS levels from `root`, or from every vertex of `roots` (ascending) as level 0
 Levels *build_levels(const mpk_csr *A, int32_t root, cudaStream_t s, const std::vector<int32_t> *roots = nullptr);
-void validate_csr(const mpk_csr *A, cudaStream_t s);
+// bandwidth, if given: the largest |column - row|
+void validate_csr(const mpk_csr *A, cudaStream_t s, int32_t *bandwidth = nullptr);
 
 // planner (mpk_plan.cu)
 // inst_row / inst_p: batch plans only (instance row offsets, count + 1 entries; powers per instance)
@@ -420,6 +434,8 @@ void validate_csr(const mpk_csr *A, cudaStream_t s);
 void next_epoch(Plan &P, cudaStream_t s);
 // kernel arguments of P for the unit table of power p
 KArgs base_args(Plan &P, int32_t p);
+// the wave kernel's arguments of a launch with p powers (none if the set is not there)
+void wave_args(const WaveSet &w, int32_t p, KArgs &a);
 Plan *build_plan(const mpk_csr *A, const Levels *L, const mpk_plan_opts *o, cudaStream_t s,
                  const std::vector<int32_t> *inst_row = nullptr, const std::vector<int32_t> *inst_p = nullptr);
 void export_csr(const Plan &P, int32_t *rp, int32_t *ci, double *va, cudaStream_t s);

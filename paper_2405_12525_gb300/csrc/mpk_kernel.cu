@@ -521,7 +521,7 @@ static void *select_wave(int mode, int m, int vtype, bool a32, int *smem) {
 
 void launch_mpk(const Plan &P, KArgs &a, int mode, cudaStream_t s) {
     const bool a32 = P.accum == MPK_F32;
-    if (P.wave && a.v_cell != nullptr && a.drop_unit < 0) {
+    if (a.v_cell != nullptr && a.drop_unit < 0) {
         const int grid = std::min(device_sms(), a.v_maxsl);
         int smem = 0;
         void *fn = select_wave(mode, P.m, P.val_type, a32, &smem);

@@ -459,21 +459,27 @@ __device__ __forceinline__ void unit_rows(const KArgs &a, int k, int64_t at, boo
     }
 }
 
-// One unit: the 32 / M rows from row r0 + q * 32 / M of a slice (those below `end`), every right-hand
-// side, step k: lane l owns row l / M of them and right-hand side l % M.  sv / sc: the entries of
-// the slice's first row (they advance by lane row here).
+// One unit: 32 / M rows of a slice, every right-hand side, step k.  Lane l owns the slice's row
+// rl = q * 32 / M + l / M (row number `row`, if valid) and right-hand side l % M; sv / sc: the entries of
+// the slice's first row.
 template <int M, int MODE, class AT, class VP, class CP>
-__device__ __forceinline__ void unit_run(const KArgs &a, int k, VP sv, CP sc, int width, int64_t r0, int q, int64_t end,
+__device__ __forceinline__ void unit_row(const KArgs &a, int k, VP sv, CP sc, int width, int rl, int64_t row, bool valid,
                                          const double *xin, const AT *xacc, int lane) {
-    const int rl = q * (32 / M) + lane / M, cl = lane % M;
-    const bool valid = r0 + rl < end;
-    const int64_t at = (r0 + rl) * M + cl;
+    const int cl = lane % M;
+    const int64_t at = row * M + cl;
     double own = 0.0, back = 0.0, old = 0.0;
     unit_rows<MODE>(a, k, at, valid, xin, own, back, old);  // on their way during the sums
     sv.p += rl;
     sc.p += rl;
     const AT acc = unit_sum<M, AT>(sv, sc, width, xacc + cl);
     unit_epilogue<M, MODE, AT>(a, k, at, valid, lane, acc, own, back, old);
+}
+// unit q of a slice of consecutive rows from r0 (those below `end`)
+template <int M, int MODE, class AT, class VP, class CP>
+__device__ __forceinline__ void unit_run(const KArgs &a, int k, VP sv, CP sc, int width, int64_t r0, int q, int64_t end,
+                                         const double *xin, const AT *xacc, int lane) {
+    const int rl = q * (32 / M) + lane / M;
+    unit_row<M, MODE, AT>(a, k, sv, sc, width, rl, r0 + rl, r0 + rl < end, xin, xacc, lane);
 }
 
 // ----------------------------------------------------------------------------- K-MPK

@@ -2,17 +2,15 @@
 // BFS permutation (Sec. 3, level definition, prose and Fig. 1).
 #include "mpk_internal.h"
 
-#include <cooperative_groups.h>
-
 #include <algorithm>
 #include <climits>
 
 namespace mpk {
-namespace cg = cooperative_groups;
 
-// err[0]: bad row pointer, err[1]: column out of range
+// err[0]: bad row pointer, err[1]: column out of range, err[2]: largest |column - row|
 __global__ void k_validate(int32_t n, int32_t nnz, const int32_t *rp, const int32_t *ci, int32_t *err) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    int32_t band = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += stride) {
         const int32_t a = rp[i], b = rp[i + 1];
         if (a > b || a < 0 || b > nnz || (i == 0 && a != 0) || (i == n - 1 && b != nnz)) {
@@ -25,11 +23,15 @@ __global__ void k_validate(int32_t n, int32_t nnz, const int32_t *rp, const int3
                 atomicExch(&err[1], 1);
                 break;
             }
+            band = max(band, abs(c - (int32_t)i));
         }
     }
+    band = __reduce_max_sync(0xffffffffu, band);
+    if ((threadIdx.x & 31) == 0 && band > err[2]) atomicMax(&err[2], band);
 }
 
-void validate_csr(const mpk_csr *A, cudaStream_t s) {
+void validate_csr(const mpk_csr *A, cudaStream_t s, int32_t *bandwidth) {
+    if (bandwidth) *bandwidth = 0;
     if (!A) fail(MPK_ERR_INVALID, "matrix is NULL");
     if (A->n < 0 || A->nnz < 0) fail(MPK_ERR_INVALID, "negative n (%d) or nnz (%d)", A->n, A->nnz);
     if (A->val_type != MPK_F64 && A->val_type != MPK_F32 && A->val_type != MPK_BF16)
@@ -37,17 +39,18 @@ void validate_csr(const mpk_csr *A, cudaStream_t s) {
     if (A->n == 0) return;
     if (!A->row_ptr || (A->nnz > 0 && (!A->col || !A->val)))
         fail(MPK_ERR_INVALID, "NULL CSR array");
-    Tmp<int32_t> err(2, s);
-    MPK_CUDA(cudaMemsetAsync(err.p, 0, 2 * sizeof(int32_t), s));
+    Tmp<int32_t> err(3, s);
+    MPK_CUDA(cudaMemsetAsync(err.p, 0, 3 * sizeof(int32_t), s));
     int g = (int)((A->n + 255) / 256);
     if (g > device_sms() * 16) g = device_sms() * 16;
     k_validate<<<g, 256, 0, s>>>(A->n, A->nnz, A->row_ptr, A->col, err.p);
     MPK_LAUNCHED();
-    int32_t h[2];
+    int32_t h[3];
     MPK_CUDA(cudaMemcpyAsync(h, err.p, sizeof(h), cudaMemcpyDeviceToHost, s));
     MPK_CUDA(cudaStreamSynchronize(s));
     if (h[0]) fail(MPK_ERR_INVALID, "row_ptr is not a valid CSR row pointer (0 .. nnz, non-decreasing)");
     if (h[1]) fail(MPK_ERR_INVALID, "column index outside [0, n)");
+    if (bandwidth) *bandwidth = h[2];
 }
 
 // ----------------------------------------------------------------------------- A^T pattern
@@ -66,19 +69,29 @@ __global__ void k_tfill(int32_t n, const int32_t *rp, const int32_t *ci, int32_t
 
 // ----------------------------------------------------------------------------- BFS on the device
 // The whole level-synchronous BFS in one cooperative launch (every block resident): per level the
-// blocks expand the frontier queue[head, tail) into level lev + 1 (appending at queue[tail + ..]),
-// meet at a grid barrier and all read the number found, so every block advances head, tail and
-// lev identically.  The counters rotate through three slots: phase q adds to slot q % 3 and
-// resets slot (q + 1) % 3, whose last readers (after barrier q - 2) have all passed barrier q - 1.
+// blocks expand the frontier queue[head, tail) into level lev + 1 (appending behind it) and meet at a
+// grid barrier whose word also carries the number of vertices found so far, so every block advances
+// head, tail and lev identically.  A level is bound by its chain of dependent round trips: queue
+// entry with its row bounds, columns, levels, claims, one addition to the queue's end per warp
+// beside the winners' row bounds, and the barrier's two.  Levels of up to kBfsNarrow vertices are
+// expanded by one block alone (256 / 512 / 1024 / 2048: 1500x1300 grid, 2799 levels, 13.6 / 12.6 /
+// 14.6 / 18.1 ms).  Against a version that appended neighbour by neighbour and read the count after
+// the barrier: 256^3 8.99 -> 7.97 ms, 131x127x113 3.14 -> 2.95 ms, banded 300k 2.70 -> 2.03 ms.
+// (Claims without a look at the level first, and prefetches of the winners' columns: slower.)
 // A graph whose search runs dry before every vertex is reached continues from the smallest
 // untouched vertex (a grid-wide minimum, one barrier), which opens the next level (one more
-// barrier to publish it).  Every barrier wait is bounded; on expiry the kernel records the
-// failure and all blocks leave.
+// barrier to publish it); the minima rotate through three slots, so that a slot is reset only
+// after its last readers passed the next barrier.  Every barrier wait is bounded; on expiry the
+// kernel records the failure and all blocks leave.
 constexpr int64_t kBfsWaitNs = 2000000000LL;  // bound of one grid-barrier wait (2 s)
+constexpr int kBfsBS = 512;                   // one block an SM: half the arrivals of two blocks of 256
+constexpr int kBfsNarrow = 512;               // vertices of a level that one block expands alone
+constexpr int kBfsAlone = 1 << 15;            // levels it expands before it meets the others
 struct BfsState {
-    unsigned int bar_count;  // arrivals at grid barriers, all rounds
-    int32_t cnt[3];    // vertices found per phase
-    int32_t minv[3];   // smallest untouched vertex per phase (INT_MAX: none)
+    unsigned long long bar;  // arrivals at grid barriers, all rounds, << 32 | vertices found, all levels
+    int4 left[2];      // where block 0 left the narrow levels: head, tail, level
+    int32_t tail;      // end of the queue
+    int32_t minv[3];   // smallest untouched vertex per restart (INT_MAX: none)
     int32_t levels;    // number of levels (written at the end)
     int32_t err;       // 1: a barrier wait expired, 2: the search lost track of untouched vertices
 };
@@ -92,88 +105,156 @@ __device__ __forceinline__ uint64_t bfs_clock() {
 // block): the arrivals only grow, and barrier r is passed once r * gridDim.x blocks arrived.
 // Thread 0 arrives with an acquire-release add (the block's writes, ordered before it by the
 // block barrier, are released; the earlier arrivals acquired) and polls with acquire loads.
-// False when the wait expired (recorded in st->err).
-__device__ __forceinline__ bool bfs_grid_barrier(BfsState *st, unsigned int round, int64_t limit_ns) {
-    __shared__ int s_ok;
+// `found`: what this block's threads found since the last barrier (in shared memory; cleared).
+// Returns the vertices found by all blocks so far, or -1 when the wait expired (recorded in st->err).
+__device__ __forceinline__ int64_t bfs_grid_barrier(BfsState *st, unsigned int round, int *found, int64_t limit_ns) {
+    __shared__ int64_t s_all;
     __syncthreads();
     if (threadIdx.x == 0) {
         const unsigned int target = round * gridDim.x;
-        unsigned int v;
-        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(v) : "l"(&st->bar_count) : "memory");
-        s_ok = 1;
-        if (v + 1 < target) {
-            const uint64_t t0 = bfs_clock();
-            for (;;) {
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&st->bar_count) : "memory");
-                if (v >= target) break;
-                if (bfs_clock() - t0 > (uint64_t)limit_ns) {
-                    atomicCAS(&st->err, 0, 1);
-                    s_ok = 0;
-                    break;
+        const unsigned long long add = (1ULL << 32) | (unsigned int)*found;
+        unsigned long long v;
+        asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], %2;" : "=l"(v) : "l"(&st->bar), "l"(add) : "memory");
+        v += add;
+        *found = 0;
+        bool ok = true;
+        if ((unsigned int)(v >> 32) != target) {
+            uint64_t t0 = 0;
+            for (int spin = 1;; ++spin) {
+                asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&st->bar) : "memory");
+                // (the next round's arrivals cannot come before this block passed this one)
+                if ((unsigned int)(v >> 32) >= target) break;
+                if ((spin & 63) == 0) {
+                    const uint64_t t = bfs_clock();
+                    if (t0 == 0) t0 = t;
+                    if (t - t0 > (uint64_t)limit_ns) {
+                        atomicCAS(&st->err, 0, 1);
+                        ok = false;
+                        break;
+                    }
                 }
-                __nanosleep(32);
             }
         }
+        s_all = ok ? (int64_t)(v & 0xffffffffULL) : -1;
     }
     __syncthreads();
-    return s_ok != 0;
+    return s_all;
 }
 
-// appends u at queue[tail + *cnt++]; the lanes of a warp that append together (a coalesced
-// group) share one atomic, each writing at its rank in the group
-__device__ __forceinline__ void bfs_append(int32_t *queue, int64_t tail, int32_t *cnt, int32_t u) {
-    cg::coalesced_group g = cg::coalesced_threads();
-    int32_t base = 0;
-    if (g.thread_rank() == 0) base = atomicAdd(cnt, (int32_t)g.size());
-    base = g.shfl(base, 0);
-    queue[tail + base + (int64_t)g.thread_rank()] = u;
-}
-
-// neighbours ci[e0 .. e1) of v join level `next` unless reached (CAS from -1), eight at a time:
-// their columns, then their levels, then the claims, so that a vertex's work is a few memory
-// round trips instead of two per neighbour
-__device__ __forceinline__ void bfs_visit(const int32_t *ci, int32_t e0, int32_t e1, int32_t v, int32_t *level_of,
-                                          int32_t next, int32_t *queue, int64_t tail, int32_t *cnt) {
-    for (int32_t eb = e0; eb < e1; eb += 8) {
-        int32_t u[8], l[8];
+// Neighbours vi[e0 .. e1) of v (none when e0 == e1) join level `next` unless reached (compare-and-swap
+// from -1), eight at a time, by a whole warp: the claims of all lanes, then one addition to the
+// queue's end for all that the warp won (its entries: the vertex and its row bounds).  Returns the
+// warp's wins.
+__device__ __forceinline__ int bfs_visit(const int32_t *rp, const int32_t *vi, int32_t e0, int32_t e1,
+                                         int32_t v, int32_t *level_of, int32_t next, int4 *queue, int32_t *tail, int lane) {
+    int all = 0;
+    const int most = __reduce_max_sync(0xffffffffu, e1 - e0);
+    for (int j = 0; j < most; j += 8) {
+        int32_t u[8];
+        int32_t old[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) u[q] = (eb + q < e1) ? ci[eb + q] : v;
+        for (int q = 0; q < 8; ++q) u[q] = (e0 + j + q < e1) ? vi[e0 + j + q] : v;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) l[q] = (u[q] != v) ? level_of[u[q]] : 0;
+        for (int q = 0; q < 8; ++q) old[q] = u[q] != v ? *(volatile int32_t *)&level_of[u[q]] : 0;
 #pragma unroll
         for (int q = 0; q < 8; ++q)
-            if (l[q] < 0 && atomicCAS(&level_of[u[q]], -1, next) == -1) bfs_append(queue, tail, cnt, u[q]);
+            if (old[q] == -1) old[q] = atomicCAS(&level_of[u[q]], -1, next);
+        // row bounds of the vertices won, for their queue entries: on their way with the addition below
+        int32_t b0[8], b1[8];
+        int mine = 0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            b0[q] = b1[q] = 0;
+            if (old[q] == -1) {
+                b0[q] = rp[u[q]];
+                b1[q] = rp[u[q] + 1];
+                ++mine;
+            }
+        }
+        int end = mine;  // inclusive prefix sum over the warp
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, end, o);
+            if (lane >= o) end += x;
+        }
+        const int total = __shfl_sync(0xffffffffu, end, 31);
+        if (total == 0) continue;
+        int base = 0;
+        if (lane == 0) base = atomicAdd(tail, total);
+        int at = __shfl_sync(0xffffffffu, base, 0) + end - mine;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (old[q] == -1) queue[at++] = make_int4(u[q], b0[q], b1[q], 0);
+        all += total;
     }
+    return all;
 }
 
-__global__ void __launch_bounds__(256) k_bfs_all(const int32_t *rp, const int32_t *ci, const int32_t *tp,
-                                                 const int32_t *tci, int32_t *level_of, int32_t *queue, int32_t n,
-                                                 int32_t head0, int32_t tail0, BfsState *st, int64_t limit_ns) {
+__global__ void __launch_bounds__(kBfsBS, 1) k_bfs_all(const int32_t *rp, const int32_t *ci, const int32_t *tp,
+                                                    const int32_t *tci, int32_t *level_of, int4 *queue, int32_t n,
+                                                    int32_t head0, int32_t tail0, BfsState *st, int64_t limit_ns) {
+    __shared__ int s_found, s_tail;
     const int64_t gtid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t gstride = (int64_t)gridDim.x * blockDim.x;
-    int64_t head = head0, tail = tail0, cursor = 0;
+    const int lane = threadIdx.x & 31;
+    int64_t head = head0, tail = tail0, cursor = 0, found0 = 0;
     int32_t lev = 0;
-    int q = 0;               // phase
+    int q = 0;               // restart
     unsigned int round = 0;  // grid barriers passed
+    if (threadIdx.x == 0) s_found = 0;
+    __syncthreads();
+    // the vertices queue[t], t = first, first + step, ... below `last` (whole warps), into level `next`
+    auto expand = [&](int64_t first, int64_t step, int64_t last, int32_t next, int32_t *end) -> int {
+        int wins = 0;
+        for (int64_t t = first; t - lane < last; t += step) {
+            const bool on = t < last;
+            const int4 e = on ? queue[t] : make_int4(0, 0, 0, 0);
+            wins += bfs_visit(rp, ci, e.y, e.z, e.x, level_of, next, queue, end, lane);
+            if (tp) {
+                const int32_t f0 = on ? tp[e.x] : 0, f1 = on ? tp[e.x + 1] : 0;
+                wins += bfs_visit(rp, tci, f0, f1, e.x, level_of, next, queue, end, lane);
+            }
+        }
+        return wins;
+    };
     for (;;) {
-        // expand level lev
-        if (gtid == 0) {
-            st->cnt[(q + 1) % 3] = 0;
-            st->minv[(q + 1) % 3] = INT_MAX;
+        if (tail > head && tail - head <= kBfsNarrow) {
+            // narrow levels: block 0 alone, with block barriers and the queue's end in shared memory,
+            // while the others wait at one grid barrier (kBfsAlone levels at most, well inside its bound)
+            if (blockIdx.x == 0) {
+                int32_t h = (int32_t)head, t = (int32_t)tail, l = lev;
+                for (int it = 0; it < kBfsAlone && t > h && t - h <= kBfsNarrow; ++it) {
+                    if (threadIdx.x == 0) s_tail = t;
+                    __syncthreads();
+                    expand(h + threadIdx.x, blockDim.x, t, l + 1, &s_tail);
+                    __syncthreads();
+                    h = t;
+                    t = s_tail;
+                    if (t > h) ++l;
+                    __syncthreads();
+                }
+                if (threadIdx.x == 0) {
+                    st->tail = t;
+                    st->left[(round + 1) & 1] = make_int4(h, t, l, 0);
+                }
+            }
+            if (bfs_grid_barrier(st, ++round, &s_found, limit_ns) < 0) return;
+            // (two places in turn: block 0 writes this one again only after the next barrier)
+            const volatile int4 *left = &st->left[round & 1];
+            head = left->x;
+            tail = left->y;
+            lev = left->z;
+            continue;
         }
-        int32_t *cnt = &st->cnt[q % 3];
-        for (int64_t t = head + gtid; t < tail; t += gstride) {
-            const int32_t v = queue[t];
-            bfs_visit(ci, rp[v], rp[v + 1], v, level_of, lev + 1, queue, tail, cnt);
-            if (tp) bfs_visit(tci, tp[v], tp[v + 1], v, level_of, lev + 1, queue, tail, cnt);
-        }
-        if (!bfs_grid_barrier(st, ++round, limit_ns)) return;
-        const int32_t found = *(volatile int32_t *)cnt;
-        ++q;
-        head = tail;
-        tail += found;
-        if (found > 0) {
-            ++lev;
+        if (tail > head) {  // expand level lev (st->tail == tail)
+            const int wins = expand(head + gtid, gstride, tail, lev + 1, &st->tail);
+            if (lane == 0 && wins) atomicAdd(&s_found, wins);
+            const int64_t all = bfs_grid_barrier(st, ++round, &s_found, limit_ns);
+            if (all < 0) return;
+            head = tail;
+            tail += all - found0;
+            if (all > found0) ++lev;
+            found0 = all;
             continue;
         }
         if (tail >= n) break;
@@ -184,11 +265,8 @@ __global__ void __launch_bounds__(256) k_bfs_all(const int32_t *rp, const int32_
                 atomicMin(mn, (int32_t)i);
                 break;
             }
-        if (gtid == 0) {
-            st->cnt[(q + 1) % 3] = 0;
-            st->minv[(q + 1) % 3] = INT_MAX;
-        }
-        if (!bfs_grid_barrier(st, ++round, limit_ns)) return;
+        if (gtid == 0) st->minv[(q + 1) % 3] = INT_MAX;
+        if (bfs_grid_barrier(st, ++round, &s_found, limit_ns) < 0) return;
         const int32_t v = *(volatile int32_t *)mn;
         ++q;
         if (v == INT_MAX) {
@@ -199,24 +277,25 @@ __global__ void __launch_bounds__(256) k_bfs_all(const int32_t *rp, const int32_
         ++lev;
         if (gtid == 0) {
             level_of[v] = lev;
-            queue[tail] = v;
+            queue[tail] = make_int4(v, rp[v], rp[v + 1], 0);
+            st->tail = (int32_t)tail + 1;
         }
         tail += 1;
-        if (!bfs_grid_barrier(st, ++round, limit_ns)) return;  // the new root before its expansion
+        if (bfs_grid_barrier(st, ++round, &s_found, limit_ns) < 0) return;  // the new root before its expansion
     }
     if (gtid == 0) st->levels = lev + 1;
 }
 
-__global__ void k_set_root(int32_t *level_of, int32_t *queue_slot, int32_t v, int32_t level) {
+__global__ void k_set_root(const int32_t *rp, int32_t *level_of, int4 *queue_slot, int32_t v, int32_t level) {
     level_of[v] = level;
-    *queue_slot = v;
+    *queue_slot = make_int4(v, rp[v], rp[v + 1], 0);
 }
 
 // level 0 = every root (roots distinct)
-__global__ void k_set_roots(int32_t *level_of, int32_t *queue, const int32_t *roots, int32_t nroots) {
+__global__ void k_set_roots(const int32_t *rp, int32_t *level_of, int4 *queue, const int32_t *roots, int32_t nroots) {
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nroots; i += gridDim.x * blockDim.x) {
         level_of[roots[i]] = 0;
-        queue[i] = roots[i];
+        queue[i] = make_int4(roots[i], rp[roots[i]], rp[roots[i] + 1], 0);
     }
 }
 
@@ -261,10 +340,10 @@ Levels *build_levels(const mpk_csr *A, int32_t root, cudaStream_t s, const std::
     Levels *L = new Levels();
     try {
         L->n = n;
-        L->level_ptr = L->arena.alloc_n<int32_t>((int64_t)n + 1);
-        L->perm = L->arena.alloc_n<int32_t>(n);
-        L->iperm = L->arena.alloc_n<int32_t>(n);
-        L->level_of = L->arena.alloc_n<int32_t>(n);
+        L->perm = L->arena.alloc_n<int32_t>(4 * (int64_t)n + 1);  // one block (a large cudaMalloc takes 50 us)
+        L->iperm = L->perm + n;
+        L->level_of = L->iperm + n;
+        L->level_ptr = L->level_of + n;
         if (n == 0) {
             MPK_CUDA(cudaMemsetAsync(L->level_ptr, 0, sizeof(int32_t), s));
             MPK_CUDA(cudaStreamSynchronize(s));
@@ -286,39 +365,40 @@ Levels *build_levels(const mpk_csr *A, int32_t root, cudaStream_t s, const std::
             MPK_CUDA(cudaStreamSynchronize(s));
         }
         // level-synchronous BFS; queue holds the levels back to back
-        Tmp<int32_t> queue(n, s);
+        Tmp<int4> queue(n, s);  // (vertex, its row bounds)
         MPK_CUDA(cudaMemsetAsync(L->level_of, 0xff, sizeof(int32_t) * (size_t)n, s));
         int64_t head = 0, tail = 1;
         if (roots) {
             const int32_t nr = (int32_t)roots->size();
             Tmp<int32_t> d_roots(nr, s);
             MPK_CUDA(cudaMemcpyAsync(d_roots.p, roots->data(), sizeof(int32_t) * (size_t)nr, cudaMemcpyHostToDevice, s));
-            k_set_roots<<<grid_n(nr), 256, 0, s>>>(L->level_of, queue.p, d_roots.p, nr);
+            k_set_roots<<<grid_n(nr), 256, 0, s>>>(A->row_ptr, L->level_of, queue.p, d_roots.p, nr);
             MPK_LAUNCHED();
             MPK_CUDA(cudaStreamSynchronize(s));  // the host root list and d_roots go out of scope
             tail = nr;
         } else {
-            k_set_root<<<1, 1, 0, s>>>(L->level_of, queue.p, root, 0);
+            k_set_root<<<1, 1, 0, s>>>(A->row_ptr, L->level_of, queue.p, root, 0);
             MPK_LAUNCHED();
         }
         // the levels, in one cooperative launch (every block resident)
         Tmp<BfsState> st(1, s);
-        MPK_CUDA(cudaMemsetAsync(st.p, 0, sizeof(BfsState), s));
+        const BfsState st0{0, {}, (int32_t)tail, {INT_MAX, INT_MAX, INT_MAX}, 0, 0};
+        MPK_CUDA(cudaMemcpyAsync(st.p, &st0, sizeof(BfsState), cudaMemcpyHostToDevice, s));
         int per_sm = 0;
-        MPK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bfs_all, 256, 0));
+        MPK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bfs_all, kBfsBS, 0));
         if (per_sm < 1) fail(MPK_ERR_CUDA, "the BFS kernel does not fit an SM");
-        // two blocks per SM: enough threads for the widest frontiers, few arrivals per barrier
-        const int grid = std::min(per_sm, 2) * device_sms();
+        const int grid = device_sms();
         const int32_t *rpp = A->row_ptr, *cip = A->col;
         const int32_t *tpp = A->is_symmetric ? nullptr : tp.p;
         const int32_t *tcip = tci.p;
-        int32_t *lvl = L->level_of, *qp = queue.p;
+        int32_t *lvl = L->level_of;
+        int4 *qp = queue.p;
         int32_t nn = n, h0 = (int32_t)head, t0 = (int32_t)tail;
         BfsState *stp = st.p;
         int64_t limit = kBfsWaitNs;
         void *args[] = {(void *)&rpp, (void *)&cip, (void *)&tpp, (void *)&tcip, (void *)&lvl, (void *)&qp,
                         (void *)&nn, (void *)&h0, (void *)&t0, (void *)&stp, (void *)&limit};
-        MPK_CUDA(cudaLaunchCooperativeKernel((const void *)k_bfs_all, dim3(grid), dim3(256), args, 0, s));
+        MPK_CUDA(cudaLaunchCooperativeKernel((const void *)k_bfs_all, dim3(grid), dim3(kBfsBS), args, 0, s));
         MPK_LAUNCHED();
         BfsState hs;
         MPK_CUDA(cudaMemcpyAsync(&hs, st.p, sizeof(BfsState), cudaMemcpyDeviceToHost, s));

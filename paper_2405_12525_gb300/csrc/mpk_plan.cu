@@ -102,7 +102,10 @@ __global__ void k_dep_bits(int32_t n, const int32_t *rowlen, const int32_t *chun
         const int32_t lo_c = hull[c].x;
         auto set = [&](int32_t owner, int32_t owner_lo, int32_t target) {
             const int32_t off = target - owner_lo;
-            atomicOr(&bits[word_off[owner] + (off >> 5)], 1u << (off & 31));
+            // (most rows of a chunk set the same few bits: look before the atomic; 1.9 M rows, this
+            // phase 580 -> 217 us)
+            uint32_t *w = &bits[word_off[owner] + (off >> 5)];
+            if (!((*w >> (off & 31)) & 1u)) atomicOr(w, 1u << (off & 31));
         };
         set(c, lo_c, c);
         int32_t last = -1;
@@ -331,61 +334,131 @@ void export_csr(const Plan &P, int32_t *rp, int32_t *ci, double *va, cudaStream_
     MPK_CUDA(cudaStreamSynchronize(s));
 }
 
-// Tables of the wave kernel.  A matrix within the cache budget beside four of its vectors is one group
-// (each power is one cell); others keep the plan's groups.  The plan goes without (and runs k_mpk)
-// when a chunk reads rows outside its own group and the two beside it, which the kernel's
-// dependency rule does not cover (levels of another matrix), when there are too many cells, or
-// when the tables do not fit the memory budget.
-static void plan_wave(Plan &P, const std::vector<int32_t> &g_slice, const std::vector<int32_t> &c_slice,
-                      const std::vector<int64_t> &sptr, const std::vector<int2> &hull, const int32_t *slice_row,
-                      bool default_budget, std::vector<int32_t> &host, cudaStream_t s) {
-    const int32_t G = P.num_groups, NS = P.num_slices, pmax = P.p_max;
-    if (P.padded / 32 >= INT32_MAX) return;
-    // groups as runs of the plan's: the kernel's cells pay for a larger budget than k_mpk's, since a
-    // block's share of a cell is what hides the cell's hand-over to the next power
-    const int64_t wave_cache = default_budget ? device_l2_bytes() / 4 * 5 : P.cache_bytes;
-    const int64_t mat = (P.val_bytes + 4) * P.padded, vec = (int64_t)8 * P.n * P.m;
-    const bool one = P.identity || mat + 4 * vec <= P.cache_bytes;
-    std::vector<int32_t> vs(1, 0);  // first slice of every group, and the end
-    const int64_t most = wave_cache / P.window;
-    int64_t bytes = 0;
-    for (int32_t g = 0; g < G && !one; ++g) {
-        const int64_t b = (P.val_bytes + 4) * (sptr[g_slice[g + 1]] - sptr[g_slice[g]]) +
-                          (4 + 16 * (int64_t)P.m) * 32 * (g_slice[g + 1] - g_slice[g]);
-        if (g > 0 && bytes + b > most) {
-            vs.push_back(g_slice[g]);
-            bytes = 0;
-        }
-        bytes += b;
+// ----------------------------------------------------------------------------- wave kernel's tables
+// width of every slice (its longest row) and, if map is given, its rows sorted by length: blocks of
+// kSortSlices slices, longest first, stable, so that the 32 rows of a slice are about equally long
+// (longer blocks pad less but spread a slice's gathers: 2 / 4 / 8 / 32 slices, XXZ L = 24 recurrence 15.1 /
+// 15.0 / 15.4 / 15.6 ms, banded graph of 300k rows 271 / 249 / 240 / 238 us)
+// (slice s holds the rows [slice_row[s], slice_row[s + 1]) of its block's sorted list).  A block never
+// crosses a group: first_slice[b] .. first_slice[b + 1] are its slices.
+constexpr int kSortSlices = 8;
+__global__ void __launch_bounds__(32 * kSortSlices)
+    k_sort_rows(const int32_t *rp, const int32_t *perm, const int32_t *slice_row, const int32_t *block_slice,
+                int32_t *width, int32_t *map) {
+    constexpr int N = 32 * kSortSlices;
+    __shared__ uint32_t key[N];
+    const int s0 = block_slice[blockIdx.x], s1 = block_slice[blockIdx.x + 1];
+    const int r0 = slice_row[s0], rows = slice_row[s1] - r0, t = threadIdx.x;
+    int32_t len = 0;
+    if (t < rows) {
+        const int32_t old = perm ? perm[r0 + t] : r0 + t;
+        len = rp[old + 1] - rp[old];
     }
-    vs.push_back(NS);
-    const int32_t VG = (int32_t)vs.size() - 1;
+    // ascending keys: longest first, then by row; lengths beyond 2^21 count as equal
+    key[t] = t < rows ? (uint32_t)((1 << 21) - min(len, (1 << 21) - 1)) << 10 | (uint32_t)t : 0xffffffffu;
+    for (int size = 2; size <= N; size <<= 1)
+        for (int d = size >> 1; d > 0; d >>= 1) {
+            __syncthreads();
+            const int o = t ^ d;
+            if (o > t) {
+                const uint32_t x = key[t], y = key[o];
+                if ((x > y) == ((t & size) == 0)) {
+                    key[t] = y;
+                    key[o] = x;
+                }
+            }
+        }
+    __syncthreads();
+    const int row = t < rows ? r0 + (int)(key[t] & (N - 1)) : -1;
+    // (slices of a block are full but for the last, so the sorted position is the slice's lane)
+    const int s = s0 + (t >> 5);
+    if (s >= s1) return;
+    map[32 * (int64_t)s + (t & 31)] = row;
+    int32_t w = 0;
+    if (row >= 0) {
+        const int32_t old = perm ? perm[row] : row;
+        w = rp[old + 1] - rp[old];
+    }
+    w = __reduce_max_sync(0xffffffffu, w);
+    if ((t & 31) == 0) width[s] = w;
+}
+
+// width of every slice of consecutive rows, one warp per slice
+__global__ void k_row_width(const int32_t *rp, const int32_t *slice_row, int32_t nslices, int32_t *width) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t s = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; s < nslices;
+         s += (int64_t)gridDim.x * blockDim.x >> 5) {
+        const int32_t r = slice_row[s] + lane;
+        const int32_t w = r < slice_row[s + 1] ? rp[r + 1] - rp[r] : 0;
+        const int32_t m = __reduce_max_sync(0xffffffffu, w);
+        if (lane == 0) width[s] = m;
+    }
+}
+
+__global__ void k_entries_of_width(const int32_t *width, int32_t nslices, int64_t *entries) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < nslices; s += stride)
+        entries[s] = 32 * (int64_t)width[s];
+}
+
+// the sliced copy, padding included, one warp per slice (coalesced writes)
+template <class T>
+__global__ void k_fill_slices(int32_t nslices, const int32_t *rp, const int32_t *ci, const T *va, const int32_t *perm,
+                              const int32_t *iperm, const int32_t *slice_row, const int32_t *map, const int64_t *sptr,
+                              T *sval, int32_t *scol) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t s = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; s < nslices;
+         s += (int64_t)gridDim.x * blockDim.x >> 5) {
+        int32_t row = map ? map[32 * s + lane] : slice_row[s] + lane;
+        if (!map && row >= slice_row[s + 1]) row = -1;
+        int32_t e0 = 0, len = 0;
+        if (row >= 0) {
+            const int32_t old = perm ? perm[row] : row;
+            e0 = rp[old];
+            len = rp[old + 1] - e0;
+        }
+        const int64_t base = sptr[s] + lane;
+        const int32_t w = (int32_t)((sptr[s + 1] - sptr[s]) >> 5);
+        for (int32_t j = 0; j < w; ++j) {
+            const bool on = j < len;
+            const int32_t c = on ? ci[e0 + j] : -1;
+            scol[base + 32 * (int64_t)j] = on && iperm ? iperm[c] : c;
+            sval[base + 32 * (int64_t)j] = on ? va[e0 + j] : T(0);
+        }
+    }
+}
+
+// the slices' records: (first entry / 32, entries a row, first row or row map entry, rows)
+__global__ void k_slice_records(const int64_t *sptr, const int32_t *slice_row, int32_t nslices, int mapped, int4 *rec) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < nslices; s += stride) {
+        const int64_t e0 = sptr[s], e1 = sptr[s + 1];
+        rec[s] = make_int4((int32_t)(e0 >> 5), (int32_t)((e1 - e0) >> 5), mapped ? (int32_t)(32 * s) : slice_row[s],
+                           slice_row[s + 1] - slice_row[s]);
+    }
+}
+
+// Tables of the wave kernel over the slices of `srow` (first rows, and the end), whose groups start
+// at the slices vs: cells, rows of the slices, slices of the groups, counters (zero), in one block of
+// device memory.  False, and nothing done, when there are too many cells or they do not fit the
+// memory budget.
+static bool wave_tables(Plan &P, WaveSet &w, const std::vector<int32_t> &vs, const int64_t *sptr, const int32_t *d_srow,
+                        int32_t NS,
+                        std::vector<int32_t> &host, int64_t extra, cudaStream_t s) {
+    const int32_t VG = (int32_t)vs.size() - 1, pmax = P.p_max;
     const int64_t ncell = (int64_t)VG * pmax * (pmax + 1) / 2;
-    if ((int64_t)VG * pmax >= kWaveMaxCells || ncell > (1 << 22)) return;
-    if (!one) {
-        if ((int32_t)hull.size() != P.num_chunks) return;
-        // (c_slice ascends: chunk c starts at slice c_slice[c])
-        std::vector<int32_t> vc0((size_t)VG + 1);  // first chunk of every group
-        for (int32_t g = 0; g <= VG; ++g)
-            vc0[g] = (int32_t)(std::lower_bound(c_slice.begin(), c_slice.end(), vs[g]) - c_slice.begin());
-        for (int32_t g = 0; g < VG; ++g) {
-            const int32_t lo = vc0[std::max(g - 1, 0)], hi = vc0[std::min(g + 2, VG)];
-            for (int32_t c = vc0[g]; c < vc0[g + 1]; ++c)
-                if (hull[c].x < lo || hull[c].y >= hi) return;
-        }
-    }
-    // one block of device memory: cells, rows of the slices, slices of the groups, counters (zero)
+    if ((int64_t)VG * pmax >= kWaveMaxCells || ncell > (1 << 22)) return false;
     const int64_t ncount = (int64_t)(pmax + 1) * VG;
-    const int64_t words = 4 * ncell + ((int64_t)NS + 1) + VG + ncount;
-    if (P.arena.budget > 0 && P.arena.bytes + 4 * words > P.arena.budget) return;
+    const int64_t words = 4 * ncell + 4 * (int64_t)NS + VG + ncount;
+    if (P.arena.budget > 0 && P.arena.bytes + 4 * words + extra > P.arena.budget) return false;
     host.assign((size_t)(4 * ncell + VG), 0);  // the caller keeps it until the copies are done
     int32_t *vc = host.data(), *gsl = host.data() + 4 * ncell;
     for (int32_t g = 0; g < VG; ++g) gsl[g] = vs[g + 1] - vs[g];
-    P.v_maxsl = *std::max_element(gsl, gsl + VG);
-    P.v_cell_off.assign((size_t)pmax + 2, 0);
+    w.maxsl = *std::max_element(gsl, gsl + VG);
+    w.cell_off.assign((size_t)pmax + 2, 0);
     int32_t c = 0;
     for (int32_t p = 1; p <= pmax; ++p) {  // lines g + kSlotSkew * k ascending, k ascending inside a line
-        P.v_cell_off[p] = c;
+        w.cell_off[p] = c;
         for (int32_t d = kSlotSkew; d <= VG - 1 + kSlotSkew * p; ++d)
             for (int32_t k = 1; k <= p; ++k) {
                 const int32_t g = d - kSlotSkew * k;
@@ -396,23 +469,185 @@ static void plan_wave(Plan &P, const std::vector<int32_t> &g_slice, const std::v
                 ++c;
             }
     }
-    P.v_cell_off[pmax + 1] = c;
-    P.v_ngroups = VG;
+    w.cell_off[pmax + 1] = c;
+    w.ngroups = VG;
     int32_t *dev = P.arena.alloc_n<int32_t>(words);
-    P.v_cell = reinterpret_cast<int4 *>(dev);
-    P.v_gsl = dev + 4 * ncell;
-    P.v_count = P.v_gsl + VG;
-    P.slice_row = P.v_count + ncount;
-    MPK_CUDA(cudaMemcpyAsync(dev, host.data(), sizeof(int32_t) * host.size(), cudaMemcpyHostToDevice, s));
-    MPK_CUDA(cudaMemsetAsync(P.v_count, 0, sizeof(int32_t) * (size_t)ncount, s));
-    MPK_CUDA(cudaMemcpyAsync(P.slice_row, slice_row, sizeof(int32_t) * ((size_t)NS + 1), cudaMemcpyDeviceToDevice, s));
-    P.wave = true;
+    w.cell = reinterpret_cast<int4 *>(dev);
+    w.slice = w.cell + ncell;
+    w.gsl = dev + 4 * (ncell + NS);
+    w.count = w.gsl + VG;
+    MPK_CUDA(cudaMemcpyAsync(w.cell, vc, sizeof(int4) * (size_t)ncell, cudaMemcpyHostToDevice, s));
+    MPK_CUDA(cudaMemcpyAsync(w.gsl, gsl, sizeof(int32_t) * (size_t)VG, cudaMemcpyHostToDevice, s));
+    MPK_CUDA(cudaMemsetAsync(w.count, 0, sizeof(int32_t) * (size_t)ncount, s));
+    k_slice_records<<<grid_n(NS), 256, 0, s>>>(sptr, d_srow, NS, w.rowmap != nullptr, w.slice);
+    MPK_LAUNCHED();
+    return true;
+}
+
+// A sliced copy of its own for the wave kernel: the rows in A's numbering (perm NULL) or in plan
+// order, groups of the rows g_row, sorted by length inside blocks of kSortSlices slices when the
+// padding of unsorted slices is over 4 % of the entries.  False when it does not fit.
+static bool wave_copy(Plan &P, WaveSet &w, const mpk_csr *A, const int32_t *perm, const int32_t *iperm,
+                      const std::vector<int32_t> &g_row, std::vector<int32_t> &host, cudaStream_t s) {
+    const int32_t VG = (int32_t)g_row.size() - 1;
+    std::vector<int32_t> vs(1, 0), srow, blocks;
+    for (int32_t g = 0; g < VG; ++g) {
+        const int32_t s0 = (int32_t)srow.size();
+        for (int32_t r = g_row[g]; r < g_row[g + 1]; r += 32) srow.push_back(r);
+        for (int32_t b = s0; b < (int32_t)srow.size(); b += kSortSlices) blocks.push_back(b);
+        vs.push_back((int32_t)srow.size());
+    }
+    const int32_t NS = (int32_t)srow.size();
+    srow.push_back(g_row[VG]);
+    blocks.push_back(NS);
+    Tmp<int32_t> d_srow((int64_t)NS + 1, s), d_width(NS, s), d_block((int64_t)blocks.size(), s);
+    Tmp<int64_t> d_ent((int64_t)NS + 1, s);
+    MPK_CUDA(cudaMemcpyAsync(d_srow.p, srow.data(), sizeof(int32_t) * srow.size(), cudaMemcpyHostToDevice, s));
+    int32_t *map = nullptr;
+    auto total = [&]() {
+        k_entries_of_width<<<grid_n(NS), 256, 0, s>>>(d_width.p, NS, d_ent.p);
+        MPK_LAUNCHED();
+        exclusive_scan(d_ent.p, d_ent.p, NS, s);
+        int64_t h = 0;
+        MPK_CUDA(cudaMemcpyAsync(&h, d_ent.p + NS, sizeof(h), cudaMemcpyDeviceToHost, s));
+        MPK_CUDA(cudaStreamSynchronize(s));
+        return h;
+    };
+    int64_t entries = 0;
+    if (!perm) {
+        k_row_width<<<grid_n(32 * (int64_t)NS), 256, 0, s>>>(A->row_ptr, d_srow.p, NS, d_width.p);
+        MPK_LAUNCHED();
+        entries = total();
+    }
+    if (perm || entries > A->nnz + A->nnz / 25) {
+        MPK_CUDA(cudaMemcpyAsync(d_block.p, blocks.data(), sizeof(int32_t) * blocks.size(), cudaMemcpyHostToDevice, s));
+        const int64_t bytes = 4 * 32 * (int64_t)NS;
+        if (P.arena.budget > 0 && P.arena.bytes + bytes > P.arena.budget) return false;
+        map = P.arena.alloc_n<int32_t>(32 * (int64_t)NS);
+        k_sort_rows<<<(int)blocks.size() - 1, 32 * kSortSlices, 0, s>>>(A->row_ptr, perm, d_srow.p, d_block.p, d_width.p,
+                                                                       map);
+        MPK_LAUNCHED();
+        entries = total();
+    }
+    if (entries / 32 >= INT32_MAX) return false;
+    const int64_t bytes = (P.val_bytes + 4) * (entries + 32);
+    w.rowmap = map;
+    if (!wave_tables(P, w, vs, d_ent.p, d_srow.p, NS, host, bytes, s)) return false;
+    int32_t *col = static_cast<int32_t *>(P.arena.alloc((entries + 32) * (4 + P.val_bytes)));  // columns, then values
+    void *val = col + (entries + 32);
+#define FILL(T)                                                                                                \
+    k_fill_slices<T><<<grid_n(32 * (int64_t)NS), 256, 0, s>>>(NS, A->row_ptr, A->col, static_cast<const T *>(A->val), \
+                                                              perm, iperm, d_srow.p, map, d_ent.p, static_cast<T *>(val), col)
+    if (P.val_type == MPK_F64)
+        FILL(double);
+    else if (P.val_type == MPK_F32)
+        FILL(float);
+    else
+        FILL(uint16_t);
+#undef FILL
+    MPK_LAUNCHED();
+    w.val = val;
+    w.col = col;
+    w.ok = true;
+    return true;
+}
+
+// Runs make(), which builds a set that the plan can do without: when it returns false, or device
+// memory runs out, what it allocated is freed and the set stays empty.
+template <class F> static bool spare(Plan &P, WaveSet &w, F make) {
+    const size_t mark = P.arena.ptrs.size();
+    bool made = false;
+    try {
+        made = make();
+    } catch (const Fail &f) {
+        if (f.status != MPK_ERR_OOM && f.status != MPK_ERR_BUDGET) throw;
+        cudaGetLastError();
+    }
+    if (!made) {
+        while (P.arena.ptrs.size() > mark) P.arena.free(P.arena.ptrs.back());
+        w = WaveSet();
+    }
+    return made;
+}
+
+// The wave kernel's sets of a plan.
+// Plan order: a matrix within the cache budget beside four of its vectors is one group (each power is
+// one cell); others take runs of the plan's groups.  The plan goes without (and runs k_mpk) when a
+// chunk reads rows outside its own group and the two beside it, which the kernel's dependency rule
+// does not cover (levels of another matrix).  It works on the plan's own sliced copy, or, when that
+// has over 4 % of padding, on one with its rows sorted by length.
+// A's own numbering (plans of original order): no gather before and no scatter after the kernel.
+// Groups are runs of at least `band` rows (the largest |column - row|), so that a row reads its own
+// group and the two beside it.  Taken when the rows of x that a sweep reads around a row fit a
+// quarter of L2: a wider band is better served by the plan's level order.
+static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector<int32_t> &g_row,
+                      const std::vector<int32_t> &g_slice, const std::vector<int32_t> &c_slice,
+                      const std::vector<int64_t> &sptr, const std::vector<int32_t> &s_row, const std::vector<int2> &hull,
+                      const int32_t *d_srow, bool default_budget, std::vector<int32_t> (&host)[2], cudaStream_t s) {
+    const int32_t G = P.num_groups, NS = P.num_slices, n = P.n;
+    if (P.padded / 32 >= INT32_MAX) return;
+    // the kernel's cells pay for a larger budget than k_mpk's, since a block's share of a cell is what
+    // hides the cell's hand-over to the next power (256^3, p = 8: 97 / 130 / 160 / 200 MB took 2.18 /
+    // 2.09 / 2.09 / 2.14 ms)
+    const int64_t wave_cache = default_budget ? device_l2_bytes() / 4 * 5 : P.cache_bytes;
+    const int64_t vec = (int64_t)8 * n * P.m, most = wave_cache / P.window;
+    const int64_t row_bytes = 4 + 16 * (int64_t)P.m;
+    const bool one = P.identity || (P.val_bytes + 4) * P.padded + 4 * vec <= P.cache_bytes;
+    std::vector<int32_t> vs(1, 0);  // first slice of every group, and the end
+    int64_t bytes = 0;
+    for (int32_t g = 0; g < G && !one; ++g) {
+        const int64_t b = (P.val_bytes + 4) * (sptr[g_slice[g + 1]] - sptr[g_slice[g]]) +
+                          row_bytes * (g_row[g + 1] - g_row[g]);
+        if (g > 0 && bytes + b > most) {
+            vs.push_back(g_slice[g]);
+            bytes = 0;
+        }
+        bytes += b;
+    }
+    vs.push_back(NS);
+    const int32_t VG = (int32_t)vs.size() - 1;
+    bool near = one || (int32_t)hull.size() == P.num_chunks;
+    if (!one && near) {  // (chunk c starts at slice c_slice[c], ascending)
+        std::vector<int32_t> vc0((size_t)VG + 1);  // first chunk of every group
+        for (int32_t g = 0; g <= VG; ++g)
+            vc0[g] = (int32_t)(std::lower_bound(c_slice.begin(), c_slice.end(), vs[g]) - c_slice.begin());
+        for (int32_t g = 0; g < VG && near; ++g) {
+            const int32_t lo = vc0[std::max(g - 1, 0)], hi = vc0[std::min(g + 2, VG)];
+            for (int32_t c = vc0[g]; c < vc0[g + 1]; ++c) near = near && hull[c].x >= lo && hull[c].y < hi;
+        }
+    }
+    if (near) {
+        bool own = false;
+        if (P.padded > P.nnz + P.nnz / 25) {
+            std::vector<int32_t> vrow;
+            for (int32_t g = 0; g <= VG; ++g) vrow.push_back(s_row[vs[g]]);
+            own = spare(P, P.wave, [&]() { return wave_copy(P, P.wave, A, P.perm, P.iperm, vrow, host[0], s); });
+        }
+        if (!own && spare(P, P.wave, [&]() { return wave_tables(P, P.wave, vs, P.slice_ptr, d_srow, NS, host[0], 0, s); })) {
+            P.wave.val = P.val;
+            P.wave.col = P.col;
+            P.wave.ok = true;
+        }
+    }
+    if (P.identity || P.order != MPK_ORDER_ORIGINAL) return;
+    if (std::min<int64_t>(n, 2 * (int64_t)band + 32) * 8 * P.m > device_l2_bytes() / 4) return;
+    int64_t rows = n;
+    if (!one) {
+        rows = std::max<int64_t>(band, most / ((P.val_bytes + 4) * (P.nnz / std::max(n, 1) + 1) + row_bytes));
+        rows = std::max<int64_t>(32, (rows + 31) / 32 * 32);
+        if (rows >= n) rows = n;
+    }
+    std::vector<int32_t> nrow;
+    for (int64_t r = 0; r < n; r += rows) nrow.push_back((int32_t)r);
+    nrow.push_back(n);
+    spare(P, P.natural, [&]() { return wave_copy(P, P.natural, A, nullptr, nullptr, nrow, host[1], s); });
 }
 
 Plan *build_plan(const mpk_csr *A, const Levels *L, const mpk_plan_opts *o, cudaStream_t s,
                  const std::vector<int32_t> *inst_row, const std::vector<int32_t> *inst_p) {
     if (!o) fail(MPK_ERR_INVALID, "options are NULL");
-    validate_csr(A, s);
+    int32_t band = 0;
+    validate_csr(A, s, &band);
     if (o->p_max < 1 || o->p_max > kMaxP) fail(MPK_ERR_INVALID, "p_max must be in [1, %d]", kMaxP);
     if (!(o->nrhs == 1 || o->nrhs == 2 || o->nrhs == 4 || o->nrhs == 8 || o->nrhs == 16))
         fail(MPK_ERR_UNSUPPORTED, "nrhs must be 1, 2, 4, 8 or 16 (got %d)", o->nrhs);
@@ -482,13 +717,14 @@ Plan *build_plan(const mpk_csr *A, const Levels *L, const mpk_plan_opts *o, cuda
         }
 
         // ---- permutation (plan-owned copies)
+        // (arrays that live together share a block: a large cudaMalloc and its cudaFree take 100 us)
+        P->rowlen = P->arena.alloc_n<int32_t>((P->identity ? 1 : 3) * (int64_t)std::max(n, 1));
         if (!P->identity && n > 0) {
-            P->perm = P->arena.alloc_n<int32_t>(n);
-            P->iperm = P->arena.alloc_n<int32_t>(n);
+            P->perm = P->rowlen + n;
+            P->iperm = P->perm + n;
             MPK_CUDA(cudaMemcpyAsync(P->perm, L->perm, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s));
             MPK_CUDA(cudaMemcpyAsync(P->iperm, L->iperm, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s));
         }
-        P->rowlen = P->arena.alloc_n<int32_t>(n > 0 ? n : 1);
         if (n > 0) {
             k_rowlen<<<grid_n(n), 256, 0, s>>>(n, A->row_ptr, P->perm, P->rowlen);
             MPK_LAUNCHED();
@@ -668,8 +904,8 @@ Plan *build_plan(const mpk_csr *A, const Levels *L, const mpk_plan_opts *o, cuda
         P->slice_ptr = P->arena.alloc_n<int64_t>((int64_t)NS + 1);
         MPK_CUDA(cudaMemcpyAsync(P->slice_ptr, sptr.data(), sizeof(int64_t) * ((size_t)NS + 1), cudaMemcpyHostToDevice, s));
         Tmp<int32_t> cor(n, s);
-        P->val = P->arena.alloc((P->padded + 32) * P->val_bytes);
-        P->col = P->arena.alloc_n<int32_t>(P->padded + 32);
+        P->col = static_cast<int32_t *>(P->arena.alloc((P->padded + 32) * (4 + P->val_bytes)));  // columns, then values
+        P->val = P->col + (P->padded + 32);
         MPK_CUDA(cudaMemsetAsync(P->val, 0, (size_t)P->val_bytes * (size_t)(P->padded + 32), s));  // +0 in every type
         MPK_CUDA(cudaMemsetAsync(P->col, 0xff, sizeof(int32_t) * (size_t)(P->padded + 32), s));  // padding: col = -1
 
@@ -1091,12 +1327,13 @@ Plan *build_plan(const mpk_csr *A, const Levels *L, const mpk_plan_opts *o, cuda
         P->work_slots = std::max(pmax + 1, 4);  // all powers (original order) or ring of 3 + accumulator
         P->work = P->arena.alloc_n<double>((int64_t)P->work_slots * n * m + 1);
         if (P->accum == MPK_F32) P->shadow = P->arena.alloc_n<float>(2 * (int64_t)n * m + 1);
-        std::vector<int32_t> wave_host;
+        std::vector<int32_t> wave_host[2];
         // ---- wave kernel: single plans of the staged engine, at the planner's block shape or the
         //      unstaged one
         if (o->engine == MPK_ENGINE_STAGED && (o->shape == 0 || o->shape == 3) && !batch && !P->level_capped && !P->split_levels &&
             !o->trace && o->shuffle_seed == 0 && n > 0)
-            plan_wave(*P, g_slice, c_slice, sptr, chunk_hull, d_srow.p, o->cache_bytes == 0, wave_host, s);
+            plan_wave(*P, A, band, g_row, g_slice, c_slice, sptr, s_row, chunk_hull, d_srow.p, o->cache_bytes == 0,
+                      wave_host, s);
         MPK_CUDA(cudaStreamSynchronize(s));  // host vectors above must outlive their copies
     } catch (...) {
         P->arena.release();

@@ -26,8 +26,7 @@ namespace mpk {
 //    neighbouring slices.  The copies need no dependency and run ahead of the cells by the
 //    buffer's size;
 //  - warp 2 (poller) reads the completion counters of the cells that the next 32 cells depend on
-//    (relaxed loads, then one acquire fence for all that became ready) and stores how many
-//    cells may run in s_ready;
+//    and stores how many cells may run in s_ready;
 //  - warp 3 (publisher) sees from the warps' progress words which cells the block has finished,
 //    issues one fence at GPU scope for all of them and adds the block's slices to the cells'
 //    counters;
@@ -71,7 +70,7 @@ template <class VT> struct WaveBuf {
 struct __align__(16) WaveDesc {
     int32_t e32;    // first entry of the slice / 32
     int32_t width;  // entries a row; top bit: first of a run of neighbouring slices
-    int32_t row0;
+    int32_t row0;   // first row, or the slice's first entry of the row map
     uint32_t ckr;   // cell << 11 | power << 6 | rows
 };
 
@@ -180,13 +179,11 @@ __global__ void __launch_bounds__(kWaveBS, 1) k_wave(const KArgs a) {
                 const int gk = __shfl_sync(0xffffffffu, ce.z, qc);
                 WaveDesc d{0, 0, 0, 0};
                 if (t < total) {
-                    const int s = first + (t - (qend - csize));
-                    const int64_t e0 = __ldg(a.slice_ptr + s), e1 = __ldg(a.slice_ptr + s + 1);
-                    const int r0 = __ldg(a.slice_row + s), r1 = __ldg(a.slice_row + s + 1);
-                    d.e32 = (int32_t)(e0 >> 5);
-                    d.width = (int32_t)((e1 - e0) >> 5);
-                    d.row0 = r0;
-                    d.ckr = (uint32_t)(c0 + qc) << 11 | (uint32_t)(gk & 31) << 6 | (uint32_t)(r1 - r0);
+                    const int4 rec = __ldg(a.v_slice + first + (t - (qend - csize)));
+                    d.e32 = rec.x;
+                    d.width = rec.y;
+                    d.row0 = rec.z;
+                    d.ckr = (uint32_t)(c0 + qc) << 11 | (uint32_t)(gk & 31) << 6 | (uint32_t)rec.w;
                 }
                 const int cnt = min(32, total - t0);
                 // where the entries go, and where runs start: at a cell's first slice, after a slice
@@ -301,9 +298,9 @@ __global__ void __launch_bounds__(kWaveBS, 1) k_wave(const KArgs a) {
             if (head && run > 0) {
                 // the launch's last power is the last use of the entries (see k_mpk)
                 const bool last_use = a.stream_last && ((d.ckr >> 6) & 31u) == (uint32_t)a.p_launch;
-                bulk_g2s(sval + o, static_cast<const T *>(a.val) + 32 * (int64_t)d.e32, run * (uint32_t)sizeof(T), &full[b],
+                bulk_g2s(sval + o, static_cast<const T *>(a.v_val) + 32 * (int64_t)d.e32, run * (uint32_t)sizeof(T), &full[b],
                          last_use);
-                bulk_g2s(scol + o, a.col + 32 * (int64_t)d.e32, run * 4u, &full[b], last_use);
+                bulk_g2s(scol + o, a.v_col + 32 * (int64_t)d.e32, run * 4u, &full[b], last_use);
             }
             next += cnt;
             if (lane == b) t_desc = next;
@@ -341,16 +338,17 @@ __global__ void __launch_bounds__(kWaveBS, 1) k_wave(const KArgs a) {
                     if (!ok) {
                         int got[3];
 #pragma unroll
-                        for (int q = 0; q < 3; ++q) got[q] = need[q] > 0 ? ld_relaxed(cnt + g - 1 + q) : 0;
+                        for (int q = 0; q < 3; ++q) got[q] = need[q] > 0 ? (ng == 1 ? ld_acquire(cnt + g - 1 + q) : ld_relaxed(cnt + g - 1 + q)) : 0;
                         ok = got[0] >= need[0] && got[1] >= need[1] && got[2] >= need[2];
                     }
                     const unsigned int m = __ballot_sync(0xffffffffu, ok);
                     const int run = m == 0xffffffffu ? 32 : __ffs(~m) - 1;
                     if (run > known) {
-                        // the counted rows before this block's reads of them (an acquire load of the
-                        // counters instead has to be waited for too, and is no faster then: 256^3,
-                        // p = 8, 2.04 against 2.00 ms)
-                        fence_acq_rel_gpu();
+                        // The counted rows before this block's reads of them.  With one group the loads
+                        // above acquire (a fence after them would add 900 cycles to every power; L1
+                        // holds nothing worth keeping while the block waits); with many they would
+                        // empty L1 at every poll, and one fence serves all that became ready.
+                        if (ng > 1) fence_acq_rel_gpu();
                         __syncwarp();
                         if (lane == 0) st_release_cta_shared(&s_ready, c0 + run);
                         known = run;
@@ -485,14 +483,18 @@ __global__ void __launch_bounds__(kWaveBS, 1) k_wave(const KArgs a) {
             if (q * G < rows) {
                 const double *xin = input_block<M>(a, k);
                 const AT *xacc = InputAcc<M, AT>::get(a, k);
-                const int64_t r0 = d.row0, end = r0 + rows;
+                const int rl = q * G + lane / M;
+                const bool valid = rl < rows;
+                // rows in order, or the row map's (slices of rows sorted by length)
+                const int64_t row = a.v_rowmap ? (valid ? __ldg(a.v_rowmap + d.row0 + rl) : 0) : d.row0 + rl;
                 if (lc >= 0) {
                     const int o = 32 * (lc & 0xffff);
-                    unit_run<M, MODE, AT>(a, k, SVal<VT, AT>{sval + o}, SCol{scol + o}, d.width, r0, q, end, xin, xacc, lane);
+                    unit_row<M, MODE, AT>(a, k, SVal<VT, AT>{sval + o}, SCol{scol + o}, d.width, rl, row, valid, xin, xacc,
+                                          lane);
                 } else {  // a slice wider than the buffer takes: entries from global memory
                     const int64_t e = 32 * (int64_t)d.e32;
-                    unit_run<M, MODE, AT>(a, k, GVal<VT, AT>{static_cast<const T *>(a.val) + e}, GCol{a.col + e}, d.width, r0,
-                                          q, end, xin, xacc, lane);
+                    unit_row<M, MODE, AT>(a, k, GVal<VT, AT>{static_cast<const T *>(a.v_val) + e}, GCol{a.v_col + e}, d.width,
+                                          rl, row, valid, xin, xacc, lane);
                 }
             }
             __syncwarp();

@@ -114,6 +114,7 @@ class Server:
             if idle:
                 plan = idle.pop()
             else:
+                self.backend.room = self.budget - self.used - buf  # a plan may take more than its estimate
                 plan = self.backend.make_plan(key)
                 nbytes = self.backend.actual_plan_bytes(plan, plan_need)
                 self.plan_bytes[id(plan)] = nbytes
@@ -216,13 +217,15 @@ class GpuBackend:
         return int(plan.describe()["device_bytes"])
 
     def make_plan(self, key):
-        from . import MPK_ERR_OOM, ORDER_ORIGINAL, MpkError, plan
+        """A plan within the room the server has left, if it gave one (a plan that has room keeps
+        its matrix in the request's numbering too)."""
+        from . import MPK_ERR_BUDGET, MPK_ERR_OOM, ORDER_ORIGINAL, MpkError, plan
         A = self.mats[key[0]][0]
         try:
             return plan(A, self.levels[key[0]], p_max=self._plan_p(key), nrhs=key[2], order=ORDER_ORIGINAL,
-                        shape=self.shape)
+                        shape=self.shape, mem_budget=max(0, int(getattr(self, "room", 0))))
         except MpkError as e:
-            if e.status != MPK_ERR_OOM:
+            if e.status not in (MPK_ERR_OOM, MPK_ERR_BUDGET):
                 raise
             # freed request buffers may still sit in torch's allocator cache: return them
             self.torch.cuda.synchronize()

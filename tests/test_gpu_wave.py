@@ -83,6 +83,31 @@ def test_many_groups(mpk, cache_bytes, m, val, accum):
            cache_bytes=cache_bytes)
 
 
+@pytest.mark.parametrize("order", [0, 1])
+@pytest.mark.parametrize("m", [1, 2, 8])
+@pytest.mark.parametrize("cache_bytes", [0, 60000])
+def test_sorted_rows_and_own_numbering(mpk, order, m, cache_bytes):
+    """Rows of very different lengths (slices sorted by length), a narrow band, in A's own numbering
+    (original order) and in plan order: powers, the recurrence and host buffers."""
+    A = _widths_matrix(1501, (1, 30, 4, 17, 0, 9, 2), 930)
+    _check(mpk, A, m, 5, order, cache_bytes=cache_bytes)
+    dA = mpk.CsrMatrix.from_host(A)
+    L = mpk.build_levels(dA, 0)
+    P = mpk.plan(dA, L, p_max=5, nrhs=m, order=order, cache_bytes=cache_bytes)
+    X = gen.vector(A.n, m, stream=6)
+    perm = L.perm.cpu().numpy() if order == mpk.ORDER_PLAN else np.arange(A.n)
+    Xin = torch.from_numpy(np.ascontiguousarray(X[perm]))
+    c = np.linspace(1.0, -0.5, 12)
+    out = P.cheb_filter(Xin.cuda(), 11, c, scale=9.0, shift=0.3).cpu().numpy()
+    want = oracle.cheb(A, X, 11, c, scale=9.0, shift=0.3)[perm]
+    assert np.array_equal(out.view(np.uint64), np.ascontiguousarray(want).view(np.uint64))
+    Yh = P.apply_host(Xin.pin_memory(), 5)
+    torch.cuda.synchronize()
+    P.sync_status()
+    want = oracle.mpk(A, X, 5)[:, perm]
+    assert np.array_equal(Yh.numpy().view(np.uint64), np.ascontiguousarray(want).view(np.uint64))
+
+
 @pytest.mark.parametrize("m,p", [(1, 3), (2, 3), (2, 6)])
 def test_hand_over_of_small_cells(mpk, m, p):
     """Cells of a few slices, run many times into poisoned outputs: a block must see every row that

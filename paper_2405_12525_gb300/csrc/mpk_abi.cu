@@ -231,7 +231,8 @@ extern "C" mpk_status mpk_apply(const mpk_plan_t *Ph, const double *X, int32_t p
         return MPK_OK;
     }
     next_epoch(P, s);
-    const bool natural = runs_natural(P);
+    // (X inside Y, but for Y[0] itself, takes the workspace path: it reads X before it writes Y)
+    const bool natural = runs_natural(P) && (X == Y ? !overlap(X, nm, Y + nm, nm * p) : !overlap(X, nm, Y, nm * (p + 1)));
     KArgs a = base_args(P, p);
     a.ring = p + 1;
     if (natural) wave_args(P.natural, p, a);

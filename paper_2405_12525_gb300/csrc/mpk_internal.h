@@ -51,6 +51,12 @@ void set_error(const char *fmt, ...);
 
 inline cudaStream_t as_stream(mpk_stream s) { return reinterpret_cast<cudaStream_t>(s); }
 
+// whether n doubles at a and m at b share memory
+inline bool overlap(const double *a, int64_t n, const double *b, int64_t m) {
+    return reinterpret_cast<uintptr_t>(a) < reinterpret_cast<uintptr_t>(b + m) &&
+           reinterpret_cast<uintptr_t>(b) < reinterpret_cast<uintptr_t>(a + n);
+}
+
 // ----------------------------------------------------------------------------- memory
 // Device allocation with byte accounting against an optional budget.
 struct Arena {
@@ -287,7 +293,7 @@ struct KArgs {
     int32_t ngroups;
     int32_t p_launch;              // powers of this launch (local 1..p_launch)
     // wave kernel (static schedule): its sliced copy, the cells of this launch in line order as
-    // (first slice, slices, g << 5 | k, 0), the rows of every slice, the slices of every group and
+    // (first slice, slices, g << 5 | k, instance << 2 | neighbours: 1 before, 2 after), the rows of every slice, the slices of every group and
     // the finished slices per (power, group), zero when the launch starts
     const void *v_val;
     const int32_t *v_col;
@@ -306,6 +312,19 @@ constexpr int kWaveMaxCells = 1 << 20;  // cells of a wave launch (a descriptor 
 // warp-ticketed engine: slices per item, claim queues (one per warp of a block)
 constexpr int kWarpSlices = 1;
 constexpr int kWarpQueues = 16;
+
+// The vectors of a batch plan's instances, passed by value: X and the powers Y (rows x m blocks) of
+// the rows [row0, row0 + rows) of the batch.
+constexpr int kWaveInst = 64;
+constexpr int kWaveBatchMode = 3;  // kernel mode of such a launch
+struct WaveInst {
+    const double *x;
+    double *y;
+    int64_t row0, rows;
+};
+struct WaveBatch {
+    WaveInst at[kWaveInst];
+};
 
 // Tables of the wave kernel over one sliced copy of the matrix (device memory of the plan)
 struct WaveSet {
@@ -380,6 +399,8 @@ struct Plan {
 };
 
 // kernels (mpk_kernel.cu)
+// the wave kernel on a batch plan (arguments of wave_args)
+void launch_wave_batch(const Plan &P, KArgs &a, WaveBatch &inst, cudaStream_t s);
 void launch_mpk(const Plan &P, KArgs &a, int mode, cudaStream_t s);
 void launch_spmv(const Plan &P, const double *x, double *y, cudaStream_t s);
 // one SpMV on the plan-order rows [lo, hi) only

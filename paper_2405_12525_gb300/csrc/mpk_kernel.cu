@@ -506,8 +506,8 @@ static int occupancy_grid_w(int mode, int m, int vtype) {
 
 // The wave kernel for (mode, width, value type, accumulator), ready to launch, and its shared memory
 static void *select_wave(int mode, int m, int vtype, bool a32, int *smem) {
-    static bool ready[3][3][5][2] = {};  // width index: log2 of m
-    if (vtype < 0 || vtype > 2 || mode < 0 || mode > 2) fail(MPK_ERR_UNSUPPORTED, "value type %d, mode %d", vtype, mode);
+    static bool ready[3][4][5][2] = {};  // width index: log2 of m
+    if (vtype < 0 || vtype > 2 || mode < 0 || mode > kWaveBatchMode) fail(MPK_ERR_UNSUPPORTED, "value type %d, mode %d", vtype, mode);
     void *fn = vtype == MPK_F64 ? select_wave_f64(mode, m, a32, smem)
                                 : (vtype == MPK_F32 ? select_wave_f32(mode, m, a32, smem)
                                                     : select_wave_bf16(mode, m, a32, smem));
@@ -517,6 +517,14 @@ static void *select_wave(int mode, int m, int vtype, bool a32, int *smem) {
         r = true;
     }
     return fn;
+}
+
+void launch_wave_batch(const Plan &P, KArgs &a, WaveBatch &inst, cudaStream_t s) {
+    int smem = 0;
+    void *fn = select_wave(kWaveBatchMode, P.m, P.val_type, false, &smem);
+    const int grid = std::min(device_sms(), a.v_maxsl);
+    void *args[] = {&a, &inst};
+    MPK_CUDA(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kWaveBS), args, (size_t)smem, s));
 }
 
 void launch_mpk(const Plan &P, KArgs &a, int mode, cudaStream_t s) {

@@ -438,46 +438,70 @@ __global__ void k_slice_records(const int64_t *sptr, const int32_t *slice_row, i
     }
 }
 
+// A run of groups whose powers are computed together: a whole plan, or an instance of a batch plan
+struct WaveRange {
+    int32_t g0, g1;  // groups
+    int32_t p;       // powers (batch plans; a single plan has a table for every p)
+    int64_t bytes;   // matrix and vectors
+};
+
 // Tables of the wave kernel over the slices of `srow` (first rows, and the end), whose groups start
-// at the slices vs: cells, rows of the slices, slices of the groups, counters (zero), in one block of
+// at the slices vs: cells, records of the slices, slices of the groups, counters (zero), in one block of
 // device memory.  False, and nothing done, when there are too many cells or they do not fit the
 // memory budget.
-static bool wave_tables(Plan &P, WaveSet &w, const std::vector<int32_t> &vs, const int64_t *sptr, const int32_t *d_srow,
-                        int32_t NS,
-                        std::vector<int32_t> &host, int64_t extra, cudaStream_t s) {
+// A batch plan's instances are taken in bundles that fit L2 together: inside a bundle the lines of all
+// instances alternate, so that one instance's cells fill the hand-over of another's powers.
+static bool wave_tables(Plan &P, WaveSet &w, const std::vector<int32_t> &vs, const std::vector<WaveRange> &ranges,
+                        const int64_t *sptr, const int32_t *d_srow, int32_t NS, std::vector<int32_t> &host, int64_t extra,
+                        cudaStream_t s) {
     const int32_t VG = (int32_t)vs.size() - 1, pmax = P.p_max;
-    const int64_t ncell = (int64_t)VG * pmax * (pmax + 1) / 2;
-    if ((int64_t)VG * pmax >= kWaveMaxCells || ncell > (1 << 22)) return false;
-    const int64_t ncount = (int64_t)(pmax + 1) * VG;
+    const bool batch = !P.inst_p.empty();
+    if ((int64_t)VG * pmax >= kWaveMaxCells || (int64_t)VG * pmax * (pmax + 1) / 2 > (1 << 22)) return false;
+    std::vector<int32_t> vc;  // 4 per cell
+    w.cell_off.assign((size_t)pmax + 2, 0);
+    for (int32_t p = batch ? pmax : 1; p <= pmax; ++p) {
+        w.cell_off[p] = (int32_t)(vc.size() / 4);
+        for (size_t i = 0; i < ranges.size();) {
+            size_t e = i;
+            int64_t bytes = 0;
+            int32_t dmax = 0;
+            for (; e < ranges.size() && (e == i || bytes + ranges[e].bytes <= device_l2_bytes() / 4 * 3); ++e) {
+                bytes += ranges[e].bytes;
+                dmax = std::max(dmax, ranges[e].g1 - ranges[e].g0 - 1 + kSlotSkew * (batch ? ranges[e].p : p));
+            }
+            for (int32_t d = kSlotSkew; d <= dmax; ++d)  // lines g + kSlotSkew * k ascending
+                for (size_t r = i; r < e; ++r) {
+                    const WaveRange &R = ranges[r];
+                    for (int32_t k = 1; k <= (batch ? R.p : p); ++k) {  // k ascending inside a line
+                        const int32_t g = R.g0 + d - kSlotSkew * k;
+                        if (g < R.g0 || g >= R.g1) continue;
+                        vc.push_back(vs[g]);
+                        vc.push_back(vs[g + 1] - vs[g]);
+                        vc.push_back((g << 5) | k);
+                        vc.push_back((int32_t)r << 2 | (g > R.g0 ? 1 : 0) | (g + 1 < R.g1 ? 2 : 0));
+                    }
+                }
+            i = e;
+        }
+    }
+    const int64_t ncell = (int64_t)vc.size() / 4, ncount = (int64_t)(pmax + 1) * VG;
+    w.cell_off[pmax + 1] = (int32_t)ncell;
     const int64_t words = 4 * ncell + 4 * (int64_t)NS + VG + ncount;
     if (P.arena.budget > 0 && P.arena.bytes + 4 * words + extra > P.arena.budget) return false;
-    host.assign((size_t)(4 * ncell + VG), 0);  // the caller keeps it until the copies are done
-    int32_t *vc = host.data(), *gsl = host.data() + 4 * ncell;
-    for (int32_t g = 0; g < VG; ++g) gsl[g] = vs[g + 1] - vs[g];
-    w.maxsl = *std::max_element(gsl, gsl + VG);
-    w.cell_off.assign((size_t)pmax + 2, 0);
-    int32_t c = 0;
-    for (int32_t p = 1; p <= pmax; ++p) {  // lines g + kSlotSkew * k ascending, k ascending inside a line
-        w.cell_off[p] = c;
-        for (int32_t d = kSlotSkew; d <= VG - 1 + kSlotSkew * p; ++d)
-            for (int32_t k = 1; k <= p; ++k) {
-                const int32_t g = d - kSlotSkew * k;
-                if (g < 0 || g >= VG) continue;
-                vc[4 * (int64_t)c] = vs[g];
-                vc[4 * (int64_t)c + 1] = gsl[g];
-                vc[4 * (int64_t)c + 2] = (g << 5) | k;
-                ++c;
-            }
+    w.maxsl = 0;
+    for (int32_t g = 0; g < VG; ++g) {
+        vc.push_back(vs[g + 1] - vs[g]);
+        w.maxsl = std::max(w.maxsl, vs[g + 1] - vs[g]);
     }
-    w.cell_off[pmax + 1] = c;
+    host.swap(vc);  // the caller keeps it until the copies are done
     w.ngroups = VG;
     int32_t *dev = P.arena.alloc_n<int32_t>(words);
     w.cell = reinterpret_cast<int4 *>(dev);
     w.slice = w.cell + ncell;
     w.gsl = dev + 4 * (ncell + NS);
     w.count = w.gsl + VG;
-    MPK_CUDA(cudaMemcpyAsync(w.cell, vc, sizeof(int4) * (size_t)ncell, cudaMemcpyHostToDevice, s));
-    MPK_CUDA(cudaMemcpyAsync(w.gsl, gsl, sizeof(int32_t) * (size_t)VG, cudaMemcpyHostToDevice, s));
+    MPK_CUDA(cudaMemcpyAsync(w.cell, host.data(), sizeof(int4) * (size_t)ncell, cudaMemcpyHostToDevice, s));
+    MPK_CUDA(cudaMemcpyAsync(w.gsl, host.data() + 4 * ncell, sizeof(int32_t) * (size_t)VG, cudaMemcpyHostToDevice, s));
     MPK_CUDA(cudaMemsetAsync(w.count, 0, sizeof(int32_t) * (size_t)ncount, s));
     k_slice_records<<<grid_n(NS), 256, 0, s>>>(sptr, d_srow, NS, w.rowmap != nullptr, w.slice);
     MPK_LAUNCHED();
@@ -488,7 +512,8 @@ static bool wave_tables(Plan &P, WaveSet &w, const std::vector<int32_t> &vs, con
 // order, groups of the rows g_row, sorted by length inside blocks of kSortSlices slices when the
 // padding of unsorted slices is over 4 % of the entries.  False when it does not fit.
 static bool wave_copy(Plan &P, WaveSet &w, const mpk_csr *A, const int32_t *perm, const int32_t *iperm,
-                      const std::vector<int32_t> &g_row, std::vector<int32_t> &host, cudaStream_t s) {
+                      const std::vector<int32_t> &g_row, const std::vector<WaveRange> &ranges,
+                      std::vector<int32_t> &host, cudaStream_t s) {
     const int32_t VG = (int32_t)g_row.size() - 1;
     std::vector<int32_t> vs(1, 0), srow, blocks;
     for (int32_t g = 0; g < VG; ++g) {
@@ -532,7 +557,7 @@ static bool wave_copy(Plan &P, WaveSet &w, const mpk_csr *A, const int32_t *perm
     if (entries / 32 >= INT32_MAX) return false;
     const int64_t bytes = (P.val_bytes + 4) * (entries + 32);
     w.rowmap = map;
-    if (!wave_tables(P, w, vs, d_ent.p, d_srow.p, NS, host, bytes, s)) return false;
+    if (!wave_tables(P, w, vs, ranges, d_ent.p, d_srow.p, NS, host, bytes, s)) return false;
     int32_t *col = static_cast<int32_t *>(P.arena.alloc((entries + 32) * (4 + P.val_bytes)));  // columns, then values
     void *val = col + (entries + 32);
 #define FILL(T)                                                                                                \
@@ -590,19 +615,49 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
     // hides the cell's hand-over to the next power (256^3, p = 8: 97 / 130 / 160 / 200 MB took 2.18 /
     // 2.09 / 2.09 / 2.14 ms)
     const int64_t wave_cache = default_budget ? device_l2_bytes() / 4 * 5 : P.cache_bytes;
-    const int64_t vec = (int64_t)8 * n * P.m, most = wave_cache / P.window;
-    const int64_t row_bytes = 4 + 16 * (int64_t)P.m;
-    const bool one = P.identity || (P.val_bytes + 4) * P.padded + 4 * vec <= P.cache_bytes;
-    std::vector<int32_t> vs(1, 0);  // first slice of every group, and the end
-    int64_t bytes = 0;
-    for (int32_t g = 0; g < G && !one; ++g) {
-        const int64_t b = (P.val_bytes + 4) * (sptr[g_slice[g + 1]] - sptr[g_slice[g]]) +
-                          row_bytes * (g_row[g + 1] - g_row[g]);
-        if (g > 0 && bytes + b > most) {
-            vs.push_back(g_slice[g]);
-            bytes = 0;
+    const bool batch = !P.inst_p.empty();
+    const int64_t row_bytes = 4 + 16 * (int64_t)P.m, vec_bytes = 32 * (int64_t)P.m;
+    // the instances: rows, plan groups, the budget of a group, and whether one group holds it all
+    struct Inst {
+        int32_t r0, r1, g0, g1, p;
+        int64_t most, bytes;
+        bool one;
+    };
+    std::vector<Inst> in;
+    const size_t ni = batch ? P.inst_p.size() : 1;
+    if (ni > kWaveInst) return;
+    bool one = true;  // every instance is one group
+    for (size_t i = 0; i < ni; ++i) {
+        Inst t;
+        t.r0 = batch ? P.inst_row[i] : 0;
+        t.r1 = batch ? P.inst_row[i + 1] : n;
+        t.p = batch ? P.inst_p[i] : P.p_max;
+        t.g0 = (int32_t)(std::lower_bound(g_row.begin(), g_row.end() - 1, t.r0) - g_row.begin());
+        t.g1 = t.r1 == n ? G : (int32_t)(std::lower_bound(g_row.begin(), g_row.end() - 1, t.r1) - g_row.begin());
+        if (t.r1 == t.r0) t.g1 = t.g0;
+        const int64_t entries = sptr[g_slice[t.g1]] - sptr[g_slice[t.g0]];
+        t.bytes = (P.val_bytes + 4) * entries + vec_bytes * (t.r1 - t.r0);
+        t.one = P.identity || t.bytes <= P.cache_bytes;
+        t.most = wave_cache / (kSlotSkew * t.p + 1);
+        one = one && t.one;
+        in.push_back(t);
+    }
+    std::vector<int32_t> vs;  // first slice of every group, and the end
+    std::vector<WaveRange> ranges;
+    for (const Inst &t : in) {
+        WaveRange r{(int32_t)vs.size(), 0, t.p, t.bytes};
+        int64_t bytes = 0;
+        for (int32_t g = t.g0; g < t.g1; ++g) {
+            const int64_t b = (P.val_bytes + 4) * (sptr[g_slice[g + 1]] - sptr[g_slice[g]]) +
+                              row_bytes * (g_row[g + 1] - g_row[g]);
+            if (g == t.g0 || (!t.one && bytes + b > t.most)) {
+                vs.push_back(g_slice[g]);
+                bytes = 0;
+            }
+            bytes += b;
         }
-        bytes += b;
+        r.g1 = (int32_t)vs.size();
+        ranges.push_back(r);  // (an empty instance has no groups)
     }
     vs.push_back(NS);
     const int32_t VG = (int32_t)vs.size() - 1;
@@ -621,9 +676,10 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
         if (P.padded > P.nnz + P.nnz / 25) {
             std::vector<int32_t> vrow;
             for (int32_t g = 0; g <= VG; ++g) vrow.push_back(s_row[vs[g]]);
-            own = spare(P, P.wave, [&]() { return wave_copy(P, P.wave, A, P.perm, P.iperm, vrow, host[0], s); });
+            own = spare(P, P.wave, [&]() { return wave_copy(P, P.wave, A, P.perm, P.iperm, vrow, ranges, host[0], s); });
         }
-        if (!own && spare(P, P.wave, [&]() { return wave_tables(P, P.wave, vs, P.slice_ptr, d_srow, NS, host[0], 0, s); })) {
+        if (!own && spare(P, P.wave, [&]() { return wave_tables(P, P.wave, vs, ranges, P.slice_ptr, d_srow, NS, host[0], 0, s);
+                        })) {
             P.wave.val = P.val;
             P.wave.col = P.col;
             P.wave.ok = true;
@@ -631,16 +687,21 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
     }
     if (P.identity || P.order != MPK_ORDER_ORIGINAL) return;
     if (std::min<int64_t>(n, 2 * (int64_t)band + 32) * 8 * P.m > device_l2_bytes() / 4) return;
-    int64_t rows = n;
-    if (!one) {
-        rows = std::max<int64_t>(band, most / ((P.val_bytes + 4) * (P.nnz / std::max(n, 1) + 1) + row_bytes));
-        rows = std::max<int64_t>(32, (rows + 31) / 32 * 32);
-        if (rows >= n) rows = n;
-    }
     std::vector<int32_t> nrow;
-    for (int64_t r = 0; r < n; r += rows) nrow.push_back((int32_t)r);
+    ranges.clear();
+    for (const Inst &t : in) {
+        WaveRange r{(int32_t)nrow.size(), 0, t.p, t.bytes};
+        int64_t rows = t.r1 - t.r0;
+        if (!t.one) {
+            rows = std::max<int64_t>(band, t.most / ((P.val_bytes + 4) * (P.nnz / std::max(n, 1) + 1) + row_bytes));
+            rows = std::max<int64_t>(32, (rows + 31) / 32 * 32);
+        }
+        for (int64_t q = t.r0; q < t.r1; q += rows) nrow.push_back((int32_t)q);
+        r.g1 = (int32_t)nrow.size();
+        ranges.push_back(r);
+    }
     nrow.push_back(n);
-    spare(P, P.natural, [&]() { return wave_copy(P, P.natural, A, nullptr, nullptr, nrow, host[1], s); });
+    spare(P, P.natural, [&]() { return wave_copy(P, P.natural, A, nullptr, nullptr, nrow, ranges, host[1], s); });
 }
 
 Plan *build_plan(const mpk_csr *A, const Levels *L, const mpk_plan_opts *o, cudaStream_t s,
@@ -1330,7 +1391,7 @@ Plan *build_plan(const mpk_csr *A, const Levels *L, const mpk_plan_opts *o, cuda
         std::vector<int32_t> wave_host[2];
         // ---- wave kernel: single plans of the staged engine, at the planner's block shape or the
         //      unstaged one
-        if (o->engine == MPK_ENGINE_STAGED && (o->shape == 0 || o->shape == 3) && !batch && !P->level_capped && !P->split_levels &&
+        if (o->engine == MPK_ENGINE_STAGED && (o->shape == 0 || o->shape == 3) && !P->level_capped && !P->split_levels &&
             !o->trace && o->shuffle_seed == 0 && n > 0)
             plan_wave(*P, A, band, g_row, g_slice, c_slice, sptr, s_row, chunk_hull, d_srow.p, o->cache_bytes == 0,
                       wave_host, s);

@@ -101,8 +101,10 @@ __device__ __forceinline__ int2 wave_share(int nsl, int block, int blocks) {
     return make_int2((int)((int64_t)nsl * block / blocks), (int)((int64_t)nsl * (block + 1) / blocks));
 }
 
-template <int M, int MODE, class VT, bool A32>
-__global__ void __launch_bounds__(kWaveBS, 1) k_wave(const KArgs a) {
+// The body of the kernel.  BATCH (powers of a batch plan): the vectors of the instances lie apart, at
+// the places in `inst`.
+template <int M, int MODE, class VT, bool A32, bool BATCH>
+__device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst) {
     using AT = typename std::conditional<A32, float, double>::type;
     using T = typename VT::T;
     constexpr int G = 32 / M;  // rows of a unit
@@ -111,6 +113,7 @@ __global__ void __launch_bounds__(kWaveBS, 1) k_wave(const KArgs a) {
     T *const sval = reinterpret_cast<T *>(smem);
     int32_t *const scol = reinterpret_cast<int32_t *>(smem + Buf::ALL * sizeof(T));
     __shared__ WaveDesc desc[kDescRing];
+    __shared__ uint8_t dinst[BATCH ? kDescRing : 1];  // instance of each descriptor
     __shared__ uint32_t vpos[kDescRing];  // entries of the buffer's slices before this one, all in all
     __shared__ int loc[kDescRing];  // where a slice's entries are: offset / 32, tile << 16, phase << 24; -1: global memory
     __shared__ __align__(8) uint64_t full[kWaveTiles];
@@ -135,7 +138,7 @@ __global__ void __launch_bounds__(kWaveBS, 1) k_wave(const KArgs a) {
     }
     __syncthreads();
     const int32_t epoch = s_epoch;
-    const int4 *cells = a.v_cell;  // (first slice, slices, g << 5 | k, unused)
+    const int4 *cells = a.v_cell;  // (first slice, slices, g << 5 | k, instance << 2 | neighbours: 1 before, 2 after)
     const int ncells = a.v_ncells;
 
     auto give_up = [&]() {  // a wait expired: tell this block and the others
@@ -177,6 +180,7 @@ __global__ void __launch_bounds__(kWaveBS, 1) k_wave(const KArgs a) {
                 const int csize = __shfl_sync(0xffffffffu, sh.y - sh.x, qc);
                 const int qend = __shfl_sync(0xffffffffu, end, qc);
                 const int gk = __shfl_sync(0xffffffffu, ce.z, qc);
+                const int ci = BATCH ? __shfl_sync(0xffffffffu, ce.w, qc) >> 2 : 0;
                 WaveDesc d{0, 0, 0, 0};
                 if (t < total) {
                     const int4 rec = __ldg(a.v_slice + first + (t - (qend - csize)));
@@ -220,6 +224,7 @@ __global__ void __launch_bounds__(kWaveBS, 1) k_wave(const KArgs a) {
                 }
                 if (lane < cnt) {
                     desc[(pushed + lane) & (kDescRing - 1)] = d;
+                    if constexpr (BATCH) dinst[(pushed + lane) & (kDescRing - 1)] = (uint8_t)ci;
                     vpos[(pushed + lane) & (kDescRing - 1)] = vp;
                 }
                 pushed += cnt;
@@ -321,15 +326,15 @@ __global__ void __launch_bounds__(kWaveBS, 1) k_wave(const KArgs a) {
             const int ng = a.v_ngroups;
             bool stop = false;
             for (int c0 = 0; c0 < ncells && !stop; c0 += 32) {
-                const int gk = c0 + lane < ncells ? __ldg(cells + c0 + lane).z : 0;
-                const int k = gk & 31, g = gk >> 5;
+                const int4 ce = c0 + lane < ncells ? __ldg(cells + c0 + lane) : make_int4(0, 0, 0, 0);
+                const int k = ce.z & 31, g = ce.z >> 5;
                 const int32_t *cnt = a.v_count + (int64_t)(k - 1) * ng;
                 int need[3];
                 bool ok = k <= 1;
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
-                    const int h = g - 1 + q;
-                    need[q] = (!ok && h >= 0 && h < ng) ? __ldg(a.v_gsl + h) : 0;
+                    // the group itself, and its neighbours inside the instance
+                    need[q] = !ok && (q == 1 || (ce.w & (q == 0 ? 1 : 2))) ? __ldg(a.v_gsl + g - 1 + q) : 0;
                 }
                 int known = 0;  // leading cells of the 32 already announced
                 Deadline w0;
@@ -481,17 +486,38 @@ __global__ void __launch_bounds__(kWaveBS, 1) k_wave(const KArgs a) {
                 }
             }
             if (q * G < rows) {
-                const double *xin = input_block<M>(a, k);
-                const AT *xacc = InputAcc<M, AT>::get(a, k);
                 const int rl = q * G + lane / M;
                 const bool valid = rl < rows;
                 // rows in order, or the row map's (slices of rows sorted by length)
                 const int64_t row = a.v_rowmap ? (valid ? __ldg(a.v_rowmap + d.row0 + rl) : 0) : d.row0 + rl;
-                if (lc >= 0) {
+                if constexpr (BATCH) {
+                    // the instance's vectors, addressed by rows of the whole batch
+                    const WaveInst in = inst->at[dinst[idx & (kDescRing - 1)]];
+                    const int64_t at = row * M + lane % M;
+                    double *const y = in.y + (k * in.rows - in.row0) * M;
+                    const double *const x = (k == 1 ? in.x - in.row0 * M : y - in.rows * M) + lane % M;
+                    double own = 0.0;
+                    const bool copy = k == 1 && in.y != in.x && valid;
+                    if (copy) own = in.x[at - in.row0 * M];
+                    double acc;
+                    if (lc >= 0) {
+                        const int o = 32 * (lc & 0xffff) + rl;
+                        acc = unit_sum<M, double>(SVal<VT>{sval + o}, SCol{scol + o}, d.width, x);
+                    } else {
+                        const int64_t e = 32 * (int64_t)d.e32 + rl;
+                        acc = unit_sum<M, double>(GVal<VT>{static_cast<const T *>(a.v_val) + e}, GCol{a.v_col + e}, d.width, x);
+                    }
+                    if (valid) y[at] = acc;
+                    if (copy) in.y[at - in.row0 * M] = own;
+                } else if (lc >= 0) {
+                    const double *xin = input_block<M>(a, k);
+                    const AT *xacc = InputAcc<M, AT>::get(a, k);
                     const int o = 32 * (lc & 0xffff);
                     unit_row<M, MODE, AT>(a, k, SVal<VT, AT>{sval + o}, SCol{scol + o}, d.width, rl, row, valid, xin, xacc,
                                           lane);
                 } else {  // a slice wider than the buffer takes: entries from global memory
+                    const double *xin = input_block<M>(a, k);
+                    const AT *xacc = InputAcc<M, AT>::get(a, k);
                     const int64_t e = 32 * (int64_t)d.e32;
                     unit_row<M, MODE, AT>(a, k, GVal<VT, AT>{static_cast<const T *>(a.v_val) + e}, GCol{a.v_col + e}, d.width,
                                           rl, row, valid, xin, xacc, lane);
@@ -504,7 +530,18 @@ __global__ void __launch_bounds__(kWaveBS, 1) k_wave(const KArgs a) {
     }
 }
 
+template <int M, int MODE, class VT, bool A32>
+__global__ void __launch_bounds__(kWaveBS, 1) k_wave(const __grid_constant__ KArgs a) {
+    wave_body<M, MODE, VT, A32, false>(a, nullptr);
+}
+template <int M, class VT>
+__global__ void __launch_bounds__(kWaveBS, 1) k_wave_batch(const __grid_constant__ KArgs a,
+                                                           const __grid_constant__ WaveBatch inst) {
+    wave_body<M, MODE_POWERS, VT, false, true>(a, &inst);
+}
+
 template <class VT, int M> static void *wave_fn(int mode, bool a32) {
+    if (mode == kWaveBatchMode) return (void *)k_wave_batch<M, VT>;
     if constexpr (!std::is_same<VT, ValF64>::value)
         if (a32) {
             if (mode == MODE_HOST) {

@@ -125,3 +125,40 @@ def test_hand_over_of_small_cells(mpk, m, p):
         Y.fill_(float("nan"))
         P.apply(Xd, p, Y=Y)
         assert torch.equal(Y, want)
+
+
+@pytest.mark.parametrize("order", [0, 1])
+@pytest.mark.parametrize("m", [1, 4])
+@pytest.mark.parametrize("cache_bytes", [0, 30000])
+def test_batch_instances(mpk, order, m, cache_bytes):
+    """Uneven instances with their own powers, an empty one, outputs apart, in the workspace, and an X
+    inside another instance's output."""
+    mats = [gen.laplacian_3d(9, 8, 7), gen.laplacian_2d(40, 31), gen.CSR([0], [], np.zeros(0)), gen.laplacian_1d(5),
+            _widths_matrix(900, (1, 30, 4, 17, 0), 940), gen.laplacian_3d(15, 14, 13)]
+    ps = [5, 2, 3, 7, 4, 6]
+    dAs = [mpk.CsrMatrix.from_host(A) for A in mats]
+    B = mpk.batch_plan(dAs, ps, nrhs=m, order=order, cache_bytes=cache_bytes)
+    Xh = [gen.vector(A.n, m, stream=20 + i) if A.n else np.zeros((0, m)) for i, A in enumerate(mats)]
+    perms = [mpk.build_levels(d, 0).perm.cpu().numpy() if A.n else np.zeros(0, int) for d, A in zip(dAs, mats)]
+    want = [oracle.mpk(A, X, p) if A.n else np.zeros((p + 1, 0, m)) for A, X, p in zip(mats, Xh, ps)]
+    if order == mpk.ORDER_PLAN:
+        Xin, out = [X[q] for X, q in zip(Xh, perms)], [w[:, q] for w, q in zip(want, perms)]
+    else:
+        Xin, out = Xh, want
+    Xs = [torch.from_numpy(np.ascontiguousarray(X)).cuda() for X in Xin]
+
+    def same(Ys, ref):
+        for Y, w in zip(Ys, ref):
+            assert np.array_equal(Y.cpu().numpy().view(np.uint64), np.ascontiguousarray(w).view(np.uint64))
+
+    Ys = [torch.full(w.shape, float("nan"), dtype=torch.float64, device="cuda") for w in out]
+    for _ in range(3):
+        B.apply(Xs, Ys)
+        same(Ys, out)
+    same(B.apply(Xs, in_place=True), [w[:, q] for w, q in zip(want, perms)])
+    # instance 0's X lies inside instance 5's output
+    flat = Ys[5].reshape(-1)
+    inside = flat[100:100 + Xs[0].numel()].view(Xs[0].shape)
+    inside.copy_(Xs[0])
+    B.apply([inside] + Xs[1:], Ys)
+    same(Ys, out)

@@ -152,6 +152,7 @@ void mpk::wave_args(const WaveSet &w, int32_t p, KArgs &a) {
     a.v_col = w.col;
     a.v_slice = w.slice;
     a.v_rowmap = w.rowmap;
+    a.v_dict = w.dict;
     a.v_cell = w.cell + w.cell_off[p];
     a.v_ncells = w.cell_off[p + 1] - w.cell_off[p];
     a.v_gsl = w.gsl;

@@ -298,6 +298,7 @@ struct KArgs {
     const void *v_val;
     const int32_t *v_col;
     const int4 *v_slice;       // slices: (first entry / 32, entries a row, first row or row map entry, rows)
+    const double *v_dict;      // packed copies: the table of values (v_val is the slices' stream)
     const int32_t *v_rowmap;   // row of every lane of every slice (-1: none), or null: consecutive rows
     const int4 *v_cell;
     const int32_t *v_gsl;
@@ -308,6 +309,13 @@ struct KArgs {
     // stay there between launches)
     int32_t stream_last;
 };
+// A packed slice of w entries a row: w smallest columns (int32, padded to 16 bytes), 32 w column
+// distances (16 bits; 32-bit columns if they do not fit: `wide`), 32 w value numbers (8 bits); in units
+// of 16 bytes
+inline __host__ __device__ int32_t packed_units(int32_t w, bool wide) { return (w + 3) / 4 + (wide ? 10 : 6) * w; }
+constexpr int32_t kWideSlice = 1 << 30;  // in the width of a packed slice's record
+constexpr int kNoCol = 0xffff;  // the distance that stands for no entry; real ones lie below
+constexpr int kDictSize = 256;
 constexpr int kWaveMaxCells = 1 << 20;  // cells of a wave launch (a descriptor holds 21 bits)
 // warp-ticketed engine: slices per item, claim queues (one per warp of a block)
 constexpr int kWarpSlices = 1;
@@ -331,6 +339,7 @@ struct WaveSet {
     bool ok = false;
     const void *val = nullptr;
     const int32_t *col = nullptr;
+    const double *dict = nullptr;     // packed copy: its table of values (val is the stream)
     const int32_t *rowmap = nullptr;  // rows of the slices' lanes when they are sorted by length
     int32_t ngroups = 0, maxsl = 0;
     int4 *cell = nullptr;             // cells of every p, concatenated

@@ -505,13 +505,14 @@ static int occupancy_grid_w(int mode, int m, int vtype) {
 }
 
 // The wave kernel for (mode, width, value type, accumulator), ready to launch, and its shared memory
-static void *select_wave(int mode, int m, int vtype, bool a32, int *smem) {
-    static bool ready[3][4][5][2] = {};  // width index: log2 of m
+static void *select_wave(int mode, int m, int vtype, bool packed, bool a32, int *smem) {
+    static bool ready[4][4][5][2] = {};  // packed copies: value type 3; width index: log2 of m
     if (vtype < 0 || vtype > 2 || mode < 0 || mode > kWaveBatchMode) fail(MPK_ERR_UNSUPPORTED, "value type %d, mode %d", vtype, mode);
-    void *fn = vtype == MPK_F64 ? select_wave_f64(mode, m, a32, smem)
-                                : (vtype == MPK_F32 ? select_wave_f32(mode, m, a32, smem)
-                                                    : select_wave_bf16(mode, m, a32, smem));
-    bool &r = ready[vtype][mode][__builtin_ctz((unsigned)m)][a32 ? 1 : 0];
+    void *fn = packed             ? select_wave_dict(mode, m, a32, smem)
+               : vtype == MPK_F64 ? select_wave_f64(mode, m, a32, smem)
+               : vtype == MPK_F32 ? select_wave_f32(mode, m, a32, smem)
+                                  : select_wave_bf16(mode, m, a32, smem);
+    bool &r = ready[packed ? 3 : vtype][mode][__builtin_ctz((unsigned)m)][a32 ? 1 : 0];
     if (!r) {
         MPK_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, *smem));
         r = true;
@@ -521,7 +522,7 @@ static void *select_wave(int mode, int m, int vtype, bool a32, int *smem) {
 
 void launch_wave_batch(const Plan &P, KArgs &a, WaveBatch &inst, cudaStream_t s) {
     int smem = 0;
-    void *fn = select_wave(kWaveBatchMode, P.m, P.val_type, false, &smem);
+    void *fn = select_wave(kWaveBatchMode, P.m, P.val_type, false, false, &smem);
     const int grid = std::min(device_sms(), a.v_maxsl);
     void *args[] = {&a, &inst};
     MPK_CUDA(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kWaveBS), args, (size_t)smem, s));
@@ -532,7 +533,7 @@ void launch_mpk(const Plan &P, KArgs &a, int mode, cudaStream_t s) {
     if (a.v_cell != nullptr && a.drop_unit < 0) {
         const int grid = std::min(device_sms(), a.v_maxsl);
         int smem = 0;
-        void *fn = select_wave(mode, P.m, P.val_type, a32, &smem);
+        void *fn = select_wave(mode, P.m, P.val_type, a.v_dict != nullptr, a32, &smem);
         void *args[] = {&a};
         MPK_CUDA(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kWaveBS), args, (size_t)smem, s));
         return;

@@ -219,14 +219,20 @@ template <class VT> struct ToAcc<VT, float> {
 template <class VT, class AT = double> struct GVal {
     const typename VT::T *p;
     __device__ __forceinline__ AT operator[](int64_t i) const { return ToAcc<VT, AT>::get(__ldg(p + i)); }
+    __device__ __forceinline__ void lane(int l) { p += l; }        // to lane row l
+    __device__ __forceinline__ void skip(int n) { p += 32 * n; }  // past n entries of the row
 };
 template <class VT, class AT = double> struct SVal {
     const typename VT::T *p;
     __device__ __forceinline__ AT operator[](int64_t i) const { return ToAcc<VT, AT>::get(p[i]); }
+    __device__ __forceinline__ void lane(int l) { p += l; }
+    __device__ __forceinline__ void skip(int n) { p += 32 * n; }
 };
 struct GCol {
     const int32_t *p;
     __device__ __forceinline__ int32_t operator[](int64_t i) const { return __ldg(p + i); }
+    __device__ __forceinline__ void lane(int l) { p += l; }
+    __device__ __forceinline__ void skip(int n) { p += 32 * n; }
 };
 
 __device__ __forceinline__ int hi_bits(double v) { return __double2hiint(v); }
@@ -367,6 +373,31 @@ constexpr int kBatch = 8;  // entries of a row whose x values are gathered toget
 struct SCol {
     const int32_t *p;
     __device__ __forceinline__ int32_t operator[](int64_t i) const { return p[i]; }
+    __device__ __forceinline__ void lane(int l) { p += l; }
+    __device__ __forceinline__ void skip(int n) { p += 32 * n; }
+};
+
+// Packed slices (matrices of at most 256 different values): values as 8-bit numbers of a table, columns
+// as 16-bit distances from the smallest column among the slice's rows at the same entry
+template <class AT> struct DictVal {
+    const uint8_t *p;
+    const AT *table;
+    __device__ __forceinline__ AT operator[](int64_t i) const { return table[p[i]]; }
+    __device__ __forceinline__ void lane(int l) { p += l; }
+    __device__ __forceinline__ void skip(int n) { p += 32 * n; }
+};
+struct NearCol {
+    const uint16_t *p;
+    const int32_t *first;  // smallest column of every entry
+    __device__ __forceinline__ int32_t operator[](int64_t i) const {
+        const int d = p[i];
+        return d == kNoCol ? -1 : first[i >> 5] + d;
+    }
+    __device__ __forceinline__ void lane(int l) { p += l; }
+    __device__ __forceinline__ void skip(int n) {
+        p += 32 * n;
+        first += n;
+    }
 };
 
 // Epilogue of one (row, column) of step j at local power k: w is its row sum.  own / back: its
@@ -428,8 +459,8 @@ template <int M, class AT, class VP, class CP>
 __device__ __forceinline__ AT unit_sum(VP sv, CP sc, int width, const AT *x, AT acc = AT(0)) {
     for (; width >= kBatch; width -= kBatch) {
         unit_batch<kBatch, M, AT>(sv, sc, x, acc);
-        sc.p += 32 * kBatch;
-        sv.p += 32 * kBatch;
+        sc.skip(kBatch);
+        sv.skip(kBatch);
     }
     switch (width) {
         case 1: unit_batch<1, M, AT>(sv, sc, x, acc); break;
@@ -469,8 +500,8 @@ __device__ __forceinline__ void unit_row(const KArgs &a, int k, VP sv, CP sc, in
     const int64_t at = row * M + cl;
     double own = 0.0, back = 0.0, old = 0.0;
     unit_rows<MODE>(a, k, at, valid, xin, own, back, old);  // on their way during the sums
-    sv.p += rl;
-    sc.p += rl;
+    sv.lane(rl);
+    sc.lane(rl);
     const AT acc = unit_sum<M, AT>(sv, sc, width, xacc + cl);
     unit_epilogue<M, MODE, AT>(a, k, at, valid, lane, acc, own, back, old);
 }

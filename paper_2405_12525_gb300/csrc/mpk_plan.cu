@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <memory>
 
 namespace mpk {
 
@@ -384,12 +385,17 @@ __global__ void __launch_bounds__(32 * kSortSlices)
 }
 
 // width of every slice of consecutive rows, one warp per slice
-__global__ void k_row_width(const int32_t *rp, const int32_t *slice_row, int32_t nslices, int32_t *width) {
+__global__ void k_row_width(const int32_t *rp, const int32_t *perm, const int32_t *slice_row, int32_t nslices,
+                            int32_t *width) {
     const int lane = threadIdx.x & 31;
     for (int64_t s = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; s < nslices;
          s += (int64_t)gridDim.x * blockDim.x >> 5) {
         const int32_t r = slice_row[s] + lane;
-        const int32_t w = r < slice_row[s + 1] ? rp[r + 1] - rp[r] : 0;
+        int32_t w = 0;
+        if (r < slice_row[s + 1]) {
+            const int32_t old = perm ? perm[r] : r;
+            w = rp[old + 1] - rp[old];
+        }
         const int32_t m = __reduce_max_sync(0xffffffffu, w);
         if (lane == 0) width[s] = m;
     }
@@ -428,13 +434,153 @@ __global__ void k_fill_slices(int32_t nslices, const int32_t *rp, const int32_t 
     }
 }
 
-// the slices' records: (first entry / 32, entries a row, first row or row map entry, rows)
-__global__ void k_slice_records(const int64_t *sptr, const int32_t *slice_row, int32_t nslices, int mapped, int4 *rec) {
+// the slices' records: (first entry / 32, entries a row, first row or row map entry, rows); packed
+// copies (width given): (first unit, width and flag, ...)
+__global__ void k_slice_records(const int64_t *sptr, const int32_t *width, const int32_t *slice_row, int32_t nslices,
+                                int mapped, int4 *rec) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < nslices; s += stride) {
         const int64_t e0 = sptr[s], e1 = sptr[s + 1];
-        rec[s] = make_int4((int32_t)(e0 >> 5), (int32_t)((e1 - e0) >> 5), mapped ? (int32_t)(32 * s) : slice_row[s],
-                           slice_row[s + 1] - slice_row[s]);
+        rec[s] = make_int4(width ? (int32_t)e0 : (int32_t)(e0 >> 5), width ? width[s] : (int32_t)((e1 - e0) >> 5),
+                           mapped ? (int32_t)(32 * s) : slice_row[s], slice_row[s + 1] - slice_row[s]);
+    }
+}
+
+// Different values of a matrix, as bit patterns in an open hash table; given up beyond kDictSize.
+constexpr int kDictSlots = 4 * kDictSize;
+constexpr unsigned long long kNoValue = 0x7ff8a5c3e1f00d01ULL;  // (a NaN; a matrix holding it is given up)
+struct Dict {
+    unsigned long long key[kDictSlots];
+    int32_t index[kDictSlots];  // number of the slot's value
+    double value[kDictSize];
+    int32_t count, over;
+};
+__device__ __forceinline__ unsigned long long value_bits(double v) { return (unsigned long long)__double_as_longlong(v); }
+__device__ __forceinline__ unsigned long long value_bits(float v) { return __float_as_uint(v); }
+__device__ __forceinline__ unsigned long long value_bits(uint16_t v) { return v; }
+__device__ __forceinline__ int dict_slot(unsigned long long b) { return (int)((b * 0x9e3779b97f4a7c15ULL) >> 54) & (kDictSlots - 1); }
+__global__ void k_dict_init(Dict *d) {
+    for (int i = threadIdx.x; i < kDictSlots; i += blockDim.x) d->key[i] = kNoValue;
+    for (int i = threadIdx.x; i < kDictSize; i += blockDim.x) d->value[i] = 0.0;
+    if (threadIdx.x == 0) d->count = d->over = 0;
+}
+template <class T> __global__ void k_dict(int64_t nnz, const T *va, Dict *d) {
+    __shared__ unsigned long long seen[kDictSlots];  // the block's own table: most entries end here
+    for (int i = threadIdx.x; i < kDictSlots; i += blockDim.x) seen[i] = kNoValue;
+    __syncthreads();
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    unsigned long long last = kNoValue;
+    int step = 0;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nnz; e += stride) {
+        const unsigned long long b = value_bits(va[e]);
+        if ((step++ & 15) == 0 && *(volatile int32_t *)&d->over) return;
+        if (b == kNoValue) d->over = 1;
+        if (b == last) continue;
+        last = b;
+        bool known = false;
+        for (int s = dict_slot(b), i = 0; i < kDictSlots; ++i, s = (s + 1) & (kDictSlots - 1)) {
+            unsigned long long k = *(volatile unsigned long long *)&seen[s];
+            if (k == kNoValue) k = atomicCAS(&seen[s], kNoValue, b);
+            known = k == b;
+            if (known || k == kNoValue) break;
+        }
+        if (known) continue;
+        for (int s = dict_slot(b), i = 0; i < kDictSlots; ++i, s = (s + 1) & (kDictSlots - 1)) {
+            if (*(volatile int32_t *)&d->over) return;
+            const unsigned long long k = atomicCAS(&d->key[s], kNoValue, b);
+            if (k == kNoValue && atomicAdd(&d->count, 1) >= kDictSize) d->over = 1;
+            if (k == b || k == kNoValue) break;
+        }
+    }
+}
+// numbers the values found (one block); vt: their stored type
+__global__ void k_dict_number(Dict *d, int vt) {
+    __shared__ int n;
+    if (threadIdx.x == 0) n = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < kDictSlots; i += blockDim.x) {
+        const unsigned long long b = d->key[i];
+        if (b == kNoValue) continue;
+        const int q = atomicAdd(&n, 1);
+        if (q >= kDictSize) continue;  // given up
+        d->index[i] = q;
+        d->value[q] = vt == MPK_F64   ? __longlong_as_double((long long)b)
+                      : vt == MPK_F32 ? widen_value(__uint_as_float((uint32_t)b))
+                                      : widen_value((uint16_t)b);
+    }
+}
+
+// One warp per slice: the row of every lane, as k_fill_slices; f(j, entry of the row or -1) for every
+// entry a row of the slice
+template <class F>
+__device__ __forceinline__ void slice_entries(int64_t s, int w, const int32_t *rp, const int32_t *perm, const int32_t *slice_row,
+                                              const int32_t *map, int lane, F f) {
+    int32_t row = map ? map[32 * s + lane] : slice_row[s] + lane;
+    if (!map && row >= slice_row[s + 1]) row = -1;
+    int32_t e0 = 0, len = 0;
+    if (row >= 0) {
+        const int32_t old = perm ? perm[row] : row;
+        e0 = rp[old];
+        len = rp[old + 1] - e0;
+    }
+    for (int j = 0; j < w; ++j) f(j, j < len ? e0 + j : -1);
+}
+// packed slices: marks in `width` those whose columns do not fit 16-bit distances, sizes in units
+__global__ void k_pack_size(int32_t nslices, const int32_t *rp, const int32_t *ci, const int32_t *perm, const int32_t *iperm,
+                            const int32_t *slice_row, const int32_t *map, int32_t *width, int64_t *units) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t s = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; s < nslices;
+         s += (int64_t)gridDim.x * blockDim.x >> 5) {
+        const int w = width[s];
+        bool wide = false;
+        slice_entries(s, w, rp, perm, slice_row, map, lane, [&](int, int32_t e) {
+            const int32_t c = e < 0 ? -1 : (iperm ? iperm[ci[e]] : ci[e]);
+            const int32_t hi = __reduce_max_sync(0xffffffffu, c);
+            const int32_t lo = __reduce_min_sync(0xffffffffu, c < 0 ? INT_MAX : c);
+            wide = wide || hi - lo >= kNoCol;  // (an entry that no lane has: -1 - INT_MAX)
+        });
+        __syncwarp();
+        if (lane == 0) {
+            width[s] = w | (wide ? kWideSlice : 0);
+            units[s] = packed_units(w, wide);
+        }
+    }
+}
+template <class T>
+__global__ void k_pack_fill(int32_t nslices, const int32_t *rp, const int32_t *ci, const T *va, const int32_t *perm,
+                            const int32_t *iperm, const int32_t *slice_row, const int32_t *map, const int32_t *width,
+                            const int64_t *units, const Dict *d, uint8_t *stream) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long last = kNoValue;
+    int last_q = 0;
+    for (int64_t s = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; s < nslices;
+         s += (int64_t)gridDim.x * blockDim.x >> 5) {
+        const int w = width[s] & (kWideSlice - 1);
+        const bool wide = (width[s] & kWideSlice) != 0;
+        uint8_t *p = stream + 16 * units[s];
+        int32_t *first = reinterpret_cast<int32_t *>(p);
+        uint8_t *cols = p + 16 * ((w + 3) / 4), *vals = cols + (wide ? 128 : 64) * (int64_t)w;
+        slice_entries(s, w, rp, perm, slice_row, map, lane, [&](int j, int32_t e) {
+            const int32_t c = e < 0 ? -1 : (iperm ? iperm[ci[e]] : ci[e]);
+            const int32_t lo = __reduce_min_sync(0xffffffffu, c < 0 ? INT_MAX : c);
+            if (lane == 0) first[j] = lo;
+            if (wide)
+                reinterpret_cast<int32_t *>(cols)[32 * j + lane] = c;
+            else
+                reinterpret_cast<uint16_t *>(cols)[32 * j + lane] = (uint16_t)(c < 0 ? kNoCol : c - lo);
+            int q = 0;
+            if (e >= 0) {
+                const unsigned long long b = value_bits(va[e]);
+                if (b != last) {
+                    int t = dict_slot(b);
+                    for (int i = 0; i < kDictSlots && d->key[t] != b; ++i) t = (t + 1) & (kDictSlots - 1);
+                    last = b;
+                    last_q = d->index[t];
+                }
+                q = last_q;
+            }
+            vals[32 * (int64_t)j + lane] = (uint8_t)q;
+        });
     }
 }
 
@@ -452,7 +598,8 @@ struct WaveRange {
 // A batch plan's instances are taken in bundles that fit L2 together: inside a bundle the lines of all
 // instances alternate, so that one instance's cells fill the hand-over of another's powers.
 static bool wave_tables(Plan &P, WaveSet &w, const std::vector<int32_t> &vs, const std::vector<WaveRange> &ranges,
-                        const int64_t *sptr, const int32_t *d_srow, int32_t NS, std::vector<int32_t> &host, int64_t extra,
+                        const int64_t *sptr, const int32_t *d_width, const int32_t *d_srow, int32_t NS,
+                        std::vector<int32_t> &host, int64_t extra,
                         cudaStream_t s) {
     const int32_t VG = (int32_t)vs.size() - 1, pmax = P.p_max;
     const bool batch = !P.inst_p.empty();
@@ -503,16 +650,38 @@ static bool wave_tables(Plan &P, WaveSet &w, const std::vector<int32_t> &vs, con
     MPK_CUDA(cudaMemcpyAsync(w.cell, host.data(), sizeof(int4) * (size_t)ncell, cudaMemcpyHostToDevice, s));
     MPK_CUDA(cudaMemcpyAsync(w.gsl, host.data() + 4 * ncell, sizeof(int32_t) * (size_t)VG, cudaMemcpyHostToDevice, s));
     MPK_CUDA(cudaMemsetAsync(w.count, 0, sizeof(int32_t) * (size_t)ncount, s));
-    k_slice_records<<<grid_n(NS), 256, 0, s>>>(sptr, d_srow, NS, w.rowmap != nullptr, w.slice);
+    k_slice_records<<<grid_n(NS), 256, 0, s>>>(sptr, d_width, d_srow, NS, w.rowmap != nullptr, w.slice);
     MPK_LAUNCHED();
     return true;
 }
 
+// The table of A's values (256^3: 0.2 ms; a matrix of random values is given up after a few
+// entries); false if there are more than kDictSize.
+static bool find_values(const Plan &P, const mpk_csr *A, Dict *d, cudaStream_t s) {
+    k_dict_init<<<1, 1024, 0, s>>>(d);
+    MPK_LAUNCHED();
+    if (P.val_type == MPK_F64)
+        k_dict<<<grid_n(A->nnz), 256, 0, s>>>(A->nnz, static_cast<const double *>(A->val), d);
+    else if (P.val_type == MPK_F32)
+        k_dict<<<grid_n(A->nnz), 256, 0, s>>>(A->nnz, static_cast<const float *>(A->val), d);
+    else
+        k_dict<<<grid_n(A->nnz), 256, 0, s>>>(A->nnz, static_cast<const uint16_t *>(A->val), d);
+    MPK_LAUNCHED();
+    k_dict_number<<<1, 1024, 0, s>>>(d, P.val_type);
+    MPK_LAUNCHED();
+    int32_t found[2];  // number, given up
+    MPK_CUDA(cudaMemcpyAsync(found, &d->count, sizeof(found), cudaMemcpyDeviceToHost, s));
+    MPK_CUDA(cudaStreamSynchronize(s));
+    return !found[1] && found[0] <= kDictSize;
+}
+
 // A sliced copy of its own for the wave kernel: the rows in A's numbering (perm NULL) or in plan
 // order, groups of the rows g_row, sorted by length inside blocks of kSortSlices slices when the
-// padding of unsorted slices is over 4 % of the entries.  False when it does not fit.
+// padding of unsorted slices is over 4 % of the entries (sorted anyway, 256^3, p = 8, plan order,
+// packed: 1850 -> 2134 us: rows that were neighbours no longer share their loads and stores of
+// vectors).  With the table of A's values (dict) the slices are packed.  False when it does not fit.
 static bool wave_copy(Plan &P, WaveSet &w, const mpk_csr *A, const int32_t *perm, const int32_t *iperm,
-                      const std::vector<int32_t> &g_row, const std::vector<WaveRange> &ranges,
+                      const std::vector<int32_t> &g_row, const std::vector<WaveRange> &ranges, const Dict *dict,
                       std::vector<int32_t> &host, cudaStream_t s) {
     const int32_t VG = (int32_t)g_row.size() - 1;
     std::vector<int32_t> vs(1, 0), srow, blocks;
@@ -538,13 +707,10 @@ static bool wave_copy(Plan &P, WaveSet &w, const mpk_csr *A, const int32_t *perm
         MPK_CUDA(cudaStreamSynchronize(s));
         return h;
     };
-    int64_t entries = 0;
-    if (!perm) {
-        k_row_width<<<grid_n(32 * (int64_t)NS), 256, 0, s>>>(A->row_ptr, d_srow.p, NS, d_width.p);
-        MPK_LAUNCHED();
-        entries = total();
-    }
-    if (perm || entries > A->nnz + A->nnz / 25) {
+    k_row_width<<<grid_n(32 * (int64_t)NS), 256, 0, s>>>(A->row_ptr, perm, d_srow.p, NS, d_width.p);
+    MPK_LAUNCHED();
+    int64_t entries = total();
+    if (entries > A->nnz + A->nnz / 25) {
         MPK_CUDA(cudaMemcpyAsync(d_block.p, blocks.data(), sizeof(int32_t) * blocks.size(), cudaMemcpyHostToDevice, s));
         const int64_t bytes = 4 * 32 * (int64_t)NS;
         if (P.arena.budget > 0 && P.arena.bytes + bytes > P.arena.budget) return false;
@@ -555,9 +721,39 @@ static bool wave_copy(Plan &P, WaveSet &w, const mpk_csr *A, const int32_t *perm
         entries = total();
     }
     if (entries / 32 >= INT32_MAX) return false;
-    const int64_t bytes = (P.val_bytes + 4) * (entries + 32);
     w.rowmap = map;
-    if (!wave_tables(P, w, vs, ranges, d_ent.p, d_srow.p, NS, host, bytes, s)) return false;
+    if (dict) {
+        k_pack_size<<<grid_n(32 * (int64_t)NS), 256, 0, s>>>(NS, A->row_ptr, A->col, perm, iperm, d_srow.p, map, d_width.p,
+                                                             d_ent.p);
+        MPK_LAUNCHED();
+        exclusive_scan(d_ent.p, d_ent.p, NS, s);
+        int64_t units = 0;
+        MPK_CUDA(cudaMemcpyAsync(&units, d_ent.p + NS, sizeof(units), cudaMemcpyDeviceToHost, s));
+        MPK_CUDA(cudaStreamSynchronize(s));
+        if (units >= INT32_MAX) return false;
+        const int64_t bytes = 16 * units + (int64_t)sizeof(dict->value);
+        if (!wave_tables(P, w, vs, ranges, d_ent.p, d_width.p, d_srow.p, NS, host, bytes, s)) return false;
+        uint8_t *dev = static_cast<uint8_t *>(P.arena.alloc(bytes));  // the table, then the stream
+        uint8_t *stream = dev + sizeof(dict->value);
+        MPK_CUDA(cudaMemcpyAsync(dev, dict->value, sizeof(dict->value), cudaMemcpyDeviceToDevice, s));
+#define PACK(T)                                                                                                  \
+    k_pack_fill<T><<<grid_n(32 * (int64_t)NS), 256, 0, s>>>(NS, A->row_ptr, A->col, static_cast<const T *>(A->val), perm, \
+                                                            iperm, d_srow.p, map, d_width.p, d_ent.p, dict, stream)
+        if (P.val_type == MPK_F64)
+            PACK(double);
+        else if (P.val_type == MPK_F32)
+            PACK(float);
+        else
+            PACK(uint16_t);
+#undef PACK
+        MPK_LAUNCHED();
+        w.val = stream;
+        w.dict = reinterpret_cast<const double *>(dev);
+        w.ok = true;
+        return true;
+    }
+    const int64_t bytes = (P.val_bytes + 4) * (entries + 32);
+    if (!wave_tables(P, w, vs, ranges, d_ent.p, nullptr, d_srow.p, NS, host, bytes, s)) return false;
     int32_t *col = static_cast<int32_t *>(P.arena.alloc((entries + 32) * (4 + P.val_bytes)));  // columns, then values
     void *val = col + (entries + 32);
 #define FILL(T)                                                                                                \
@@ -642,13 +838,40 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
         one = one && t.one;
         in.push_back(t);
     }
+    // A matrix larger than the cache that has few different values gets packed copies (about 3.2 bytes an
+    // entry in place of 12): the copies into shared memory, not HBM, are what they save, so they also help
+    // at p = 1.  Measured, us, plain -> packed copies, 256^3 7-point / 150^3 27-point, p = 8:
+    //   binary64, A's order:              2215 -> 1966 / 1907 -> 1348;  plan order: 2035 -> 1850 / 1912 -> 1306
+    //   binary32, plan order:             1807 -> 1852 / 1477 -> 1306
+    //   bfloat16, binary32 sums, A's order: 1470 -> 1524 / 825 -> 715
+    //   bfloat16, binary64 sums, A's order: 1974 -> 1968 / 1300 -> 1348
+    // and more columns (bfloat16 27-point 100^3, 8 columns: 3054 -> 3277) use an entry too often for
+    // its unpacking.
+    const bool long_rows = P.nnz / std::max(n, 1) >= 16;
+    const bool pack = !batch && !one && P.m == 1 &&
+                      (P.val_type == MPK_F64 || (long_rows && (P.val_type == MPK_F32 || P.accum == MPK_F32)));
+    const bool natural = !P.identity && P.order == MPK_ORDER_ORIGINAL &&
+                         std::min<int64_t>(n, 2 * (int64_t)band + 32) * 8 * P.m <= device_l2_bytes() / 4;
+    std::unique_ptr<Tmp<Dict>> table;
+    bool packed = false;
+    if (pack) try {
+            table.reset(new Tmp<Dict>(1, s));
+            packed = find_values(P, A, table->p, s);
+        } catch (const Fail &f) {  // no memory for the table
+            if (f.status != MPK_ERR_OOM) throw;
+            cudaGetLastError();
+        }
+    const Dict *dict = packed ? table->p : nullptr;
+    const Dict *plan_dict = natural ? nullptr : dict;
+    const double packed_entry = 3.2, entry_bytes = packed ? packed_entry : P.val_bytes + 4;
+    const double plan_entry = plan_dict ? packed_entry : P.val_bytes + 4;
     std::vector<int32_t> vs;  // first slice of every group, and the end
     std::vector<WaveRange> ranges;
     for (const Inst &t : in) {
         WaveRange r{(int32_t)vs.size(), 0, t.p, t.bytes};
         int64_t bytes = 0;
         for (int32_t g = t.g0; g < t.g1; ++g) {
-            const int64_t b = (P.val_bytes + 4) * (sptr[g_slice[g + 1]] - sptr[g_slice[g]]) +
+            const int64_t b = (int64_t)(plan_entry * (double)(sptr[g_slice[g + 1]] - sptr[g_slice[g]])) +
                               row_bytes * (g_row[g + 1] - g_row[g]);
             if (g == t.g0 || (!t.one && bytes + b > t.most)) {
                 vs.push_back(g_slice[g]);
@@ -673,35 +896,41 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
     }
     if (near) {
         bool own = false;
-        if (P.padded > P.nnz + P.nnz / 25) {
+        if (plan_dict || P.padded > P.nnz + P.nnz / 25) {
             std::vector<int32_t> vrow;
             for (int32_t g = 0; g <= VG; ++g) vrow.push_back(s_row[vs[g]]);
-            own = spare(P, P.wave, [&]() { return wave_copy(P, P.wave, A, P.perm, P.iperm, vrow, ranges, host[0], s); });
+            own = spare(P, P.wave, [&]() {
+                return wave_copy(P, P.wave, A, P.perm, P.iperm, vrow, ranges, plan_dict, host[0], s);
+            });
         }
-        if (!own && spare(P, P.wave, [&]() { return wave_tables(P, P.wave, vs, ranges, P.slice_ptr, d_srow, NS, host[0], 0, s);
-                        })) {
+        if (!own && spare(P, P.wave, [&]() {
+                return wave_tables(P, P.wave, vs, ranges, P.slice_ptr, nullptr, d_srow, NS, host[0], 0, s);
+            })) {
             P.wave.val = P.val;
             P.wave.col = P.col;
             P.wave.ok = true;
         }
     }
-    if (P.identity || P.order != MPK_ORDER_ORIGINAL) return;
-    if (std::min<int64_t>(n, 2 * (int64_t)band + 32) * 8 * P.m > device_l2_bytes() / 4) return;
+    if (!natural) return;
     std::vector<int32_t> nrow;
     ranges.clear();
     for (const Inst &t : in) {
         WaveRange r{(int32_t)nrow.size(), 0, t.p, t.bytes};
         int64_t rows = t.r1 - t.r0;
         if (!t.one) {
-            rows = std::max<int64_t>(band, t.most / ((P.val_bytes + 4) * (P.nnz / std::max(n, 1) + 1) + row_bytes));
-            rows = std::max<int64_t>(32, (rows + 31) / 32 * 32);
+            rows = std::max<int64_t>(band, (int64_t)((double)t.most / (entry_bytes * (double)(P.nnz / std::max(n, 1) + 1) +
+                                                                       (double)row_bytes)));
+            // equal shares for the blocks where a group has a few slices for each (27-point stencil on
+            // 150^3, p = 8, packed: 1349 -> 1261 us; below, a whole slice more for each would be too much)
+            const int64_t even = 32 * (int64_t)device_sms();
+            rows = rows >= 2 * even ? (rows + even - 1) / even * even : std::max<int64_t>(32, (rows + 31) / 32 * 32);
         }
         for (int64_t q = t.r0; q < t.r1; q += rows) nrow.push_back((int32_t)q);
         r.g1 = (int32_t)nrow.size();
         ranges.push_back(r);
     }
     nrow.push_back(n);
-    spare(P, P.natural, [&]() { return wave_copy(P, P.natural, A, nullptr, nullptr, nrow, ranges, host[1], s); });
+    spare(P, P.natural, [&]() { return wave_copy(P, P.natural, A, nullptr, nullptr, nrow, ranges, dict, host[1], s); });
 }
 
 Plan *build_plan(const mpk_csr *A, const Levels *L, const mpk_plan_opts *o, cudaStream_t s,

@@ -1,5 +1,6 @@
 // The wave kernel: level-blocked powers on a static schedule (device code; instantiated per
-// value type in mpk_wave_f64.cu, mpk_wave_f32.cu and mpk_wave_bf16.cu).
+// value type in mpk_wave_f64.cu, mpk_wave_f32.cu and mpk_wave_bf16.cu, for packed copies in
+// mpk_wave_dict.cu).
 #pragma once
 #include "mpk_kernel_dev.cuh"
 
@@ -9,9 +10,19 @@ namespace mpk {
 // all SMs), so 256^3, p = 8 needs 1.58 ms of it; k_mpk's units (claimed through a ticket, handed
 // over block-wide, 8 FMA slots for a row of 7 entries) took 2.08 ms.  Here nothing is claimed and
 // nothing handed over block-wide, a row takes exactly its slice's width of FMAs, and 28 warps
-// work on as many slices: 1.99 ms; binary32 sums, bound by instruction issue and the latency of the
-// gathers: 1.45 -> 1.33 ms.  Blocks of right-hand sides, where k_mpk's gathers of one column at a
-// time made L1 the bound: 100^3 27-point stencil, 8 columns, p = 8: 4.21 -> 3.42 ms.
+// work on as many slices: 2.03 ms, and 1.84 ms with packed copies (below); binary32 sums, bound by
+// instruction issue and the latency of the gathers: 1.45 -> 1.37 ms.  Blocks of right-hand sides,
+// where k_mpk's gathers of one column at a time made L1 the bound: 100^3 27-point stencil, 8
+// columns, p = 8: 4.21 -> 2.90 ms.  What is left above the FMAs is the cells' hand-over (blocks
+// that wait for the slowest one) and slices that wait for their copies.
+//
+// Packed copies (VT = ValDict; matrices of at most 256 different values, one right-hand side): a
+// slice is one stream of 16-byte units, per entry the smallest column among the 32 rows, then 32
+// column distances of 16 bits (32-bit columns in a slice where they do not fit), then 32 value
+// numbers of 8 bits, whose values lie in a table in shared memory.  About 3.2 bytes an entry in
+// place of 12, so the buffer holds three times the slices, the copies run further ahead, and a cell
+// of the same bytes has more rows; the FMAs and their operands are the same.  27-point stencil
+// on 150^3, p = 8: 1.91 -> 1.31 ms.
 //
 // One cooperative launch, one block per SM.  The Lp-diagram cells (group g, power k) are walked
 // in line order, as k_mpk does; every cell's 32-row slices are divided evenly over the blocks,
@@ -55,21 +66,35 @@ constexpr int kWaveWarps = 28;  // compute warps: 16 / 20 / 24 / 28 took 2.34 / 
 constexpr int kWaveBS = 32 * (kWaveWarps + kWaveAux);
 constexpr int kDescRing = 512;  // slice descriptors in shared memory
 constexpr int kWaveTiles = 32;  // tiles in shared memory or in flight
+constexpr int kStagedWidth = 64;  // entries a row of the widest slice that the buffer takes
 // Entries of the circular buffer, of the widest slice it takes (a wider one is read from global
 // memory) and of a tile.  A slice that starts near the end of the buffer runs on past it, into
 // room for one slice.
 template <class VT> struct WaveBuf {
     static constexpr int ENTRY = (int)sizeof(typename VT::T) + 4;
-    static constexpr int SLICE = 32 * 64;
+    static constexpr int SLICE = 32 * kStagedWidth;
     static constexpr int CAP = (200 * 1024 / ENTRY - SLICE) / 256 * 256;
     static constexpr int TILE = CAP / 3;
     static constexpr int ALL = CAP + SLICE + 32 * kBatch;  // a batch may read past its slice
     static_assert(TILE >= SLICE, "a slice fits a tile");
 };
 
+// packed slices: positions and sizes count 16-byte units
+struct ValDict {
+    using T = uint8_t;
+};
+template <> struct WaveBuf<ValDict> {
+    static constexpr int ENTRY = 16;
+    static constexpr int SLICE = (kStagedWidth + 3) / 4 + 10 * kStagedWidth;
+    static constexpr int CAP = (200 * 1024 / ENTRY - SLICE) / 16 * 16;
+    static constexpr int TILE = CAP / 3;
+    static constexpr int ALL = CAP + SLICE;
+    static_assert(TILE >= SLICE, "a slice fits a tile");
+};
+
 struct __align__(16) WaveDesc {
-    int32_t e32;    // first entry of the slice / 32
-    int32_t width;  // entries a row; top bit: first of a run of neighbouring slices
+    int32_t e32;    // first entry of the slice / 32 (packed: its place in the stream, units)
+    int32_t width;  // entries a row; top bit: first of a run of neighbouring slices; packed: next bit: wide
     int32_t row0;   // first row, or the slice's first entry of the row map
     uint32_t ckr;   // cell << 11 | power << 6 | rows
 };
@@ -107,11 +132,18 @@ template <int M, int MODE, class VT, bool A32, bool BATCH>
 __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst) {
     using AT = typename std::conditional<A32, float, double>::type;
     using T = typename VT::T;
+    constexpr bool PACK = std::is_same<VT, ValDict>::value;
+    // a slice's entries a row and its size in the buffer, from the width field of its record
+    auto width_of = [](int f) { return PACK ? f & (kWideSlice - 1) : f & 0x7fffffff; };
+    auto size_of = [&](int f) { return PACK ? packed_units(width_of(f), (f & kWideSlice) != 0) : 32 * width_of(f); };
     constexpr int G = 32 / M;  // rows of a unit
     using Buf = WaveBuf<VT>;
     extern __shared__ __align__(128) unsigned char smem[];  // values, then columns
     T *const sval = reinterpret_cast<T *>(smem);
-    int32_t *const scol = reinterpret_cast<int32_t *>(smem + Buf::ALL * sizeof(T));
+    int32_t *const scol = reinterpret_cast<int32_t *>(smem + Buf::ALL * sizeof(T));  // (packed: unused)
+    __shared__ AT s_dict[PACK ? kDictSize : 1];
+    if constexpr (PACK)
+        for (int i = threadIdx.x; i < kDictSize; i += kWaveBS) s_dict[i] = (AT)a.v_dict[i];  // exact
     __shared__ WaveDesc desc[kDescRing];
     __shared__ uint8_t dinst[BATCH ? kDescRing : 1];  // instance of each descriptor
     __shared__ uint32_t vpos[kDescRing];  // entries of the buffer's slices before this one, all in all
@@ -192,7 +224,7 @@ __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst)
                 const int cnt = min(32, total - t0);
                 // where the entries go, and where runs start: at a cell's first slice, after a slice
                 // that is not copied, and where the buffer starts over
-                const int size = d.width <= Buf::SLICE / 32 ? 32 * d.width : 0;
+                const int size = width_of(d.width) <= kStagedWidth ? size_of(d.width) : 0;
                 uint32_t vp = (uint32_t)size;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -267,9 +299,8 @@ __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst)
                 d = desc[(next + lane) & (kDescRing - 1)];
                 vp = vpos[(next + lane) & (kDescRing - 1)];
             }
-            const int width = d.width & 0x7fffffff;
-            const bool staged = width <= Buf::SLICE / 32;
-            const uint32_t ve = vp + (staged ? 32u * (uint32_t)width : 0u);
+            const bool staged = width_of(d.width) <= kStagedWidth;
+            const uint32_t ve = vp + (staged ? (uint32_t)size_of(d.width) : 0u);
             const uint32_t v0 = __shfl_sync(0xffffffffu, vp, 0);
             const unsigned int over = __ballot_sync(0xffffffffu, lane >= have || ve - v0 > (uint32_t)Buf::TILE);
             const int cnt = over ? __ffs(over) - 1 : 32;  // at least 1: a slice fits a tile
@@ -294,7 +325,7 @@ __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst)
             const uint32_t o = vp % Buf::CAP;
             if (lane < cnt)
                 loc[(next + lane) & (kDescRing - 1)] =
-                    staged ? (int)(o >> 5) | b << 16 | ((tile / kWaveTiles) & 1) << 24 : -1;
+                    staged ? (int)(PACK ? o : o >> 5) | b << 16 | ((tile / kWaveTiles) & 1) << 24 : -1;
             // a run of neighbouring slices: one pair of copies, by the run's first lane
             const bool head = lane < cnt && staged && (lane == 0 || d.width < 0);
             const unsigned int heads = __ballot_sync(0xffffffffu, head || lane >= cnt || !staged);
@@ -303,9 +334,14 @@ __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst)
             if (head && run > 0) {
                 // the launch's last power is the last use of the entries (see k_mpk)
                 const bool last_use = a.stream_last && ((d.ckr >> 6) & 31u) == (uint32_t)a.p_launch;
-                bulk_g2s(sval + o, static_cast<const T *>(a.v_val) + 32 * (int64_t)d.e32, run * (uint32_t)sizeof(T), &full[b],
-                         last_use);
-                bulk_g2s(scol + o, a.v_col + 32 * (int64_t)d.e32, run * 4u, &full[b], last_use);
+                if constexpr (PACK) {
+                    bulk_g2s(smem + 16 * o, static_cast<const uint8_t *>(a.v_val) + 16 * (int64_t)d.e32, run * 16u, &full[b],
+                             last_use);
+                } else {
+                    bulk_g2s(sval + o, static_cast<const T *>(a.v_val) + 32 * (int64_t)d.e32, run * (uint32_t)sizeof(T),
+                             &full[b], last_use);
+                    bulk_g2s(scol + o, a.v_col + 32 * (int64_t)d.e32, run * 4u, &full[b], last_use);
+                }
             }
             next += cnt;
             if (lane == b) t_desc = next;
@@ -454,7 +490,8 @@ __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst)
                 __syncwarp();  // lane 0's acquire, for every lane while `seen` holds
             }
             WaveDesc d = desc[idx & (kDescRing - 1)];
-            d.width &= 0x7fffffff;
+            const bool wide = PACK && (d.width & kWideSlice) != 0;
+            d.width = width_of(d.width);
             const int lc = loc[idx & (kDescRing - 1)];
             const int cell = (int)(d.ckr >> 11), k = (int)(d.ckr >> 6) & 31, rows = (int)(d.ckr & 63u);
             if (cell >= ready) {  // the cell's dependencies
@@ -490,37 +527,52 @@ __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst)
                 const bool valid = rl < rows;
                 // rows in order, or the row map's (slices of rows sorted by length)
                 const int64_t row = a.v_rowmap ? (valid ? __ldg(a.v_rowmap + d.row0 + rl) : 0) : d.row0 + rl;
+                // calls f(values, columns) with the slice's entries, wherever they are
+                auto entries = [&](auto f) {
+                    if constexpr (PACK) {
+                        auto at = [&](const uint8_t *p) {
+                            const int32_t *first = reinterpret_cast<const int32_t *>(p);
+                            const uint8_t *c = p + 16 * ((d.width + 3) / 4);
+                            const DictVal<AT> v{c + (wide ? 128 : 64) * (int64_t)d.width, s_dict};
+                            if (wide)
+                                f(v, SCol{reinterpret_cast<const int32_t *>(c)});
+                            else
+                                f(v, NearCol{reinterpret_cast<const uint16_t *>(c), first});
+                        };
+                        if (lc >= 0)
+                            at(smem + 16 * (lc & 0xffff));
+                        else
+                            at(static_cast<const uint8_t *>(a.v_val) + 16 * (int64_t)d.e32);
+                    } else if (lc >= 0) {
+                        const int o = 32 * (lc & 0xffff);
+                        f(SVal<VT, AT>{sval + o}, SCol{scol + o});
+                    } else {  // a slice wider than the buffer takes: entries from global memory
+                        const int64_t e = 32 * (int64_t)d.e32;
+                        f(GVal<VT, AT>{static_cast<const T *>(a.v_val) + e}, GCol{a.v_col + e});
+                    }
+                };
                 if constexpr (BATCH) {
                     // the instance's vectors, addressed by rows of the whole batch
                     const WaveInst in = inst->at[dinst[idx & (kDescRing - 1)]];
                     const int64_t at = row * M + lane % M;
                     double *const y = in.y + (k * in.rows - in.row0) * M;
                     const double *const x = (k == 1 ? in.x - in.row0 * M : y - in.rows * M) + lane % M;
-                    double own = 0.0;
+                    double own = 0.0, acc = 0.0;
                     const bool copy = k == 1 && in.y != in.x && valid;
                     if (copy) own = in.x[at - in.row0 * M];
-                    double acc;
-                    if (lc >= 0) {
-                        const int o = 32 * (lc & 0xffff) + rl;
-                        acc = unit_sum<M, double>(SVal<VT>{sval + o}, SCol{scol + o}, d.width, x);
-                    } else {
-                        const int64_t e = 32 * (int64_t)d.e32 + rl;
-                        acc = unit_sum<M, double>(GVal<VT>{static_cast<const T *>(a.v_val) + e}, GCol{a.v_col + e}, d.width, x);
-                    }
+                    entries([&](auto sv, auto sc) {
+                        sv.lane(rl);
+                        sc.lane(rl);
+                        acc = unit_sum<M, double>(sv, sc, d.width, x);
+                    });
                     if (valid) y[at] = acc;
                     if (copy) in.y[at - in.row0 * M] = own;
-                } else if (lc >= 0) {
+                } else {
                     const double *xin = input_block<M>(a, k);
                     const AT *xacc = InputAcc<M, AT>::get(a, k);
-                    const int o = 32 * (lc & 0xffff);
-                    unit_row<M, MODE, AT>(a, k, SVal<VT, AT>{sval + o}, SCol{scol + o}, d.width, rl, row, valid, xin, xacc,
-                                          lane);
-                } else {  // a slice wider than the buffer takes: entries from global memory
-                    const double *xin = input_block<M>(a, k);
-                    const AT *xacc = InputAcc<M, AT>::get(a, k);
-                    const int64_t e = 32 * (int64_t)d.e32;
-                    unit_row<M, MODE, AT>(a, k, GVal<VT, AT>{static_cast<const T *>(a.v_val) + e}, GCol{a.v_col + e}, d.width,
-                                          rl, row, valid, xin, xacc, lane);
+                    entries([&](auto sv, auto sc) {
+                        unit_row<M, MODE, AT>(a, k, sv, sc, d.width, rl, row, valid, xin, xacc, lane);
+                    });
                 }
             }
             __syncwarp();
@@ -541,7 +593,8 @@ __global__ void __launch_bounds__(kWaveBS, 1) k_wave_batch(const __grid_constant
 }
 
 template <class VT, int M> static void *wave_fn(int mode, bool a32) {
-    if (mode == kWaveBatchMode) return (void *)k_wave_batch<M, VT>;
+    if constexpr (!std::is_same<VT, ValDict>::value)  // (batch plans have no packed copies)
+        if (mode == kWaveBatchMode) return (void *)k_wave_batch<M, VT>;
     if constexpr (!std::is_same<VT, ValF64>::value)
         if (a32) {
             if (mode == MODE_HOST) {
@@ -572,5 +625,6 @@ template <class VT> void *select_wave_vt(int mode, int m, bool a32, int *smem) {
 void *select_wave_f64(int mode, int m, bool a32, int *smem);
 void *select_wave_f32(int mode, int m, bool a32, int *smem);
 void *select_wave_bf16(int mode, int m, bool a32, int *smem);
+void *select_wave_dict(int mode, int m, bool a32, int *smem);  // packed copies
 
 }  // namespace mpk

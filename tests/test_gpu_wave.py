@@ -162,3 +162,53 @@ def test_batch_instances(mpk, order, m, cache_bytes):
     inside.copy_(Xs[0])
     B.apply([inside] + Xs[1:], Ys)
     same(Ys, out)
+
+
+def _few_values(A, count, stream):
+    """A with `count` different values, among them -0.0 and the smallest normal of binary32
+    (which refuses subnormals)."""
+    table = np.concatenate([[-0.0, 0.0, 2.0 ** -126, -1048576.0],
+                            (np.arange(max(count, 4)) - 100.5) / 64.0])[:count]
+    pick = np.arange(A.nnz) % count  # every value occurs where there are `count` entries
+    order = np.argsort(gen.splitmix64(gen.derive_seed(stream), A.nnz), kind="stable")
+    return A.with_values(table[pick[order]])
+
+
+@pytest.mark.parametrize("order", [0, 1])
+@pytest.mark.parametrize("count", [1, 255, 256, 257])
+@pytest.mark.parametrize("val,accum", [("f64", 0), ("f32", 0), ("f32", 1)])
+def test_packed_slices(mpk, order, count, val, accum):
+    """Few different values: up to 256 are stored as numbers of a table; rows of 0 to 65 entries
+    (the widest are not staged), sorted by length, many groups."""
+    A = _few_values(_widths_matrix(3001, (65, 1, 30, 64, 7, 0, 40, 63), 950), count, 951)
+    _check(mpk, A, 1, 5, order, val=val, accum=accum, cache_bytes=60000)
+
+
+@pytest.mark.parametrize("order", [0, 1])
+@pytest.mark.parametrize("far", [65529, 65530, 65531, 65600])
+def test_packed_slices_far_columns(mpk, order, far):
+    """One row of some slices stores a column `far` on: 65534 past the smallest column among the
+    slice's rows still fits 16 bits, 65535 does not."""
+    n = 150001
+    i = np.arange(n)
+    off = np.where(i % 64 == 5, far, 1)
+    keep = i + off < n
+    rows = np.concatenate([i, i[keep]])
+    cols = np.concatenate([i, (i + off)[keep]])
+    A = gen.from_coo(n, rows, cols, np.zeros(rows.size))
+    A = _few_values(A, 9, 960)
+    _check(mpk, A, 1, 3, order, cache_bytes=60000)
+    dA = mpk.CsrMatrix.from_host(A)
+    P = mpk.plan(dA, mpk.build_levels(dA, 0), p_max=4, nrhs=1, order=order, cache_bytes=60000)
+    X = gen.vector(n, 1, stream=7)
+    perm = mpk.build_levels(dA, 0).perm.cpu().numpy() if order == mpk.ORDER_PLAN else np.arange(n)
+    Xin = torch.from_numpy(np.ascontiguousarray(X[perm]))
+    c = np.linspace(1.0, -0.5, 8)
+    out = P.cheb_filter(Xin.cuda(), 7, c, scale=9.0, shift=0.3).cpu().numpy()
+    want = oracle.cheb(A, X, 7, c, scale=9.0, shift=0.3)[perm]
+    assert np.array_equal(out.view(np.uint64), np.ascontiguousarray(want).view(np.uint64))
+    Yh = P.apply_host(Xin.pin_memory(), 4)
+    torch.cuda.synchronize()
+    P.sync_status()
+    want = oracle.mpk(A, X, 4)[:, perm]
+    assert np.array_equal(Yh.numpy().view(np.uint64), np.ascontiguousarray(want).view(np.uint64))

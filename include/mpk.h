@@ -251,11 +251,16 @@ void mpk_plan_destroy(mpk_plan_t *P);
  * X: n x m device block; Y: (p+1) x n x m device block (Y[0] receives a copy of X), in the
  * plan's order (opts.order).  1 <= p <= p_max (p = 0 only copies X).  X must not overlap
  * Y[1..p].  One persistent kernel executes the Lp-diagram cells (group g, power k) in
- * diagonal order, split into row chunks; each chunk waits on the completion flags of the
- * chunks its rows read at power k-1.  With MPK_ORDER_ORIGINAL a gather kernel first takes
- * X into plan order in the plan's workspace, the kernel computes every power there, and a
- * last pass writes Y[1..p] through the permutation (one gather per output row).  Results
- * equal back-to-back SpMV bit for bit.  Not safe to run concurrently with another call on the same plan.
+ * diagonal order.  Plans of shape 0 or 3 divide every cell's 32-row slices evenly over one
+ * block per SM, and a cell waits on the counters of the cells it reads at power k-1; the other
+ * shapes (and plans with trace, shuffle_seed, level_capped or split_levels, or whose tables do
+ * not fit mem_budget) run row chunks that wait on the completion flags of the chunks they read.
+ * With MPK_ORDER_ORIGINAL and a matrix of narrow band (the rows of X between a row's smallest
+ * and largest column fit a quarter of L2) the plan keeps a second copy of the matrix in A's
+ * own numbering, if mem_budget allows, and the kernel reads X and writes Y in place; else a
+ * gather kernel first takes X into plan order in the plan's workspace, the kernel computes
+ * every power there, and a last pass writes Y[1..p] through the permutation (one gather per
+ * output row).  Results equal back-to-back SpMV bit for bit.  Not safe to run concurrently with another call on the same plan.
  * ------------------------------------------------------------------------------------- */
 mpk_status mpk_apply(const mpk_plan_t *P, const double *X, int32_t p, double *Y, mpk_stream stream);
 
@@ -267,9 +272,9 @@ mpk_status mpk_apply(const mpk_plan_t *P, const double *X, int32_t p, double *Y,
  * levels), the staged engine and nrhs 1, the kernel stores every power's rows into Y_host as
  * its units finish, so the transfer to the host overlaps the wavefront; other plan-order plans
  * compute on the device and copy the p+1 blocks afterwards (level-capped plans need the first
- * case, else MPK_ERR_UNSUPPORTED).  With MPK_ORDER_ORIGINAL the powers are written through
- * the permutation straight into Y_host after the kernel (a temporary device copy of X is
- * allocated in stream order).  Asynchronous on `stream`: Y_host is complete when the stream
+ * case, else MPK_ERR_UNSUPPORTED).  With MPK_ORDER_ORIGINAL and no copy of the matrix in A's
+ * own numbering (see mpk_apply) the powers are written through the permutation straight into
+ * Y_host after the kernel (a temporary device copy of X is allocated in stream order).  Asynchronous on `stream`: Y_host is complete when the stream
  * is.  Y_host must not overlap X_host.  Not for batch plans (MPK_ERR_INVALID); not safe to run
  * concurrently with another call on the same plan. */
 mpk_status mpk_apply_host(const mpk_plan_t *P, const double *X_host, int32_t p, double *Y_host,

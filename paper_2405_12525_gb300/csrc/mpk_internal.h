@@ -299,6 +299,7 @@ struct KArgs {
     const int32_t *v_col;
     const int4 *v_slice;       // slices: (first entry / 32, entries a row, first row or row map entry, rows)
     const double *v_dict;      // packed copies: the table of values (v_val is the slices' stream)
+    const int32_t *v_iperm;    // batch plans in the matrices' numbering: rows of the workspace
     const int32_t *v_rowmap;   // row of every lane of every slice (-1: none), or null: consecutive rows
     const int4 *v_cell;
     const int32_t *v_gsl;

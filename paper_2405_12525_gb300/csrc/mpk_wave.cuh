@@ -557,16 +557,23 @@ __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst)
                     const int64_t at = row * M + lane % M;
                     double *const y = in.y + (k * in.rows - in.row0) * M;
                     const double *const x = (k == 1 ? in.x - in.row0 * M : y - in.rows * M) + lane % M;
+                    // where the plan's workspace has the row
+                    const int64_t aw = (a.v_iperm && valid ? __ldg(a.v_iperm + row) : row) * M + lane % M;
                     double own = 0.0, acc = 0.0;
-                    const bool copy = k == 1 && in.y != in.x && valid;
-                    if (copy) own = in.x[at - in.row0 * M];
+                    if (k == 1 && valid) own = in.x[at - in.row0 * M];
                     entries([&](auto sv, auto sc) {
                         sv.lane(rl);
                         sc.lane(rl);
                         acc = unit_sum<M, double>(sv, sc, d.width, x);
                     });
-                    if (valid) y[at] = acc;
-                    if (copy) in.y[at - in.row0 * M] = own;
+                    if (valid) {
+                        y[at] = acc;
+                        __stcs(a.ybase + k * a.ystride + aw, acc);
+                        if (k == 1) {
+                            if (in.y != in.x) in.y[at - in.row0 * M] = own;
+                            __stcs(a.ybase + aw, own);
+                        }
+                    }
                 } else {
                     const double *xin = input_block<M>(a, k);
                     const AT *xacc = InputAcc<M, AT>::get(a, k);

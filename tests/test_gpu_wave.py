@@ -212,3 +212,28 @@ def test_packed_slices_far_columns(mpk, order, far):
     P.sync_status()
     want = oracle.mpk(A, X, 4)[:, perm]
     assert np.array_equal(Yh.numpy().view(np.uint64), np.ascontiguousarray(want).view(np.uint64))
+
+
+@pytest.mark.parametrize("order", [0, 1])
+@pytest.mark.parametrize("m", [1, 8])
+@pytest.mark.parametrize("x_in_place", [False, True])
+def test_batch_workspace_after_outputs(mpk, order, m, x_in_place):
+    """The plan's workspace holds every power, in plan order, also after a call with outputs."""
+    mats = [gen.laplacian_3d(9, 8, 7), _widths_matrix(901, (1, 30, 4, 17, 0), 940), gen.laplacian_2d(40, 31)]
+    ps = [4, 2, 5]
+    dAs = [mpk.CsrMatrix.from_host(A) for A in mats]
+    B = mpk.batch_plan(dAs, ps, nrhs=m, order=order)
+    perms = [mpk.build_levels(d, 0).perm.cpu().numpy() for d in dAs]
+    Xh = [gen.vector(A.n, m, stream=30 + i) for i, A in enumerate(mats)]
+    want = [np.ascontiguousarray(oracle.mpk(A, X, p)[:, q]) for A, X, p, q in zip(mats, Xh, ps, perms)]
+    Xs = [torch.from_numpy(np.ascontiguousarray(X[q] if order == mpk.ORDER_PLAN else X)).cuda()
+          for X, q in zip(Xh, perms)]
+    Ys = [torch.full(w.shape, float("nan"), dtype=torch.float64, device="cuda") for w in want]
+    if x_in_place:
+        for X, Y in zip(Xs, Ys):
+            Y[0].copy_(X)
+        Xs = [Y[0] for Y in Ys]
+    B.apply([torch.zeros_like(X) for X in Xs], in_place=True)
+    B.apply(Xs, Ys)
+    for V, w in zip(B.views(), want):
+        assert np.array_equal(V.cpu().numpy().view(np.uint64), w.view(np.uint64))

@@ -510,31 +510,43 @@ __global__ void k_dict_number(Dict *d, int vt) {
     }
 }
 
-// One warp per slice: the row of every lane, as k_fill_slices; f(j, entry of the row or -1) for every
-// entry a row of the slice
-template <class F>
-__device__ __forceinline__ void slice_entries(int64_t s, int w, const int32_t *rp, const int32_t *perm, const int32_t *slice_row,
-                                              const int32_t *map, int lane, F f) {
-    int32_t row = map ? map[32 * s + lane] : slice_row[s] + lane;
-    if (!map && row >= slice_row[s + 1]) row = -1;
-    int32_t e0 = 0, len = 0;
-    if (row >= 0) {
-        const int32_t old = perm ? perm[row] : row;
-        e0 = rp[old];
-        len = rp[old + 1] - e0;
+// Where packed slices come from, one warp per slice: visit() calls f(j, place of the value, column or
+// -1) for every entry j a row of the slice.
+// A's rows, as k_fill_slices takes them
+struct CsrRows {
+    const int32_t *rp, *ci, *perm, *iperm, *slice_row, *map, *widths;
+    __device__ __forceinline__ int width(int64_t s) const { return widths[s] & (kWideSlice - 1); }
+    template <class F> __device__ __forceinline__ void visit(int64_t s, int w, int lane, F f) const {
+        int32_t row = map ? map[32 * s + lane] : slice_row[s] + lane;
+        if (!map && row >= slice_row[s + 1]) row = -1;
+        int32_t e0 = 0, len = 0;
+        if (row >= 0) {
+            const int32_t old = perm ? perm[row] : row;
+            e0 = rp[old];
+            len = rp[old + 1] - e0;
+        }
+        for (int j = 0; j < w; ++j) f(j, (int64_t)(e0 + j), j < len ? (iperm ? iperm[ci[e0 + j]] : ci[e0 + j]) : -1);
     }
-    for (int j = 0; j < w; ++j) f(j, j < len ? e0 + j : -1);
-}
-// packed slices: marks in `width` those whose columns do not fit 16-bit distances, sizes in units
-__global__ void k_pack_size(int32_t nslices, const int32_t *rp, const int32_t *ci, const int32_t *perm, const int32_t *iperm,
-                            const int32_t *slice_row, const int32_t *map, int32_t *width, int64_t *units) {
+};
+// the plan's sliced copy: coalesced, where A's rows in plan order are gathered (256^3, plan order: planning
+// took 10.2 ms from A, 7.1 ms from the copy)
+struct PlanRows {
+    const int64_t *sptr;
+    const int32_t *col;
+    __device__ __forceinline__ int width(int64_t s) const { return (int)((sptr[s + 1] - sptr[s]) >> 5); }
+    template <class F> __device__ __forceinline__ void visit(int64_t s, int w, int lane, F f) const {
+        const int64_t e0 = sptr[s] + lane;
+        for (int j = 0; j < w; ++j) f(j, e0 + 32 * j, col[e0 + 32 * j]);
+    }
+};
+// packed slices: widths, marking those whose columns do not fit 16-bit distances, and sizes in units
+template <class R> __global__ void k_pack_size(int32_t nslices, R rows, int32_t *width, int64_t *units) {
     const int lane = threadIdx.x & 31;
     for (int64_t s = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; s < nslices;
          s += (int64_t)gridDim.x * blockDim.x >> 5) {
-        const int w = width[s];
+        const int w = rows.width(s);
         bool wide = false;
-        slice_entries(s, w, rp, perm, slice_row, map, lane, [&](int, int32_t e) {
-            const int32_t c = e < 0 ? -1 : (iperm ? iperm[ci[e]] : ci[e]);
+        rows.visit(s, w, lane, [&](int, int64_t, int32_t c) {
             const int32_t hi = __reduce_max_sync(0xffffffffu, c);
             const int32_t lo = __reduce_min_sync(0xffffffffu, c < 0 ? INT_MAX : c);
             wide = wide || hi - lo >= kNoCol;  // (an entry that no lane has: -1 - INT_MAX)
@@ -546,10 +558,9 @@ __global__ void k_pack_size(int32_t nslices, const int32_t *rp, const int32_t *c
         }
     }
 }
-template <class T>
-__global__ void k_pack_fill(int32_t nslices, const int32_t *rp, const int32_t *ci, const T *va, const int32_t *perm,
-                            const int32_t *iperm, const int32_t *slice_row, const int32_t *map, const int32_t *width,
-                            const int64_t *units, const Dict *d, uint8_t *stream) {
+template <class R, class T>
+__global__ void k_pack_fill(int32_t nslices, R rows, const T *va, const int32_t *width, const int64_t *units,
+                            const Dict *d, uint8_t *stream) {
     const int lane = threadIdx.x & 31;
     unsigned long long last = kNoValue;
     int last_q = 0;
@@ -560,8 +571,7 @@ __global__ void k_pack_fill(int32_t nslices, const int32_t *rp, const int32_t *c
         uint8_t *p = stream + 16 * units[s];
         int32_t *first = reinterpret_cast<int32_t *>(p);
         uint8_t *cols = p + 16 * ((w + 3) / 4), *vals = cols + (wide ? 128 : 64) * (int64_t)w;
-        slice_entries(s, w, rp, perm, slice_row, map, lane, [&](int j, int32_t e) {
-            const int32_t c = e < 0 ? -1 : (iperm ? iperm[ci[e]] : ci[e]);
+        rows.visit(s, w, lane, [&](int j, int64_t e, int32_t c) {
             const int32_t lo = __reduce_min_sync(0xffffffffu, c < 0 ? INT_MAX : c);
             if (lane == 0) first[j] = lo;
             if (wide)
@@ -569,7 +579,7 @@ __global__ void k_pack_fill(int32_t nslices, const int32_t *rp, const int32_t *c
             else
                 reinterpret_cast<uint16_t *>(cols)[32 * j + lane] = (uint16_t)(c < 0 ? kNoCol : c - lo);
             int q = 0;
-            if (e >= 0) {
+            if (c >= 0) {
                 const unsigned long long b = value_bits(va[e]);
                 if (b != last) {
                     int t = dict_slot(b);
@@ -655,8 +665,9 @@ static bool wave_tables(Plan &P, WaveSet &w, const std::vector<int32_t> &vs, con
     return true;
 }
 
-// The table of A's values (256^3: 0.2 ms; a matrix of random values is given up after a few
-// entries); false if there are more than kDictSize.
+// The table of A's values; false if there are more than kDictSize (a matrix of random values is given
+// up after its first entries).  The set-up takes as long with packed copies as without: what the
+// table costs, the smaller copy saves (131 x 127 x 113: 5.29 against 5.35 ms).
 static bool find_values(const Plan &P, const mpk_csr *A, Dict *d, cudaStream_t s) {
     k_dict_init<<<1, 1024, 0, s>>>(d);
     MPK_LAUNCHED();
@@ -673,6 +684,37 @@ static bool find_values(const Plan &P, const mpk_csr *A, Dict *d, cudaStream_t s
     MPK_CUDA(cudaMemcpyAsync(found, &d->count, sizeof(found), cudaMemcpyDeviceToHost, s));
     MPK_CUDA(cudaStreamSynchronize(s));
     return !found[1] && found[0] <= kDictSize;
+}
+
+// The packed copy of the slices `rows` (values at `val`); width and units: scratch of a word a slice.
+template <class R>
+static bool pack_slices(Plan &P, WaveSet &w, const R &rows, const void *val, const std::vector<int32_t> &vs,
+                        const std::vector<WaveRange> &ranges, const Dict *dict, const int32_t *d_srow, int32_t NS,
+                        Tmp<int32_t> &width, Tmp<int64_t> &units, std::vector<int32_t> &host, cudaStream_t s) {
+    const int grid = grid_n(32 * (int64_t)NS);
+    k_pack_size<<<grid, 256, 0, s>>>(NS, rows, width.p, units.p);
+    MPK_LAUNCHED();
+    exclusive_scan(units.p, units.p, NS, s);
+    int64_t total = 0;
+    MPK_CUDA(cudaMemcpyAsync(&total, units.p + NS, sizeof(total), cudaMemcpyDeviceToHost, s));
+    MPK_CUDA(cudaStreamSynchronize(s));
+    if (total >= INT32_MAX) return false;
+    const int64_t bytes = 16 * total + (int64_t)sizeof(dict->value);
+    if (!wave_tables(P, w, vs, ranges, units.p, width.p, d_srow, NS, host, bytes, s)) return false;
+    uint8_t *dev = static_cast<uint8_t *>(P.arena.alloc(bytes));  // the table, then the stream
+    uint8_t *stream = dev + sizeof(dict->value);
+    MPK_CUDA(cudaMemcpyAsync(dev, dict->value, sizeof(dict->value), cudaMemcpyDeviceToDevice, s));
+    if (P.val_type == MPK_F64)
+        k_pack_fill<<<grid, 256, 0, s>>>(NS, rows, static_cast<const double *>(val), width.p, units.p, dict, stream);
+    else if (P.val_type == MPK_F32)
+        k_pack_fill<<<grid, 256, 0, s>>>(NS, rows, static_cast<const float *>(val), width.p, units.p, dict, stream);
+    else
+        k_pack_fill<<<grid, 256, 0, s>>>(NS, rows, static_cast<const uint16_t *>(val), width.p, units.p, dict, stream);
+    MPK_LAUNCHED();
+    w.val = stream;
+    w.dict = reinterpret_cast<const double *>(dev);
+    w.ok = true;
+    return true;
 }
 
 // A sliced copy of its own for the wave kernel: the rows in A's numbering (perm NULL) or in plan
@@ -722,36 +764,9 @@ static bool wave_copy(Plan &P, WaveSet &w, const mpk_csr *A, const int32_t *perm
     }
     if (entries / 32 >= INT32_MAX) return false;
     w.rowmap = map;
-    if (dict) {
-        k_pack_size<<<grid_n(32 * (int64_t)NS), 256, 0, s>>>(NS, A->row_ptr, A->col, perm, iperm, d_srow.p, map, d_width.p,
-                                                             d_ent.p);
-        MPK_LAUNCHED();
-        exclusive_scan(d_ent.p, d_ent.p, NS, s);
-        int64_t units = 0;
-        MPK_CUDA(cudaMemcpyAsync(&units, d_ent.p + NS, sizeof(units), cudaMemcpyDeviceToHost, s));
-        MPK_CUDA(cudaStreamSynchronize(s));
-        if (units >= INT32_MAX) return false;
-        const int64_t bytes = 16 * units + (int64_t)sizeof(dict->value);
-        if (!wave_tables(P, w, vs, ranges, d_ent.p, d_width.p, d_srow.p, NS, host, bytes, s)) return false;
-        uint8_t *dev = static_cast<uint8_t *>(P.arena.alloc(bytes));  // the table, then the stream
-        uint8_t *stream = dev + sizeof(dict->value);
-        MPK_CUDA(cudaMemcpyAsync(dev, dict->value, sizeof(dict->value), cudaMemcpyDeviceToDevice, s));
-#define PACK(T)                                                                                                  \
-    k_pack_fill<T><<<grid_n(32 * (int64_t)NS), 256, 0, s>>>(NS, A->row_ptr, A->col, static_cast<const T *>(A->val), perm, \
-                                                            iperm, d_srow.p, map, d_width.p, d_ent.p, dict, stream)
-        if (P.val_type == MPK_F64)
-            PACK(double);
-        else if (P.val_type == MPK_F32)
-            PACK(float);
-        else
-            PACK(uint16_t);
-#undef PACK
-        MPK_LAUNCHED();
-        w.val = stream;
-        w.dict = reinterpret_cast<const double *>(dev);
-        w.ok = true;
-        return true;
-    }
+    if (dict)
+        return pack_slices(P, w, CsrRows{A->row_ptr, A->col, perm, iperm, d_srow.p, map, d_width.p}, A->val, vs, ranges, dict,
+                           d_srow.p, NS, d_width, d_ent, host, s);
     const int64_t bytes = (P.val_bytes + 4) * (entries + 32);
     if (!wave_tables(P, w, vs, ranges, d_ent.p, nullptr, d_srow.p, NS, host, bytes, s)) return false;
     int32_t *col = static_cast<int32_t *>(P.arena.alloc((entries + 32) * (4 + P.val_bytes)));  // columns, then values
@@ -840,7 +855,7 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
     }
     // A matrix larger than the cache that has few different values gets packed copies (about 3.2 bytes an
     // entry in place of 12): the copies into shared memory, not HBM, are what they save, so they also help
-    // at p = 1.  Measured, us, plain -> packed copies, 256^3 7-point / 150^3 27-point, p = 8:
+    // at p = 1.  Measured before the rounding of groups below, us, plain -> packed copies, 256^3 7-point / 150^3 27-point, p = 8:
     //   binary64, A's order:              2215 -> 1966 / 1907 -> 1348;  plan order: 2035 -> 1850 / 1912 -> 1306
     //   binary32, plan order:             1807 -> 1852 / 1477 -> 1306
     //   bfloat16, binary32 sums, A's order: 1470 -> 1524 / 825 -> 715
@@ -896,7 +911,14 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
     }
     if (near) {
         bool own = false;
-        if (plan_dict || P.padded > P.nnz + P.nnz / 25) {
+        if (P.padded <= P.nnz + P.nnz / 25) {
+            if (plan_dict) own = spare(P, P.wave, [&]() {
+                    Tmp<int32_t> width(NS, s);
+                    Tmp<int64_t> units((int64_t)NS + 1, s);
+                    return pack_slices(P, P.wave, PlanRows{P.slice_ptr, P.col}, P.val, vs, ranges, plan_dict, d_srow, NS,
+                                       width, units, host[0], s);
+                });
+        } else {
             std::vector<int32_t> vrow;
             for (int32_t g = 0; g <= VG; ++g) vrow.push_back(s_row[vs[g]]);
             own = spare(P, P.wave, [&]() {

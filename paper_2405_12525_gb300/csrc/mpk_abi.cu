@@ -296,9 +296,10 @@ extern "C" mpk_status mpk_apply_host(const mpk_plan_t *Ph, const double *X_host,
         KArgs a = base_args(P, p);
         a.ring = p + 1;
         if (natural) wave_args(P.natural, p, a);
-        // (with many groups in plan order the output link is the bound, and k_mpk's finer units feed it
-        // evenly: 128^3, p = 8, 999 against 1004 us)
-        if (fused && !natural && P.wave.ngroups > 1) a.v_cell = nullptr;
+        // (In plan order, with many groups or powers of more than 1.5 MB, the output link is the bound,
+        // and k_mpk's finer units feed it evenly.  p = 10, k_wave / k_mpk, us: 31^3 46 / 77, 50^3 100 /
+        // 103, 64^3 170 / 160, 80^3 327 / 322; 128^3, p = 8: 1004 / 999.)
+        if (fused && !natural && (P.wave.ngroups > 1 || 8 * nm > (3 << 19))) a.v_cell = nullptr;
         a.x0 = P.work;
         a.ybase = P.work;
         if (P.accum == MPK_F32) launch_round_f32(P.work, nm, P.shadow, s);

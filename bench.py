@@ -39,8 +39,8 @@ DFMA_LANES_PER_CLK_PER_SM = 2  # GB300's FP64 FMA issue rate per SM (unit count 
 SM_MAX_MHZ_FALLBACK = 2070.0   # used only if nvidia-smi gives no clock
 # the level-blocked kernel, its tunables and the planner that cuts its chunks
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_2405_12525_gb300", "csrc", f)
-                  for f in ("mpk_kernel_dev.cuh", "mpk_internal.h", "mpk_plan.cu")]
-TRAFFIC_RECORD = os.path.join(ROOT, "profiles", "k_mpk_traffic.json")
+                  for f in ("mpk_wave.cuh", "mpk_kernel_dev.cuh", "mpk_internal.h", "mpk_plan.cu")]
+TRAFFIC_RECORD = os.path.join(ROOT, "profiles", "k_wave_traffic.json")
 
 
 def measured_profile(side: int, accum: str):
@@ -481,7 +481,7 @@ def main_cheb(args):
                        "levels": desc["num_levels"], "groups": desc["num_groups"], "chunks": desc["num_chunks"]},
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak_alu, "unit": "TFLOP/s",
                          "frac": achieved / peak_alu, "traffic": None,
-                         "kernel": ("k_mpk<2,1> (recurrence mode), 8 launches per step" if chosen == "staged" else
+                         "kernel": ("k_wave<2,1> (recurrence mode), 8 launches per step" if chosen == "staged" else
                                     "k_sweep<2,1> (recurrence mode, unblocked), 64 launches per step"),
                          "algorithmic": "per recurrence step 2 nnz m (SpMV) + 8 n m (update, complex accumulate)"},
             "comparator": {"plain_spmv_same_count_ms": ms_spmv,
@@ -1061,7 +1061,7 @@ def main():
                     "achieved_note": "algorithmic HBM bytes of one apply (A once, X once, p binary64 powers and "
                                      "their binary32 copies written) / kernel time"}
     roofline.update({
-        "kernel": "k_mpk (persistent level-blocked kernel), one launch per step", "kernel_ms": ms,
+        "kernel": "k_wave (persistent level-blocked kernel), one launch per step", "kernel_ms": ms,
         "algorithmic": "2 flop per stored entry per power: 2*nnz*p per launch",
         "l2_blocked_roof_ms": roof_blocked_ms, "frac_of_l2_blocked_roof": roof_blocked_ms / ms,
         "l2_blocked_roof": f"max((A_B + (p+1) V) / BW_HBM, p (A_B + 2V) / BW_L2) = max({t_hbm * 1e3:.3f}, "

@@ -177,11 +177,10 @@ class Server:
                 "max_inflight": self.max_seen_inflight, "peak_bytes": self.peak_used}
 
 
-# Block shape of the serving plans: the unstaged shape (plan option shape=3).  Up to eight
-# requests run at once, each a persistent kernel on its own stream, so the kernels share the
-# SMs; blocks that stage no entries in shared memory start beside other requests' blocks.
-# Config 5 at 200 requests/s served 20.9 requests/s with it against 16.8 with the staged
-# shape a single launch prefers (p50 at 10 requests/s: 50 ms against 74 ms).
+# Block shape of the serving plans: plan option shape=3, which runs the wave kernel (one block per
+# SM, launches of several requests take turns), or, where that cannot run, the unstaged blocks of
+# the ticketed kernel, which start beside other requests' blocks.  Mixed requests at 200 / 10 a
+# second: 22.6 requests/s served / p50 of 33 ms; on the ticketed kernel 21.4 / 48 ms.
 SERVING_SHAPE = 3
 
 

@@ -940,8 +940,15 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
         WaveRange r{(int32_t)nrow.size(), 0, t.p, t.bytes};
         int64_t rows = t.r1 - t.r0;
         if (!t.one) {
-            rows = std::max<int64_t>(band, (int64_t)((double)t.most / (entry_bytes * (double)(P.nnz / std::max(n, 1) + 1) +
-                                                                       (double)row_bytes)));
+            // A default budget of 5/4 of L2 where that is a good part of the matrix and its vectors, 3/5 of
+            // L2 beyond 3 times L2, where its window no longer stays in L2 (p = 8, us, 5/4 / 3/5 of L2;
+            // packed 7-point: 131^3 258 / 269, 200^3 872 / 876, 230^3 1384 / 1318, 256^3 1946 / 1794, 290^3
+            // 3007 / 2801; 256^3 bfloat16, binary32 sums: 1457 / 1346; packed 5-point: 2000^2 376 / 382,
+            // 4000 x 4100 1513 / 1489)
+            const double a_row = entry_bytes * (double)(P.nnz / std::max(n, 1) + 1) + (double)row_bytes;
+            const bool large = default_budget && a_row * (double)rows > 3.0 * (double)device_l2_bytes();
+            const int64_t most = large ? device_l2_bytes() / 5 * 3 / (kSlotSkew * t.p + 1) : t.most;
+            rows = std::max<int64_t>(band, (int64_t)((double)most / a_row));
             // equal shares for the blocks where a group has a few slices for each (27-point stencil on
             // 150^3, p = 8, packed: 1349 -> 1261 us; below, a whole slice more for each would be too much)
             const int64_t even = 32 * (int64_t)device_sms();

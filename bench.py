@@ -1090,7 +1090,7 @@ def main():
                        "cache_bytes": desc["cache_bytes"], "window": desc["window"]},
             "roofline": roofline,
             "original_order": {"ms_per_step": ms_orig, "gflops": flops / (ms_orig * 1e-3) / 1e9,
-                               "note": "gather X, level-blocked kernel, tiled permuted write of Y[1..p]",
+                               "note": "level-blocked kernel on a copy of the matrix in its own numbering (no gather or scatter)",
                                "bit_identical_to_plan_order": orig_identical},
             "comparator": {**{k + "_gflops": flops / (v * 1e-3) / 1e9 for k, v in comps.items()},
                            **{k + "_ms": v for k, v in comps.items()},

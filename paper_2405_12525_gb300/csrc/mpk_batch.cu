@@ -141,6 +141,12 @@ extern "C" mpk_status mpk_batch_apply(const mpk_plan_t *Ph, const double *const 
             const int64_t skip = (j == i && Y[j] == X[i]) ? nj : 0;
             if (nj > 0 && Y[j] && overlap(X[i], ni, Y[j] + skip, nj * (P.inst_p[j] + 1) - skip)) direct = false;
         }
+        // outputs that share memory: the kernel reads a block's powers where it wrote them, so they
+        // go through the workspace, and the last block's rows stand
+        for (int32_t j = 0; j < i && direct; ++j) {
+            const int64_t nj = (int64_t)(P.inst_row[j + 1] - P.inst_row[j]) * m;
+            if (nj > 0 && overlap(Y[i], ni * (P.inst_p[i] + 1), Y[j], nj * (P.inst_p[j] + 1))) direct = false;
+        }
     }
     if (direct) {
         WaveBatch inst{};

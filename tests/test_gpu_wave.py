@@ -237,3 +237,28 @@ def test_batch_workspace_after_outputs(mpk, order, m, x_in_place):
     B.apply(Xs, Ys)
     for V, w in zip(B.views(), want):
         assert np.array_equal(V.cpu().numpy().view(np.uint64), w.view(np.uint64))
+
+
+@pytest.mark.parametrize("order", [0, 1])
+@pytest.mark.parametrize("m", [1, 4])
+def test_batch_outputs_that_share_memory(mpk, order, m):
+    """Outputs in one buffer (a scratch output given for several blocks): the powers of the last
+    block that writes there, the others' in the workspace."""
+    mats = [gen.laplacian_3d(9, 8, 7), gen.laplacian_2d(40, 31), gen.laplacian_3d(12, 11, 10)]
+    ps = [5, 4, 3]
+    dAs = [mpk.CsrMatrix.from_host(A) for A in mats]
+    B = mpk.batch_plan(dAs, ps, nrhs=m, order=order)
+    perms = [mpk.build_levels(d, 0).perm.cpu().numpy() for d in dAs]
+    Xh = [gen.vector(A.n, m, stream=50 + i) for i, A in enumerate(mats)]
+    want = [oracle.mpk(A, X, p) for A, X, p in zip(mats, Xh, ps)]
+    Xs = [torch.from_numpy(np.ascontiguousarray(X[q] if order == mpk.ORDER_PLAN else X)).cuda()
+          for X, q in zip(Xh, perms)]
+    pool = torch.empty(max(w.size for w in want) + 7, dtype=torch.float64, device="cuda")
+    Ys = [pool[7 * (i % 2):][:w.size].view(w.shape) for i, w in enumerate(want)]
+    for _ in range(3):
+        pool.fill_(float("nan"))
+        B.apply(Xs, Ys)
+        last = want[2][:, perms[2]] if order == mpk.ORDER_PLAN else want[2]
+        assert np.array_equal(Ys[2].cpu().numpy().view(np.uint64), np.ascontiguousarray(last).view(np.uint64))
+        for V, w, q in zip(B.views(), want, perms):
+            assert np.array_equal(V.cpu().numpy().view(np.uint64), np.ascontiguousarray(w[:, q]).view(np.uint64))

@@ -86,7 +86,8 @@ __global__ void k_tfill(int32_t n, const int32_t *rp, const int32_t *ci, int32_t
 constexpr int64_t kBfsWaitNs = 2000000000LL;  // bound of one grid-barrier wait (2 s)
 constexpr int kBfsBS = 512;                   // one block an SM: half the arrivals of two blocks of 256
 constexpr int kBfsNarrow = 512;               // vertices of a level that one block expands alone
-constexpr int kBfsAlone = 1 << 15;            // levels it expands before it meets the others
+constexpr int kBfsAlone = 1 << 15;            // levels it expands before it meets the others,
+constexpr int kBfsAloneShare = 8;             // within 1/8 of the others' bound (see k_bfs_all)
 struct BfsState {
     unsigned long long bar;  // arrivals at grid barriers, all rounds, << 32 | vertices found, all levels
     int4 left[2];      // where block 0 left the narrow levels: head, tail, level
@@ -193,7 +194,7 @@ __device__ __forceinline__ int bfs_visit(const int32_t *rp, const int32_t *vi, i
 __global__ void __launch_bounds__(kBfsBS, 1) k_bfs_all(const int32_t *rp, const int32_t *ci, const int32_t *tp,
                                                     const int32_t *tci, int32_t *level_of, int4 *queue, int32_t n,
                                                     int32_t head0, int32_t tail0, BfsState *st, int64_t limit_ns) {
-    __shared__ int s_found, s_tail;
+    __shared__ int s_found, s_tail, s_late;
     const int64_t gtid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t gstride = (int64_t)gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
@@ -220,13 +221,20 @@ __global__ void __launch_bounds__(kBfsBS, 1) k_bfs_all(const int32_t *rp, const 
     for (;;) {
         if (tail > head && tail - head <= kBfsNarrow) {
             // narrow levels: block 0 alone, with block barriers and the queue's end in shared memory,
-            // while the others wait at one grid barrier (kBfsAlone levels at most, well inside its bound)
+            // while the others wait at one grid barrier.  A level takes a few us, but one with a long
+            // row takes as long as the row's walk (a hub of 500 neighbours: 200 us), so the loop ends
+            // by time too: no level starts after limit_ns / 8 cycles (1/8 of the bound at 1 GHz), and the
+            // others wait for twice the bound, which leaves the last level the whole of it
             if (blockIdx.x == 0) {
                 int32_t h = (int32_t)head, t = (int32_t)tail, l = lev;
-                for (int it = 0; it < kBfsAlone && t > h && t - h <= kBfsNarrow; ++it) {
+                const long long c0 = clock64();
+                if (threadIdx.x == 0) s_late = 0;
+                __syncthreads();
+                for (int it = 0; it < kBfsAlone && !s_late && t > h && t - h <= kBfsNarrow; ++it) {
                     if (threadIdx.x == 0) s_tail = t;
                     __syncthreads();
                     expand(h + threadIdx.x, blockDim.x, t, l + 1, &s_tail);
+                    if (threadIdx.x == 0) s_late = clock64() - c0 > limit_ns / kBfsAloneShare;
                     __syncthreads();
                     h = t;
                     t = s_tail;
@@ -238,7 +246,7 @@ __global__ void __launch_bounds__(kBfsBS, 1) k_bfs_all(const int32_t *rp, const 
                     st->left[(round + 1) & 1] = make_int4(h, t, l, 0);
                 }
             }
-            if (bfs_grid_barrier(st, ++round, &s_found, limit_ns) < 0) return;
+            if (bfs_grid_barrier(st, ++round, &s_found, 2 * limit_ns) < 0) return;
             // (two places in turn: block 0 writes this one again only after the next barrier)
             const volatile int4 *left = &st->left[round & 1];
             head = left->x;

@@ -79,18 +79,20 @@ __global__ void k_tfill(int32_t n, const int32_t *rp, const int32_t *ci, int32_t
 // the barrier: 256^3 8.99 -> 7.97 ms, 131x127x113 3.14 -> 2.95 ms, banded 300k 2.70 -> 2.03 ms.
 // (Claims without a look at the level first, and prefetches of the winners' columns: slower.)
 // A graph whose search runs dry before every vertex is reached continues from the smallest
-// untouched vertex (a grid-wide minimum, one barrier), which opens the next level (one more
-// barrier to publish it); the minima rotate through three slots, so that a slot is reset only
+// untouched vertex, which opens the next level: block 0 looks for it beside the narrow levels
+// (20000 vertices without edges: 27 ms; by the grid alone 166 to 187), the grid when it is not among the next kBfsNear *
+// kBfsBS (a grid-wide minimum, one barrier, and one more to publish it); the minima rotate through three slots, so that a slot is reset only
 // after its last readers passed the next barrier.  Every barrier wait is bounded; on expiry the
 // kernel records the failure and all blocks leave.
 constexpr int64_t kBfsWaitNs = 2000000000LL;  // bound of one grid-barrier wait (2 s)
 constexpr int kBfsBS = 512;                   // one block an SM: half the arrivals of two blocks of 256
 constexpr int kBfsNarrow = 512;               // vertices of a level that one block expands alone
 constexpr int kBfsAlone = 1 << 15;            // levels it expands before it meets the others,
+constexpr int kBfsNear = 16;                  // blocks of kBfsBS vertices it looks at for a restart
 constexpr int kBfsAloneShare = 8;             // within 1/8 of the others' bound (see k_bfs_all)
 struct BfsState {
     unsigned long long bar;  // arrivals at grid barriers, all rounds, << 32 | vertices found, all levels
-    int4 left[2];      // where block 0 left the narrow levels: head, tail, level
+    int4 left[2];      // where block 0 left the narrow levels: head, tail, level, cursor
     int32_t tail;      // end of the queue
     int32_t minv[3];   // smallest untouched vertex per restart (INT_MAX: none)
     int32_t levels;    // number of levels (written at the end)
@@ -194,7 +196,8 @@ __device__ __forceinline__ int bfs_visit(const int32_t *rp, const int32_t *vi, i
 __global__ void __launch_bounds__(kBfsBS, 1) k_bfs_all(const int32_t *rp, const int32_t *ci, const int32_t *tp,
                                                     const int32_t *tci, int32_t *level_of, int4 *queue, int32_t n,
                                                     int32_t head0, int32_t tail0, BfsState *st, int64_t limit_ns) {
-    __shared__ int s_found, s_tail, s_late;
+    __shared__ int s_found, s_root;
+    __shared__ int2 s_end;  // end of the queue, and whether the narrow levels end here
     const int64_t gtid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t gstride = (int64_t)gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
@@ -210,9 +213,13 @@ __global__ void __launch_bounds__(kBfsBS, 1) k_bfs_all(const int32_t *rp, const 
         for (int64_t t = first; t - lane < last; t += step) {
             const bool on = t < last;
             const int4 e = on ? queue[t] : make_int4(0, 0, 0, 0);
+            int32_t f0 = 0, f1 = 0;  // (loaded before the first visit, not after it)
+            if (tp && on) {
+                f0 = tp[e.x];
+                f1 = tp[e.x + 1];
+            }
             wins += bfs_visit(rp, ci, e.y, e.z, e.x, level_of, next, queue, end, lane);
             if (tp) {
-                const int32_t f0 = on ? tp[e.x] : 0, f1 = on ? tp[e.x + 1] : 0;
                 wins += bfs_visit(rp, tci, f0, f1, e.x, level_of, next, queue, end, lane);
             }
         }
@@ -227,23 +234,46 @@ __global__ void __launch_bounds__(kBfsBS, 1) k_bfs_all(const int32_t *rp, const 
             // others wait for twice the bound, which leaves the last level the whole of it
             if (blockIdx.x == 0) {
                 int32_t h = (int32_t)head, t = (int32_t)tail, l = lev;
+                int64_t cur = cursor;  // all vertices below are reached
                 const long long c0 = clock64();
-                if (threadIdx.x == 0) s_late = 0;
-                __syncthreads();
-                for (int it = 0; it < kBfsAlone && !s_late && t > h && t - h <= kBfsNarrow; ++it) {
-                    if (threadIdx.x == 0) s_tail = t;
+                bool late = false;
+                for (int it = 0; it < kBfsAlone && !late && t - h <= kBfsNarrow; ++it) {
+                    if (t == h) {  // ran dry: the smallest untouched vertex, if it is near
+                        if (t >= n) break;
+                        if (threadIdx.x == 0) s_root = INT_MAX;
+                        bool any = false;
+                        for (int c = 0; c < kBfsNear && cur < n && !any; ++c, cur += any ? 0 : kBfsBS) {
+                            const int64_t i = cur + threadIdx.x;
+                            const bool free = i < n && *(volatile int32_t *)&level_of[i] < 0;
+                            any = __syncthreads_or(free);
+                            if (free) atomicMin(&s_root, (int)i);
+                        }
+                        if (!any) break;
+                        __syncthreads();
+                        cur = s_root;
+                        ++l;
+                        if (threadIdx.x == 0) {
+                            level_of[cur] = l;
+                            queue[t] = make_int4((int)cur, rp[cur], rp[cur + 1], 0);
+                        }
+                        ++t;
+                    }
+                    if (threadIdx.x == 0) s_end.x = t;
                     __syncthreads();
-                    expand(h + threadIdx.x, blockDim.x, t, l + 1, &s_tail);
-                    if (threadIdx.x == 0) s_late = clock64() - c0 > limit_ns / kBfsAloneShare;
+                    expand(h + threadIdx.x, blockDim.x, t, l + 1, &s_end.x);
+                    // (by the last thread, whose warp has the least to do)
+                    if (threadIdx.x == kBfsBS - 1) s_end.y = clock64() - c0 > limit_ns / kBfsAloneShare;
                     __syncthreads();
                     h = t;
-                    t = s_tail;
+                    const int2 end = s_end;
+                    t = end.x;
+                    late = end.y != 0;
                     if (t > h) ++l;
                     __syncthreads();
                 }
                 if (threadIdx.x == 0) {
                     st->tail = t;
-                    st->left[(round + 1) & 1] = make_int4(h, t, l, 0);
+                    st->left[(round + 1) & 1] = make_int4(h, t, l, (int32_t)min(cur, (int64_t)n));
                 }
             }
             if (bfs_grid_barrier(st, ++round, &s_found, 2 * limit_ns) < 0) return;
@@ -252,6 +282,7 @@ __global__ void __launch_bounds__(kBfsBS, 1) k_bfs_all(const int32_t *rp, const 
             head = left->x;
             tail = left->y;
             lev = left->z;
+            cursor = left->w;
             continue;
         }
         if (tail > head) {  // expand level lev (st->tail == tail)

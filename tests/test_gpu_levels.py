@@ -1,7 +1,10 @@
 """The level search (one cooperative launch) on graphs that are hard on its schedule: narrow levels
-of much work, which one block expands alone while the others wait for it."""
+of much work, which one block expands alone while the others wait for it, and many components."""
 import numpy as np
 import pytest
+
+import gen
+import oracle
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -53,3 +56,38 @@ def test_narrow_levels_of_long_rows(mpk):
     want[-1] = A.n
     assert np.array_equal(ptr, want)
     assert torch.equal(L.perm, torch.arange(A.n, dtype=torch.int32, device="cuda"))
+
+
+def _components(kind, n):
+    """Edges of a graph of n vertices with many components."""
+    i = np.arange(n)
+    if kind == "isolated":
+        return i[:0], i[:0]
+    if kind == "far":  # one component of every vertex but 7, which lie 8191, 8192, 8193 .. apart
+        skip = np.cumsum([100, 8191, 8192, 8193, 2, 9000, 1])
+        v = np.setdiff1d(i, skip)
+        return v[:-1], v[1:]
+    if kind == "stars":  # wide levels (700 leaves) between narrow ones, then vertices without edges
+        hub = i // 701 * 701
+        on = (i != hub) & (i < n - 3000)
+        return hub[on], i[on]
+    return i[:-1][i[:-1] % 3 > 0], i[1:][i[:-1] % 3 > 0]  # "paths" of three vertices
+
+
+@pytest.mark.parametrize("symmetric", [True, False])
+@pytest.mark.parametrize("kind,n", [("isolated", 1), ("isolated", 1500), ("far", 45000), ("stars", 20000), ("paths", 5000)])
+def test_many_components(mpk, kind, n, symmetric):
+    """The search goes on from the smallest untouched vertex, near (found beside the narrow levels)
+    or far (found by the whole grid), from the first vertex and from one in the middle."""
+    r, c = _components(kind, n)
+    if symmetric:
+        r, c = np.concatenate([r, c]), np.concatenate([c, r])
+    A = gen.from_coo(n, r, c, np.ones(r.size))
+    dA = mpk.CsrMatrix.from_host(A, is_symmetric=symmetric)
+    for root in (0, n // 2):
+        L = mpk.build_levels(dA, root=root)
+        lo, pe, ip, lp = oracle.levels(A, root)
+        assert L.num_levels == lp.size - 1
+        assert np.array_equal(L.level_ptr.cpu().numpy(), lp)
+        assert np.array_equal(L.perm.cpu().numpy(), pe)
+        assert np.array_equal(L.level_of.cpu().numpy(), lo)

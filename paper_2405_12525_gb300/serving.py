@@ -54,6 +54,10 @@ class _Waiting:
     req: Request = field(compare=False)
 
 
+class PlanTooLarge(Exception):
+    """A backend's plan does not fit the room the server gave it."""
+
+
 class Server:
     """Continuous admission under a device-memory budget (bytes), at most `max_inflight`
     requests in flight.  `backend` provides the device work (see GpuBackend).  keep_results:
@@ -70,21 +74,66 @@ class Server:
         self.inflight = []           # (request, handle, plan_key, plan, bytes)
         self.free_plans: dict = {}   # plan key -> list of idle plans
         self.plan_bytes: dict = {}   # id(plan) -> bytes
+        self.least: dict = {}        # plan key -> bytes, where a plan did not fit its estimate
         self.done: list[Request] = []
         self.rejected: list[Request] = []  # could never fit the budget
         self.max_seen_inflight = 0
 
     # ------------------------------------------------------------------ plans
+    def _drop(self, key, plan):
+        self.free_plans[key].remove(plan)
+        self.used -= self.plan_bytes.pop(id(plan))
+        self.backend.drop_plan(plan)
+
+    def _idle(self, keys):
+        """(bytes, key, plan) of the idle plans of `keys`, largest first."""
+        idle = [(self.plan_bytes[id(p)], key, p) for key in keys for p in self.free_plans.get(key, [])]
+        return sorted(idle, key=lambda t: -t[0])
+
     def _evict(self, need: int, keep):
         """Free idle plans of other keys (largest first) until `need` more bytes fit."""
-        idle = [(self.plan_bytes[id(p)], key, p) for key, ps in self.free_plans.items() if key != keep for p in ps]
-        for nbytes, key, p in sorted(idle, key=lambda t: -t[0]):
+        for _, key, p in self._idle([k for k in self.free_plans if k != keep]):
             if self.used + need <= self.budget:
                 break
-            self.free_plans[key].remove(p)
-            self.used -= nbytes
-            del self.plan_bytes[id(p)]
-            self.backend.drop_plan(p)
+            self._drop(key, p)
+
+    def _evict_own(self, key, buf: int):
+        """Free idle plans of the request's own key (largest first) while its buffers do not fit beside
+        them; the last one only when a plan of the size the key needs fits in its place (an idle plan
+        may hold more than that)."""
+        own = self._idle([key])
+        while own and self.used + buf > self.budget:
+            nbytes, _, p = own.pop(0)
+            if not own and self.used - nbytes + buf + self._plan_need(key) > self.budget:
+                break
+            self._drop(key, p)
+
+    def _plan_need(self, key) -> int:
+        """Bytes a plan of the key needs, as far as known."""
+        return max(self.backend.plan_bytes(key), self.least.get(key, 0))
+
+    def _new_plan(self, key, buf: int):
+        """A plan beside `buf` bytes of buffers, or None when it has to wait for requests in flight.
+        A plan takes more than it needs (for its optional copies of the matrix) only from its share of
+        what is left, among the requests that may still join, or up to a quarter where another request
+        like this one still fits.  A plan that
+        cannot be built in what is left waits; alone on the device it gets what it takes."""
+        while True:
+            room = self.budget - self.used - buf
+            need = self._plan_need(key)
+            share = room // max(1, self.max_inflight - len(self.inflight))
+            limit = need + max(0, share - need, min(need // 4, room - 2 * need - buf))
+            if limit > room:
+                self._evict(buf + need, keep=None)
+                room = self.budget - self.used - buf
+                if need > room and self.inflight:
+                    return None
+                limit = need
+            self.backend.room = limit
+            try:
+                return self.backend.make_plan(key)
+            except PlanTooLarge:
+                self.least[key] = limit + max(1, limit // 8)
 
     # ------------------------------------------------------------------ requests
     def submit(self, req: Request):
@@ -93,7 +142,8 @@ class Server:
     def _admit(self, now: float):
         """Admit waiting requests in arrival order; one that does not fit yet does not block
         later, smaller ones.  A request needs its buffers and, unless an idle plan of its key
-        exists, a new plan; idle plans of other keys are freed to make room."""
+        exists, a new plan; idle plans of other keys are freed to make room, and those of its own key
+        that are larger than what it needs.  A request waits for others in flight only: alone it runs."""
         kept = []
         while self.waiting and len(self.inflight) < self.max_inflight:
             w = heapq.heappop(self.waiting)
@@ -101,21 +151,26 @@ class Server:
             key = self.backend.plan_key(req)
             buf = self.backend.request_bytes(req)
             idle = self.free_plans.get(key)
-            plan_need = 0 if idle else self.backend.plan_bytes(key)
+            plan_need = 0 if idle else self._plan_need(key)
             if buf + self.backend.plan_bytes(key) > self.budget:  # not even on an empty device
                 req.t_done = now
                 self.rejected.append(req)
                 continue
             if self.used + buf + plan_need > self.budget:
                 self._evict(buf + plan_need, keep=key)
-            if self.used + buf + plan_need > self.budget:
+            if idle and self.used + buf > self.budget:
+                self._evict_own(key, buf)
+                plan_need = 0 if idle else self._plan_need(key)
+            if self.used + buf + plan_need > self.budget and self.inflight:
                 kept.append(w)
                 continue
             if idle:
                 plan = idle.pop()
             else:
-                self.backend.room = self.budget - self.used - buf  # a plan may take more than its estimate
-                plan = self.backend.make_plan(key)
+                plan = self._new_plan(key, buf)
+                if plan is None:
+                    kept.append(w)
+                    continue
                 nbytes = self.backend.actual_plan_bytes(plan, plan_need)
                 self.plan_bytes[id(plan)] = nbytes
                 self.used += nbytes
@@ -188,6 +243,8 @@ class GpuBackend:
     """Device work through the library: plans per (matrix, kind, width), one stream and one
     event per request; vectors in the matrix's own numbering."""
 
+    room = None  # bytes the next plan may take (None: no limit), set by the server
+
     def __init__(self, matrices: dict, p_max: int = 16, cheb_block: int = 8, streams: int = 8,
                  shape: int = SERVING_SHAPE):
         import torch
@@ -216,21 +273,23 @@ class GpuBackend:
         return int(plan.describe()["device_bytes"])
 
     def make_plan(self, key):
-        """A plan within the room the server has left, if it gave one (a plan that has room keeps
-        its matrix in the request's numbering too)."""
+        """A plan within the room the server gave (a plan that has room keeps its matrix in the
+        request's numbering too); PlanTooLarge when it cannot be built in that."""
         from . import MPK_ERR_BUDGET, MPK_ERR_OOM, ORDER_ORIGINAL, MpkError, plan
         A = self.mats[key[0]][0]
-        try:
-            return plan(A, self.levels[key[0]], p_max=self._plan_p(key), nrhs=key[2], order=ORDER_ORIGINAL,
-                        shape=self.shape, mem_budget=max(0, int(getattr(self, "room", 0))))
-        except MpkError as e:
-            if e.status not in (MPK_ERR_OOM, MPK_ERR_BUDGET):
-                raise
-            # freed request buffers may still sit in torch's allocator cache: return them
-            self.torch.cuda.synchronize()
-            self.torch.cuda.empty_cache()
-            return plan(A, self.levels[key[0]], p_max=self._plan_p(key), nrhs=key[2], order=ORDER_ORIGINAL,
-                        shape=self.shape)
+        limit = 0 if self.room is None else max(1, int(self.room))  # (mem_budget 0: no limit)
+        for retry in (False, True):
+            try:
+                return plan(A, self.levels[key[0]], p_max=self._plan_p(key), nrhs=key[2], order=ORDER_ORIGINAL,
+                            shape=self.shape, mem_budget=limit)
+            except MpkError as e:
+                if e.status == MPK_ERR_BUDGET:
+                    raise PlanTooLarge(f"{key}: more than {limit} bytes") from e
+                if retry or e.status != MPK_ERR_OOM:
+                    raise
+                # freed request buffers may still sit in torch's allocator cache: return them
+                self.torch.cuda.synchronize()
+                self.torch.cuda.empty_cache()
 
     def drop_plan(self, plan):
         del plan

@@ -146,3 +146,107 @@ def test_results_kept_for_all_none_or_selected_requests(keep, kept):
     assert len(done) == 12
     assert {r.rid for r in done if r.result is not None} == kept
     assert all(r.result == ("result", r.rid) for r in done if r.result is not None)
+
+
+class Deadline(Clock):
+    """A clock that fails a loop which makes no progress."""
+
+    def sleep(self, dt):
+        super().sleep(dt)
+        assert self.t < 60.0, "the server makes no progress"
+
+
+class GrowingBackend(FakeBackend):
+    """Plans need `least` bytes (which may be above the estimate) and take up to `most` where the
+    server leaves them room."""
+
+    def __init__(self, clock, least=100, most=180, **kw):
+        super().__init__(clock, **kw)
+        self.least, self.most = least, most
+        self.room = None
+
+    def make_plan(self, key):
+        from paper_2405_12525_gb300.serving import PlanTooLarge
+        room = self.most if self.room is None else self.room
+        assert room > 0
+        if room < self.least:
+            raise PlanTooLarge(str(key))
+        return {**super().make_plan(key), "bytes": min(room, self.most)}
+
+    def actual_plan_bytes(self, plan, estimate):
+        return plan["bytes"]
+
+    def request_bytes(self, req):
+        return self.buf_per_order * req.order
+
+
+def _run(be, clk, budget, reqs, max_inflight=8):
+    srv = Server(be, hbm_budget=budget, max_inflight=max_inflight)
+    srv.run(reqs, clock=clk, sleep=clk.sleep)
+    return srv
+
+
+@pytest.mark.parametrize("second", [2, 5, 9])
+def test_an_enlarged_idle_plan_gives_way_to_larger_buffers(second):
+    """The first request's plan takes more than its estimate; a later one of the same key whose buffers
+    do not fit beside it is served by a smaller plan."""
+    clk = Deadline()
+    be = GrowingBackend(clk)
+    srv = _run(be, clk, 200, [Request(0, 0.0, "a", "mpk", 1, 1), Request(1, 0.5, "a", "mpk", second, 1)], 1)
+    assert [r.rid for r in srv.done] == [0, 1] and not srv.rejected
+    assert srv.peak_used <= 200
+
+
+def test_a_plan_leaves_the_room_of_requests_that_may_join():
+    clk = Deadline()
+    be = GrowingBackend(clk, most=400, duration=0.1)
+    srv = _run(be, clk, 400, [Request(0, 0.0, "a", "mpk", 1, 1), Request(1, 0.0, "b", "mpk", 1, 1)], 2)
+    assert len(srv.done) == 2 and srv.max_seen_inflight == 2 and srv.peak_used <= 400
+
+
+@pytest.mark.parametrize("least", [101, 130, 170])
+def test_plans_above_the_estimate_wait_for_room(least):
+    """Plans that cannot be built in what is left wait for requests in flight, idle plans are freed for
+    them, and the budget holds."""
+    clk = Deadline()
+    be = GrowingBackend(clk, least=least, most=2 * least, duration=0.05)
+    srv = _run(be, clk, 360, [Request(i, 0.001 * i, "abc"[i % 3], "mpk", 1 + i % 4, 1) for i in range(24)], 4)
+    assert len(srv.done) == 24 and not srv.rejected and srv.peak_used <= 360
+
+
+def test_a_plan_above_the_whole_budget_runs_alone_with_what_it_needs():
+    clk = Deadline()
+    be = GrowingBackend(clk, least=230, most=1000, duration=0.05)
+    reqs = [Request(i, 0.0, "ab"[i % 2], "mpk", 1 + 4 * (i % 3), 1) for i in range(6)]
+    srv = _run(be, clk, 200, reqs, 4)
+    assert len(srv.done) == 6 and not srv.rejected
+    assert srv.max_seen_inflight == 1
+    assert srv.peak_used <= 230 * 1.25 + 90  # not the optional parts
+
+
+@pytest.mark.parametrize("room", [None, 0, 1, 5000])
+def test_a_plan_has_no_budget_only_when_the_server_gave_no_room(monkeypatch, room):
+    """mem_budget 0 means no limit: a room of 0 must not become one, and a plan that fails for its
+    budget is not built without one."""
+    import paper_2405_12525_gb300 as mpk
+    from paper_2405_12525_gb300.serving import GpuBackend, PlanTooLarge
+    asked = []
+
+    def plan(A, L, **kw):
+        asked.append(kw["mem_budget"])
+        if kw["mem_budget"] == 1:
+            raise mpk.MpkError(mpk.MPK_ERR_BUDGET, "too large")
+        return "plan"
+
+    monkeypatch.setattr(mpk, "plan", plan)
+    be = object.__new__(GpuBackend)
+    be.mats, be.levels = {"a": (None, 1.0, 0.0)}, {"a": None}
+    be.p_max, be.cheb_block, be.shape = 8, 8, 3
+    if room is not None:
+        be.room = room
+    if room in (0, 1):
+        with pytest.raises(PlanTooLarge):
+            be.make_plan(("a", "mpk", 1))
+        assert asked == [1]
+    else:
+        assert be.make_plan(("a", "mpk", 1)) == "plan" and asked == [room or 0]

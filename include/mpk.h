@@ -399,9 +399,11 @@ mpk_status mpk_sync_status(const mpk_plan_t *P, mpk_stream stream);
 
 /* Fault injection for tests of the failure path (no counterpart in the paper): in the next
  * level-blocked launch on this plan, work unit (chunk, k) computes its rows but does not
- * publish its completion flag.  Units that read those rows wait until the plan's
- * wait_limit_ns expires, record MPK_ERR_TIMEOUT and leave; every wait stays bounded and
- * the device stays usable.  mpk_sync_status then reports MPK_ERR_TIMEOUT. */
+ * publish its completion; where the launch has a cell's counters in place of the chunks'
+ * flags (see mpk_apply), it is power k of the cell with that number, or of the last one.
+ * Whatever reads those rows waits until the plan's wait_limit_ns expires, records
+ * MPK_ERR_TIMEOUT and leaves; every wait stays bounded and the device stays usable.
+ * mpk_sync_status then reports MPK_ERR_TIMEOUT.  (Nothing reads the launch's last power.) */
 mpk_status mpk_debug_drop_release(mpk_plan_t *P, int32_t chunk, int32_t k);
 
 /* ---------------------------------------------------------------------------------------

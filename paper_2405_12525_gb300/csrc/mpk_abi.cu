@@ -159,11 +159,12 @@ void mpk::wave_args(const WaveSet &w, int32_t p, KArgs &a) {
     a.v_count = w.count;
     a.v_ngroups = w.ngroups;
     a.v_maxsl = w.maxsl;
+    a.v_drop = a.drop_unit < 0 ? -1 : std::min(a.drop_unit >> 5, w.ngroups - 1) << 5 | (a.drop_unit & 31);
     a.stream_last = w.ngroups > 1;  // a matrix of one group stays in L2 between launches
 }
 
 // The launch can run in A's own numbering: vectors as the caller has them, no pass before or after.
-static bool runs_natural(const Plan &P) { return P.natural.ok && P.drop_unit < 0; }
+static bool runs_natural(const Plan &P) { return P.natural.ok; }
 
 KArgs mpk::base_args(Plan &P, int32_t p) {
     KArgs a;

@@ -127,7 +127,7 @@ extern "C" mpk_status mpk_batch_apply(const mpk_plan_t *Ph, const double *const 
     // for the copies of the powers in the workspace); it needs the matrix in the numbering of the vectors, and an output for
     // every block.
     const WaveSet &w = plan_order ? P.wave : P.natural;
-    bool direct = w.ok && P.drop_unit < 0;
+    bool direct = w.ok;
     for (int32_t i = 0; i < count && direct; ++i) {
         const int64_t ni = (int64_t)(P.inst_row[i + 1] - P.inst_row[i]) * m;
         if (ni == 0) continue;

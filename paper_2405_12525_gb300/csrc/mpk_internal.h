@@ -306,6 +306,7 @@ struct KArgs {
     int32_t *v_count;          // (p + 1) x v_ngroups
     int32_t v_ncells, v_ngroups;
     int32_t v_maxsl;           // slices of the largest group
+    int32_t v_drop;            // test hook: this cell (g << 5 | k) is never counted as finished, -1 = none
     // 1: what the launch's last power reads and writes is the first to leave L2 (the matrix does not
     // stay there between launches)
     int32_t stream_last;

@@ -530,7 +530,7 @@ void launch_wave_batch(const Plan &P, KArgs &a, WaveBatch &inst, cudaStream_t s)
 
 void launch_mpk(const Plan &P, KArgs &a, int mode, cudaStream_t s) {
     const bool a32 = P.accum == MPK_F32;
-    if (a.v_cell != nullptr && a.drop_unit < 0) {
+    if (a.v_cell != nullptr) {
         const int grid = std::min(device_sms(), a.v_maxsl);
         int smem = 0;
         void *fn = select_wave(mode, P.m, P.val_type, a.v_dict != nullptr, a32, &smem);

@@ -431,7 +431,7 @@ __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst)
                     if (__any_sync(0xffffffffu, now)) {
                         __syncwarp();         // every lane's view of the progress words
                         fence_acq_rel_gpu();  // acquires the finished slices' rows, releases them
-                        if (now)
+                        if (now && ce.z != a.v_drop)
                             atomicAdd(a.v_count + (int64_t)k * a.v_ngroups + (ce.z >> 5), size);
                         todo = todo && !now;
                         w0 = Deadline();

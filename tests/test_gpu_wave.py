@@ -264,3 +264,72 @@ def test_batch_outputs_that_share_memory(mpk, order, m):
         assert np.array_equal(got.view(np.uint64), np.ascontiguousarray(last[1:]).view(np.uint64))
         for V, w, q in zip(B.views(), want, perms):
             assert np.array_equal(V.cpu().numpy().view(np.uint64), np.ascontiguousarray(w[:, q]).view(np.uint64))
+
+
+def _expires(mpk, P, run):
+    """`run` fails with the timeout status; the next `run` succeeds and returns its outputs."""
+    run()
+    with pytest.raises(mpk.MpkError) as e:
+        P.sync_status()
+    assert e.value.status == 4
+    out = run()
+    P.sync_status()
+    return out
+
+
+@pytest.mark.parametrize("order", [0, 1])
+@pytest.mark.parametrize("kind", ["one group", "groups", "packed", "sorted rows", "blocks", "staged far"])
+def test_a_wait_that_expires(mpk, kind, order):
+    """A cell that is never counted as finished: the cells that read it give up after the plan's limit
+    with MPK_ERR_TIMEOUT, blocks leave with no copy in flight, and the next launches, of other numbers
+    of powers too, find clean counters."""
+    A = {"sorted rows": lambda: _widths_matrix(1501, (1, 30, 4, 17, 0, 9, 2), 930),
+         "staged far": lambda: gen.laplacian_3d(60, 50, 40)}.get(kind, lambda: gen.laplacian_3d(19, 17, 23))()
+    m = 4 if kind == "blocks" else 1
+    if kind != "packed":  # (a Laplacian's two values are packed where the matrix is larger than the cache)
+        A = A.with_values(gen.uniform(gen.derive_seed(970), A.nnz))
+    dA = mpk.CsrMatrix.from_host(A)
+    L = mpk.build_levels(dA, 0)
+    P = mpk.plan(dA, L, p_max=6, nrhs=m, order=order, wait_limit_ns=20_000_000,
+                 cache_bytes={"one group": 0, "staged far": 400000}.get(kind, 40000))
+    X = gen.vector(A.n, m, stream=91)
+    perm = L.perm.cpu().numpy() if order == mpk.ORDER_PLAN else np.arange(A.n)
+    Xd = torch.from_numpy(np.ascontiguousarray(X[perm])).cuda()
+    want = np.ascontiguousarray(oracle.mpk(A, X, 6)[:, perm])
+    for chunk, k, p in ((0, 1, 6), (3, 2, 5), (10 ** 6, 4, 6)):
+        P.debug_drop_release(min(chunk, P.describe()["num_chunks"] - 1), k)
+        Y = _expires(mpk, P, lambda: P.apply(Xd, p))
+        assert np.array_equal(Y.cpu().numpy().view(np.uint64), want[:p + 1].view(np.uint64))
+    Y = P.apply(Xd, 2)
+    P.sync_status()
+    assert np.array_equal(Y.cpu().numpy().view(np.uint64), want[:3].view(np.uint64))
+    c = np.linspace(1.0, -0.5, 8)
+    P.debug_drop_release(0, 1)
+    out = _expires(mpk, P, lambda: P.cheb_filter(Xd, 7, c, scale=9.0, shift=0.3)).cpu().numpy()
+    ref = oracle.cheb(A, X, 7, c, scale=9.0, shift=0.3)[perm]
+    assert np.array_equal(out.view(np.uint64), np.ascontiguousarray(ref).view(np.uint64))
+
+
+@pytest.mark.parametrize("order", [0, 1])
+def test_a_wait_that_expires_in_a_batch(mpk, order):
+    mats = [gen.laplacian_3d(9, 8, 7), gen.laplacian_2d(40, 31), gen.laplacian_3d(15, 14, 13)]
+    ps = [5, 4, 6]
+    dAs = [mpk.CsrMatrix.from_host(A) for A in mats]
+    B = mpk.batch_plan(dAs, ps, nrhs=1, order=order, cache_bytes=30000, wait_limit_ns=20_000_000)
+    perms = [mpk.build_levels(d, 0).perm.cpu().numpy() if order == mpk.ORDER_PLAN else np.arange(d.n) for d in dAs]
+    Xh = [gen.vector(A.n, 1, stream=60 + i) for i, A in enumerate(mats)]
+    Xs = [torch.from_numpy(np.ascontiguousarray(X[q])).cuda() for X, q in zip(Xh, perms)]
+    want = [np.ascontiguousarray(oracle.mpk(A, X, p)[:, q]) for A, X, p, q in zip(mats, Xh, ps, perms)]
+    lib, status = mpk.load(), lambda: mpk._check(lib.mpk_sync_status(B._h, None))
+    for in_place in (False, True):
+        mpk._check(lib.mpk_debug_drop_release(B._h, 1, 2))
+        B.apply(Xs, in_place=in_place)
+        torch.cuda.synchronize()
+        with pytest.raises(mpk.MpkError) as e:
+            status()
+        assert e.value.status == 4
+        Ys = B.apply(Xs)
+        torch.cuda.synchronize()
+        status()
+        for Y, w in zip(Ys, want):
+            assert np.array_equal(Y.cpu().numpy().view(np.uint64), w.view(np.uint64))

@@ -159,6 +159,7 @@ void mpk::wave_args(const WaveSet &w, int32_t p, KArgs &a) {
     a.v_count = w.count;
     a.v_ngroups = w.ngroups;
     a.v_maxsl = w.maxsl;
+    a.v_scattered = w.scattered ? 1 : 0;
     a.v_drop = a.drop_unit < 0 ? -1 : std::min(a.drop_unit >> 5, w.ngroups - 1) << 5 | (a.drop_unit & 31);
     a.stream_last = w.ngroups > 1;  // a matrix of one group stays in L2 between launches
 }

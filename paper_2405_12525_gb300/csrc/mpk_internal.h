@@ -306,6 +306,8 @@ struct KArgs {
     int32_t *v_count;          // (p + 1) x v_ngroups
     int32_t v_ncells, v_ngroups;
     int32_t v_maxsl;           // slices of the largest group
+    int32_t v_scattered;       // 1: the smaller entry buffer (see WaveSet)
+    int32_t v_cap;             // entries of the buffer (set by the launch)
     int32_t v_drop;            // test hook: this cell (g << 5 | k) is never counted as finished, -1 = none
     // 1: what the launch's last power reads and writes is the first to leave L2 (the matrix does not
     // stay there between launches)
@@ -339,6 +341,8 @@ struct WaveBatch {
 // Tables of the wave kernel over one sliced copy of the matrix (device memory of the plan)
 struct WaveSet {
     bool ok = false;
+    // the gathers of x touch about a line a row, and more of x than L1 holds beside the large buffer
+    bool scattered = false;
     const void *val = nullptr;
     const int32_t *col = nullptr;
     const double *dict = nullptr;     // packed copy: its table of values (val is the stream)

@@ -504,17 +504,21 @@ static int occupancy_grid_w(int mode, int m, int vtype) {
     return c;
 }
 
-// The wave kernel for (mode, width, value type, accumulator), ready to launch, and its shared memory
-static void *select_wave(int mode, int m, int vtype, bool packed, bool a32, int *smem) {
+// The wave kernel for (mode, width, value type, accumulator), ready to launch: its buffer's entries (in the
+// arguments) and shared memory
+static void *select_wave(int mode, int m, int vtype, bool packed, bool a32, KArgs &a, int *smem) {
     static bool ready[4][4][5][2] = {};  // packed copies: value type 3; width index: log2 of m
     if (vtype < 0 || vtype > 2 || mode < 0 || mode > kWaveBatchMode) fail(MPK_ERR_UNSUPPORTED, "value type %d, mode %d", vtype, mode);
-    void *fn = packed             ? select_wave_dict(mode, m, a32, smem)
-               : vtype == MPK_F64 ? select_wave_f64(mode, m, a32, smem)
-               : vtype == MPK_F32 ? select_wave_f32(mode, m, a32, smem)
-                                  : select_wave_bf16(mode, m, a32, smem);
+    WaveSize size{};
+    void *fn = packed             ? select_wave_dict(mode, m, a32, &size)
+               : vtype == MPK_F64 ? select_wave_f64(mode, m, a32, &size)
+               : vtype == MPK_F32 ? select_wave_f32(mode, m, a32, &size)
+                                  : select_wave_bf16(mode, m, a32, &size);
+    a.v_cap = size.cap[a.v_scattered];
+    *smem = size.smem(a.v_scattered != 0);
     bool &r = ready[packed ? 3 : vtype][mode][__builtin_ctz((unsigned)m)][a32 ? 1 : 0];
     if (!r) {
-        MPK_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, *smem));
+        MPK_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, size.smem(false)));
         r = true;
     }
     return fn;
@@ -522,7 +526,7 @@ static void *select_wave(int mode, int m, int vtype, bool packed, bool a32, int 
 
 void launch_wave_batch(const Plan &P, KArgs &a, WaveBatch &inst, cudaStream_t s) {
     int smem = 0;
-    void *fn = select_wave(kWaveBatchMode, P.m, P.val_type, false, false, &smem);
+    void *fn = select_wave(kWaveBatchMode, P.m, P.val_type, false, false, a, &smem);
     const int grid = std::min(device_sms(), a.v_maxsl);
     void *args[] = {&a, &inst};
     MPK_CUDA(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kWaveBS), args, (size_t)smem, s));
@@ -533,7 +537,7 @@ void launch_mpk(const Plan &P, KArgs &a, int mode, cudaStream_t s) {
     if (a.v_cell != nullptr) {
         const int grid = std::min(device_sms(), a.v_maxsl);
         int smem = 0;
-        void *fn = select_wave(mode, P.m, P.val_type, a.v_dict != nullptr, a32, &smem);
+        void *fn = select_wave(mode, P.m, P.val_type, a.v_dict != nullptr, a32, a, &smem);
         void *args[] = {&a};
         MPK_CUDA(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kWaveBS), args, (size_t)smem, s));
         return;

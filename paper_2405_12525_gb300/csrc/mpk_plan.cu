@@ -594,6 +594,137 @@ __global__ void k_pack_fill(int32_t nslices, R rows, const T *va, const int32_t 
     }
 }
 
+// How the gathers of x spread, from samples of up to 2048 rows (64 slices; of fewer when they hold over
+// 64 K entries): `lines` / `rows`, the 128-byte lines that a gather of one entry of a unit's rows touches,
+// per row, and `bytes`, those of the different 32-byte sectors that a sample's entries read (counted in
+// a bitmap of hashes, by the bits left free).
+struct GatherSpread {
+    unsigned long long lines, rows;
+    float bytes;  // of all samples
+};
+constexpr int kSpreadSlices = 64, kSpreadEntries = 1 << 16, kSpreadSamples = 64, kSpreadBits = 1 << 18;
+// rows of A (32 consecutive ones a slice)
+struct CsrSlices {
+    const int32_t *rp, *ci;
+    int32_t n;
+    // calls f with the columns of the slice's first entries (-1: a row has fewer), four at a time
+    template <class F> __device__ __forceinline__ void visit(int64_t s, int most, int lane, F f) const {
+        const int64_t r = 32 * s + lane;
+        const int32_t e0 = r < n ? rp[r] : 0, len = r < n ? rp[r + 1] - e0 : 0;
+        const int w = min(__reduce_max_sync(0xffffffffu, len), most);
+        for (int j = 0; j < w; j += 4) {
+            int32_t c[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) c[t] = j + t < len ? ci[e0 + j + t] : -1;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) f(c[t]);
+        }
+    }
+};
+// slices of the plan's copy
+struct PlanSlices {
+    const int64_t *sptr;
+    const int32_t *col;
+    template <class F> __device__ __forceinline__ void visit(int64_t s, int most, int lane, F f) const {
+        const int64_t e0 = sptr[s];
+        const int w = min((int)((sptr[s + 1] - e0) >> 5), most);
+        for (int j = 0; j < w; j += 4) {
+            int32_t c[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) c[t] = j + t < w ? col[e0 + 32 * (int64_t)(j + t) + lane] : -1;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) f(c[t]);
+        }
+    }
+};
+// Sample `block` of `blocks`, of `per` slices; xbytes: of a row of x (all its columns)
+template <class R>
+__device__ __forceinline__ void spread_sample(int64_t nslices, int per, const R &rows, int m, int xbytes, int block, int blocks,
+                                              GatherSpread *out) {
+    __shared__ uint32_t seen[kSpreadBits / 32];
+    __shared__ int s_lines, s_rows, s_set;
+    for (int i = threadIdx.x; i < kSpreadBits / 32; i += blockDim.x) seen[i] = 0;
+    if (threadIdx.x == 0) s_lines = s_rows = s_set = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, sector = max(32, xbytes);
+    const int64_t s0 = blocks > 1 ? (nslices - per) * block / (blocks - 1) : 0;
+    int lines = 0, taken = 0;
+    for (int q = threadIdx.x >> 5; q < per && s0 + q < nslices; q += blockDim.x >> 5) {
+        rows.visit(s0 + q, kSpreadEntries / 32, lane, [&](int32_t c) {
+            const unsigned int on = __ballot_sync(0xffffffffu, c >= 0);
+            bool first = false;
+            if (c >= 0) {  // (a unit: 32 / m rows)
+                const unsigned long long at = (unsigned long long)c * xbytes;
+                first = lane == __ffs(__match_any_sync(on, (uint32_t)(at >> 7) << 5 | (unsigned)(lane * m >> 5))) - 1;
+                const uint32_t h = ((uint32_t)(at / sector) * 0x9e3779b1u) >> 14;  // (18 bits: kSpreadBits)
+                if (!((*(volatile uint32_t *)&seen[h >> 5] >> (h & 31)) & 1u)) atomicOr(&seen[h >> 5], 1u << (h & 31));
+            }
+            lines += __popc(__ballot_sync(0xffffffffu, first));
+            taken += __popc(on);
+        });
+    }
+    if (lane == 0) {
+        atomicAdd(&s_lines, lines);
+        atomicAdd(&s_rows, taken);
+    }
+    __syncthreads();
+    int set = 0;
+    for (int i = threadIdx.x; i < kSpreadBits / 32; i += blockDim.x) set += __popc(seen[i]);
+    set = __reduce_add_sync(0xffffffffu, set);
+    if (lane == 0) atomicAdd(&s_set, set);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        atomicAdd(&out->lines, (unsigned long long)s_lines);
+        atomicAdd(&out->rows, (unsigned long long)s_rows);
+        const float clear = fmaxf(1.0f, (float)(kSpreadBits - s_set)) / kSpreadBits;  // linear counting
+        atomicAdd(&out->bytes, -logf(clear) * (float)kSpreadBits * (float)sector);
+    }
+}
+// samples in A's numbering into out[0], then of the plan's slices into out[1]
+__global__ void __launch_bounds__(1024) k_gather_spread(int nat_samples, int64_t nat_slices, CsrSlices nat, int64_t nslices,
+                                                        PlanSlices plan, int per, int m, int xbytes, GatherSpread *out) {
+    if ((int)blockIdx.x < nat_samples)
+        spread_sample(nat_slices, per, nat, m, xbytes, blockIdx.x, nat_samples, out);
+    else
+        spread_sample(nslices, per, plan, m, xbytes, blockIdx.x - nat_samples, gridDim.x - nat_samples, out + 1);
+}
+
+// The spread of an order, per row and sample: lines a row, bytes of a sample, and those as a part of the
+// bytes that its entries gather.
+struct Spread {
+    double lines = 0.0, bytes = 0.0, fresh = 0.0;
+    // Whether the wave kernel takes its smaller buffer (its figures beside kWaveBytes): gathers that touch
+    // about a line a row, and read more than the L1 beside the large one holds, most of it for the first
+    // time.  Measured over grids, stencils, the spin chain and banded graphs, in order, permuted and shuffled
+    // in windows, 1 to 4 columns, p = 8, time at 200 KB over that at 96 KB: lines up to 0.6 a row: 0.59 to
+    // 1.0 (spin chain 0.25 lines: 0.58 to 0.74); above, up to 40 KB: 0.7 to 0.9 (banded graph of 100k rows, 31
+    // KB), and fresh up to 0.2: 0.8 to 1.04 (same, 2 columns, 62 KB, 0.13); the rest 1.0 to 2.9, but for
+    // 63^3 in windows of 1000 rows (69 KB, 0.6): 0.92.
+    bool scattered() const { return lines > 0.62 && bytes > 40e3 && fresh > 0.22; }
+};
+// in A's numbering (at[0], if asked for) and in plan order (at[1])
+static void gather_spread(const Plan &P, const mpk_csr *A, bool natural, Spread (&at)[2], cudaStream_t s) {
+    Tmp<GatherSpread> d(2, s);
+    MPK_CUDA(cudaMemsetAsync(d.p, 0, 2 * sizeof(GatherSpread), s));
+    const int per = (int)std::max<int64_t>(1, std::min<int64_t>(kSpreadSlices, kSpreadEntries / (32 * (P.nnz / P.n + 1))));
+    const int xbytes = (P.accum == MPK_F32 ? 4 : 8) * P.m;
+    auto samples = [&](int64_t nslices) { return (int)std::max<int64_t>(1, std::min<int64_t>(kSpreadSamples, nslices / per)); };
+    const int64_t ns = ((int64_t)P.n + 31) / 32;
+    const int nat = natural ? samples(ns) : 0, plan = samples(P.num_slices);
+    k_gather_spread<<<nat + plan, 1024, 0, s>>>(nat, ns, CsrSlices{A->row_ptr, A->col, P.n}, P.num_slices,
+                                                PlanSlices{P.slice_ptr, P.col}, per, P.m, xbytes, d.p);
+    MPK_LAUNCHED();
+    GatherSpread h[2];
+    MPK_CUDA(cudaMemcpyAsync(h, d.p, sizeof(h), cudaMemcpyDeviceToHost, s));
+    MPK_CUDA(cudaStreamSynchronize(s));
+    for (int q = 0; q < 2; ++q) {
+        const double rows = (double)std::max<unsigned long long>(h[q].rows, 1);
+        at[q].lines = (double)h[q].lines / rows;
+        at[q].bytes = (double)h[q].bytes / std::max(1, q ? plan : nat);
+        at[q].fresh = (double)h[q].bytes / (rows * xbytes);
+    }
+}
+
 // A run of groups whose powers are computed together: a whole plan, or an instance of a batch plan
 struct WaveRange {
     int32_t g0, g1;  // groups
@@ -867,6 +998,10 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
                       (P.val_type == MPK_F64 || (long_rows && (P.val_type == MPK_F32 || P.accum == MPK_F32)));
     const bool natural = !P.identity && P.order == MPK_ORDER_ORIGINAL &&
                          std::min<int64_t>(n, 2 * (int64_t)band + 32) * 8 * P.m <= device_l2_bytes() / 4;
+    // (not looked at where the large buffer is as good: 8 and 16 columns within 3 %, up to 32768 rows of
+    // one column the same)
+    Spread spread[2];
+    if (P.m <= 4 && (int64_t)n * P.m > 32768) gather_spread(P, A, natural, spread, s);
     std::unique_ptr<Tmp<Dict>> table;
     bool packed = false;
     if (pack) try {
@@ -932,6 +1067,7 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
             P.wave.col = P.col;
             P.wave.ok = true;
         }
+        P.wave.scattered = spread[1].scattered();
     }
     if (!natural) return;
     std::vector<int32_t> nrow;
@@ -960,6 +1096,7 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
     }
     nrow.push_back(n);
     spare(P, P.natural, [&]() { return wave_copy(P, P.natural, A, nullptr, nullptr, nrow, ranges, dict, host[1], s); });
+    P.natural.scattered = spread[0].scattered();
 }
 
 Plan *build_plan(const mpk_csr *A, const Levels *L, const mpk_plan_opts *o, cudaStream_t s,

@@ -67,16 +67,22 @@ constexpr int kWaveBS = 32 * (kWaveWarps + kWaveAux);
 constexpr int kDescRing = 512;  // slice descriptors in shared memory
 constexpr int kWaveTiles = 32;  // tiles in shared memory or in flight
 constexpr int kStagedWidth = 64;  // entries a row of the widest slice that the buffer takes
-// Entries of the circular buffer, of the widest slice it takes (a wider one is read from global
-// memory) and of a tile.  A slice that starts near the end of the buffer runs on past it, into
-// room for one slice.
+// The circular buffer: its bytes, and its entries `cap`, of which the widest slice it takes (a wider
+// one is read from global memory) and a tile are parts.  A slice that starts near the end of the
+// buffer runs on past it, into room for one slice.
+//
+// 200 KB let the copies run furthest ahead (96 KB: structured binary64 grids the same, others 5 to
+// 30 % slower), but leave 28 KB of L1, in whose lines the gathers in flight wait for L2.  Gathers that
+// touch a line a row then queue for lines: with 96 KB a grid of 126^3 with its rows shuffled, p = 8, plan
+// order, takes 409 in place of 889 us (binary64), 463 in place of 804 us (bfloat16; the ticketed kernel,
+// whose blocks stage less: 464).  A set of tables says which of the two its gathers need (WaveSet::scattered).
+constexpr int kWaveBytes = 200 * 1024, kWaveBytesScattered = 96 * 1024;
 template <class VT> struct WaveBuf {
     static constexpr int ENTRY = (int)sizeof(typename VT::T) + 4;
     static constexpr int SLICE = 32 * kStagedWidth;
-    static constexpr int CAP = (200 * 1024 / ENTRY - SLICE) / 256 * 256;
-    static constexpr int TILE = CAP / 3;
-    static constexpr int ALL = CAP + SLICE + 32 * kBatch;  // a batch may read past its slice
-    static_assert(TILE >= SLICE, "a slice fits a tile");
+    static constexpr int CAP = (kWaveBytes / ENTRY - SLICE) / 256 * 256;
+    static constexpr int CAP_SCATTERED = (kWaveBytesScattered / ENTRY - SLICE) / 256 * 256;
+    static_assert(CAP_SCATTERED / 3 >= SLICE, "a slice fits a tile");
 };
 
 // packed slices: positions and sizes count 16-byte units
@@ -86,10 +92,9 @@ struct ValDict {
 template <> struct WaveBuf<ValDict> {
     static constexpr int ENTRY = 16;
     static constexpr int SLICE = (kStagedWidth + 3) / 4 + 10 * kStagedWidth;
-    static constexpr int CAP = (200 * 1024 / ENTRY - SLICE) / 16 * 16;
-    static constexpr int TILE = CAP / 3;
-    static constexpr int ALL = CAP + SLICE;
-    static_assert(TILE >= SLICE, "a slice fits a tile");
+    static constexpr int CAP = (kWaveBytes / ENTRY - SLICE) / 16 * 16;
+    static constexpr int CAP_SCATTERED = (kWaveBytesScattered / ENTRY - SLICE) / 16 * 16;
+    static_assert(CAP_SCATTERED / 3 >= SLICE, "a slice fits a tile");
 };
 
 struct __align__(16) WaveDesc {
@@ -138,9 +143,10 @@ __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst)
     auto size_of = [&](int f) { return PACK ? packed_units(width_of(f), (f & kWideSlice) != 0) : 32 * width_of(f); };
     constexpr int G = 32 / M;  // rows of a unit
     using Buf = WaveBuf<VT>;
+    const uint32_t cap = (uint32_t)a.v_cap;  // entries of the buffer
     extern __shared__ __align__(128) unsigned char smem[];  // values, then columns
     T *const sval = reinterpret_cast<T *>(smem);
-    int32_t *const scol = reinterpret_cast<int32_t *>(smem + Buf::ALL * sizeof(T));  // (packed: unused)
+    int32_t *const scol = reinterpret_cast<int32_t *>(smem + (cap + Buf::SLICE) * sizeof(T));  // (packed: unused)
     __shared__ AT s_dict[PACK ? kDictSize : 1];
     if constexpr (PACK)
         for (int i = threadIdx.x; i < kDictSize; i += kWaveBS) s_dict[i] = (AT)a.v_dict[i];  // exact
@@ -222,8 +228,8 @@ __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst)
                     d.ckr = (uint32_t)(c0 + qc) << 11 | (uint32_t)(gk & 31) << 6 | (uint32_t)rec.w;
                 }
                 const int cnt = min(32, total - t0);
-                // where the entries go, and where runs start: at a cell's first slice, after a slice
-                // that is not copied, and where the buffer starts over
+                // where the entries go, and where runs start: at a cell's first slice and after a slice
+                // that is not copied (and, for the loader, where the buffer starts over)
                 const int size = width_of(d.width) <= kStagedWidth ? size_of(d.width) : 0;
                 uint32_t vp = (uint32_t)size;
 #pragma unroll
@@ -234,9 +240,8 @@ __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst)
                 const uint32_t vend = vnext + __shfl_sync(0xffffffffu, vp, 31);
                 vp += vnext - (uint32_t)size;
                 vnext = vend;
-                const uint32_t prev = __shfl_up_sync(0xffffffffu, vp, 1);
                 const int psize = __shfl_up_sync(0xffffffffu, size, 1);
-                if (lane == 0 || t == qend - csize || psize == 0 || prev / Buf::CAP != vp / Buf::CAP)
+                if (lane == 0 || t == qend - csize || psize == 0)
                     d.width |= (int)0x80000000;
                 if (pushed + cnt > room) {
                     Deadline w0;
@@ -269,6 +274,8 @@ __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst)
         // ------------------------------------------------------------------ loader
         int next = 0, tile = 0, old = 0;  // next descriptor, next tile, oldest tile in use
         uint32_t tail = 0;                // position of the oldest slice in use
+        uint32_t turn = 0;                // position at which the buffer last started over, before `next`
+        const uint32_t tile_cap = cap / 3;
         int t_desc = 0;                   // descriptors before the end of the tile with number lane (mod 32)
         Deadline w0;
         bool stop = false;
@@ -302,15 +309,15 @@ __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst)
             const bool staged = width_of(d.width) <= kStagedWidth;
             const uint32_t ve = vp + (staged ? (uint32_t)size_of(d.width) : 0u);
             const uint32_t v0 = __shfl_sync(0xffffffffu, vp, 0);
-            const unsigned int over = __ballot_sync(0xffffffffu, lane >= have || ve - v0 > (uint32_t)Buf::TILE);
+            const unsigned int over = __ballot_sync(0xffffffffu, lane >= have || ve - v0 > tile_cap);
             const int cnt = over ? __ffs(over) - 1 : 32;  // at least 1: a slice fits a tile
             const uint32_t vend = __shfl_sync(0xffffffffu, ve, cnt - 1);
-            while (vend - tail > (uint32_t)Buf::CAP || tile - old >= kWaveTiles) {  // room, and a free tile
+            while (vend - tail > cap || tile - old >= kWaveTiles) {  // room, and a free tile
                 done = frontier();
                 if (lane == 0) st_release_cta_shared(&s_done, done);
                 while (old < tile && __shfl_sync(0xffffffffu, t_desc, old & 31) <= done) ++old;
                 tail = done >= next ? v0 : vpos[done & (kDescRing - 1)];
-                if (vend - tail <= (uint32_t)Buf::CAP && tile - old < kWaveTiles) break;
+                if (vend - tail <= cap && tile - old < kWaveTiles) break;
                 if (__any_sync(0xffffffffu, aborted() || w0.expired(2 * a.wait_ns + 200000000LL))) {
                     if (lane == 0) give_up();
                     stop = true;
@@ -322,12 +329,16 @@ __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst)
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // every lane that copies
             if (lane == 0) mbar_expect_tx(&full[b], (vend - v0) * (uint32_t)Buf::ENTRY);
             __syncwarp();
-            const uint32_t o = vp % Buf::CAP;
+            // (a tile is a third of the buffer at most: it starts over once at most inside it)
+            const bool over_end = vp - turn >= cap;
+            const bool before = __shfl_up_sync(0xffffffffu, over_end, 1);
+            const uint32_t o = vp - turn - (over_end ? cap : 0u);
+            if (vend - turn >= cap) turn += cap;
             if (lane < cnt)
                 loc[(next + lane) & (kDescRing - 1)] =
                     staged ? (int)(PACK ? o : o >> 5) | b << 16 | ((tile / kWaveTiles) & 1) << 24 : -1;
             // a run of neighbouring slices: one pair of copies, by the run's first lane
-            const bool head = lane < cnt && staged && (lane == 0 || d.width < 0);
+            const bool head = lane < cnt && staged && (lane == 0 || d.width < 0 || over_end != before);
             const unsigned int heads = __ballot_sync(0xffffffffu, head || lane >= cnt || !staged);
             const unsigned int after = lane == 31 ? 0u : heads & (0xfffffffeu << lane);
             const uint32_t run = __shfl_sync(0xffffffffu, ve, after ? __ffs(after) - 2 : 31) - vp;
@@ -421,7 +432,8 @@ __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst)
                 const int total = __shfl_sync(0xffffffffu, end, 31);
                 end += base;
                 base += total;
-                bool todo = size > 0 && k < a.p_launch;  // nothing waits for the last power
+                // (nothing waits for the last power)
+                bool todo = size > 0 && k < a.p_launch && ce.z != a.v_drop;
                 Deadline w0;
                 for (;;) {
                     const unsigned int left = __ballot_sync(0xffffffffu, todo);
@@ -431,7 +443,7 @@ __device__ __forceinline__ void wave_body(const KArgs &a, const WaveBatch *inst)
                     if (__any_sync(0xffffffffu, now)) {
                         __syncwarp();         // every lane's view of the progress words
                         fence_acq_rel_gpu();  // acquires the finished slices' rows, releases them
-                        if (now && ce.z != a.v_drop)
+                        if (now)
                             atomicAdd(a.v_count + (int64_t)k * a.v_ngroups + (ce.z >> 5), size);
                         todo = todo && !now;
                         w0 = Deadline();
@@ -616,8 +628,17 @@ template <class VT, int M> static void *wave_fn(int mode, bool a32) {
     return mode == MODE_POWERS ? (void *)k_wave<M, MODE_POWERS, VT, false> : (void *)k_wave<M, MODE_CHEB, VT, false>;
 }
 
-template <class VT> void *select_wave_vt(int mode, int m, bool a32, int *smem) {
-    *smem = WaveBuf<VT>::ALL * WaveBuf<VT>::ENTRY;
+// entries of the buffer, [scattered], of a slice's room after it, and bytes of one
+struct WaveSize {
+    int cap[2], slice, entry;
+    int smem(bool scattered) const { return (cap[scattered] + slice) * entry; }
+    template <class VT> void set() {
+        using Buf = WaveBuf<VT>;
+        *this = WaveSize{{Buf::CAP, Buf::CAP_SCATTERED}, Buf::SLICE, Buf::ENTRY};
+    }
+};
+template <class VT> void *select_wave_vt(int mode, int m, bool a32, WaveSize *size) {
+    size->set<VT>();
     switch (m) {
         case 1: return wave_fn<VT, 1>(mode, a32);
         case 2: return wave_fn<VT, 2>(mode, a32);
@@ -628,10 +649,10 @@ template <class VT> void *select_wave_vt(int mode, int m, bool a32, int *smem) {
     fail(MPK_ERR_UNSUPPORTED, "nrhs %d", m);
 }
 
-// defined in mpk_wave_<type>.cu: the kernel for (mode, nrhs, accumulator) 
-void *select_wave_f64(int mode, int m, bool a32, int *smem);
-void *select_wave_f32(int mode, int m, bool a32, int *smem);
-void *select_wave_bf16(int mode, int m, bool a32, int *smem);
-void *select_wave_dict(int mode, int m, bool a32, int *smem);  // packed copies
+// defined in mpk_wave_<type>.cu: the kernel for (mode, nrhs, accumulator)
+void *select_wave_f64(int mode, int m, bool a32, WaveSize *size);
+void *select_wave_f32(int mode, int m, bool a32, WaveSize *size);
+void *select_wave_bf16(int mode, int m, bool a32, WaveSize *size);
+void *select_wave_dict(int mode, int m, bool a32, WaveSize *size);  // packed copies
 
 }  // namespace mpk

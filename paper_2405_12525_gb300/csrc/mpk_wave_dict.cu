@@ -3,8 +3,8 @@
 #include "mpk_wave.cuh"
 
 namespace mpk {
-void *select_wave_dict(int mode, int m, bool a32, int *smem) {
-    *smem = WaveBuf<ValDict>::ALL * WaveBuf<ValDict>::ENTRY;
+void *select_wave_dict(int mode, int m, bool a32, WaveSize *size) {
+    size->set<ValDict>();
     if (m != 1) fail(MPK_ERR_UNSUPPORTED, "packed copies are for one right-hand side, not %d", m);
     return wave_fn<ValDict, 1>(mode, a32);
 }

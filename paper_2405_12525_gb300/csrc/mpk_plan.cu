@@ -946,7 +946,8 @@ template <class F> static bool spare(Plan &P, WaveSet &w, F make) {
 // A's own numbering (plans of original order): no gather before and no scatter after the kernel.
 // Groups are runs of at least `band` rows (the largest |column - row|), so that a row reads its own
 // group and the two beside it.  Taken when the rows of x that a sweep reads around a row fit a
-// quarter of L2: a wider band is better served by the plan's level order.
+// quarter of L2 (a wider band is better served by the plan's level order), unless its gathers are
+// scattered where the levels' are not.
 static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector<int32_t> &g_row,
                       const std::vector<int32_t> &g_slice, const std::vector<int32_t> &c_slice,
                       const std::vector<int64_t> &sptr, const std::vector<int32_t> &s_row, const std::vector<int2> &hull,
@@ -996,12 +997,21 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
     const bool long_rows = P.nnz / std::max(n, 1) >= 16;
     const bool pack = !batch && !one && P.m == 1 &&
                       (P.val_type == MPK_F64 || (long_rows && (P.val_type == MPK_F32 || P.accum == MPK_F32)));
-    const bool natural = !P.identity && P.order == MPK_ORDER_ORIGINAL &&
-                         std::min<int64_t>(n, 2 * (int64_t)band + 32) * 8 * P.m <= device_l2_bytes() / 4;
+    bool natural = !P.identity && P.order == MPK_ORDER_ORIGINAL &&
+                   std::min<int64_t>(n, 2 * (int64_t)band + 32) * 8 * P.m <= device_l2_bytes() / 4;
     // (not looked at where the large buffer is as good: 8 and 16 columns within 3 %, up to 32768 rows of
     // one column the same)
     Spread spread[2];
     if (P.m <= 4 && (int64_t)n * P.m > 32768) gather_spread(P, A, natural, spread, s);
+    // A numbering whose gathers are scattered where the levels' are not is left to the plan order: one
+    // column, more rows than the gather and scatter of the vectors make up for.  Time of k_mpk, as it was
+    // before this kernel, over A's numbering / plan order (96 KB buffers), apply p = 8 and a recurrence of
+    // 32 steps, 7-point grids: 126^3 permuted, bfloat16 1.05 0.89 / 1.01 1.02, shuffled in windows of 10 000
+    // rows, binary64 1.01 0.98 / 1.14 1.10, binary32 0.82 0.81 / 1.09 1.02, of 100 000 rows, bfloat16 and binary32
+    // sums 0.69 0.75 / 1.01 0.93; 63^3 (0.25 M rows) permuted 1.72 1.38 / 1.48 1.55, kept.  Banded graphs, whose
+    // gathers spread alike in both, are better off in A's numbering at every size (1M rows, binary32: 1.00
+    // 1.04 / 0.96 1.03), two columns of anything too (126^3 permuted: 1.52 1.15 / 1.29 1.22).
+    if (!batch && P.m == 1 && n > 1 << 18 && spread[0].lines > 0.5 && spread[0].bytes > 1.4 * spread[1].bytes) natural = false;
     std::unique_ptr<Tmp<Dict>> table;
     bool packed = false;
     if (pack) try {

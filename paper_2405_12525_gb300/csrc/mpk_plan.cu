@@ -694,13 +694,18 @@ __global__ void __launch_bounds__(1024) k_gather_spread(int nat_samples, int64_t
 struct Spread {
     double lines = 0.0, bytes = 0.0, fresh = 0.0;
     // Whether the wave kernel takes its smaller buffer (its figures beside kWaveBytes): gathers that touch
-    // about a line a row, and read more than the L1 beside the large one holds, most of it for the first
+    // about a line a row, and read more than the L1 beside the large one holds, much of it for the first
     // time.  Measured over grids, stencils, the spin chain and banded graphs, in order, permuted and shuffled
     // in windows, 1 to 4 columns, p = 8, time at 200 KB over that at 96 KB: lines up to 0.6 a row: 0.59 to
-    // 1.0 (spin chain 0.25 lines: 0.58 to 0.74); above, up to 40 KB: 0.7 to 0.9 (banded graph of 100k rows, 31
-    // KB), and fresh up to 0.2: 0.8 to 1.04 (same, 2 columns, 62 KB, 0.13); the rest 1.0 to 2.9, but for
-    // 63^3 in windows of 1000 rows (69 KB, 0.6): 0.92.
-    bool scattered() const { return lines > 0.62 && bytes > 40e3 && fresh > 0.22; }
+    // 1.0 (spin chain 0.25 lines: 0.58 to 0.74); above, up to 47 KB: 0.7 to 0.95 (banded graph of 100k rows, 31
+    // KB; a permuted grid of 1400^2, 41 KB: 1.57); above, little of it fresh: 0.8 to 1.04 (the same, 2 columns, 62
+    // KB, 0.13; of 300k rows, 60 KB, 0.25: 0.92); the rest 1.0 to 2.9, but for 63^3 in windows of 1000 rows (69 KB,
+    // 0.6): 0.92.  binary64 values with 4 columns need the lead more: banded graphs (0.23 to 0.45) 0.97, permuted
+    // grids (above) 1.06 to 1.2.
+    bool lead = false;
+    bool scattered() const {
+        return lines > 0.62 && bytes > 47e3 && (lead ? fresh > 0.5 : fresh > 0.3 || (fresh > 0.22 && bytes > 96e3));
+    }
 };
 // in A's numbering (at[0], if asked for) and in plan order (at[1])
 static void gather_spread(const Plan &P, const mpk_csr *A, bool natural, Spread (&at)[2], cudaStream_t s) {
@@ -722,6 +727,7 @@ static void gather_spread(const Plan &P, const mpk_csr *A, bool natural, Spread 
         at[q].lines = (double)h[q].lines / rows;
         at[q].bytes = (double)h[q].bytes / std::max(1, q ? plan : nat);
         at[q].fresh = (double)h[q].bytes / (rows * xbytes);
+        at[q].lead = P.val_bytes == 8 && P.m == 4;
     }
 }
 

@@ -948,7 +948,7 @@ template <class F> static bool spare(Plan &P, WaveSet &w, F make) {
 // one cell); others take runs of the plan's groups.  The plan goes without (and runs k_mpk) when a
 // chunk reads rows outside its own group and the two beside it, which the kernel's dependency rule
 // does not cover (levels of another matrix).  It works on the plan's own sliced copy, or, when that
-// has over 4 % of padding, on one with its rows sorted by length.
+// has over 4 % of padding and A's numbering is not taken, on one with its rows sorted by length.
 // A's own numbering (plans of original order): no gather before and no scatter after the kernel.
 // Groups are runs of at least `band` rows (the largest |column - row|), so that a row reads its own
 // group and the two beside it.  Taken when the rows of x that a sweep reads around a row fit a
@@ -1028,8 +1028,39 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
             cudaGetLastError();
         }
     const Dict *dict = packed ? table->p : nullptr;
-    const Dict *plan_dict = natural ? nullptr : dict;
     const double packed_entry = 3.2, entry_bytes = packed ? packed_entry : P.val_bytes + 4;
+    if (natural) {
+        std::vector<int32_t> nrow;
+        std::vector<WaveRange> nranges;
+        for (const Inst &t : in) {
+            WaveRange r{(int32_t)nrow.size(), 0, t.p, t.bytes};
+            int64_t rows = t.r1 - t.r0;
+            if (!t.one) {
+                // A default budget of 5/4 of L2 where that is a good part of the matrix and its vectors, 3/5 of
+                // L2 beyond 3 times L2, where its window no longer stays in L2 (p = 8, us, 5/4 / 3/5 of L2;
+                // packed 7-point: 131^3 258 / 269, 200^3 872 / 876, 230^3 1384 / 1318, 256^3 1946 / 1794, 290^3
+                // 3007 / 2801; 256^3 bfloat16, binary32 sums: 1457 / 1346; packed 5-point: 2000^2 376 / 382,
+                // 4000 x 4100 1513 / 1489)
+                const double a_row = entry_bytes * (double)(P.nnz / std::max(n, 1) + 1) + (double)row_bytes;
+                const bool large = default_budget && a_row * (double)rows > 3.0 * (double)device_l2_bytes();
+                const int64_t most = large ? device_l2_bytes() / 5 * 3 / (kSlotSkew * t.p + 1) : t.most;
+                rows = std::max<int64_t>(band, (int64_t)((double)most / a_row));
+                // equal shares for the blocks where a group has a few slices for each (27-point stencil on
+                // 150^3, p = 8, packed: 1349 -> 1261 us; below, a whole slice more for each would be too much)
+                const int64_t even = 32 * (int64_t)device_sms();
+                rows = rows >= 2 * even ? (rows + even - 1) / even * even : std::max<int64_t>(32, (rows + 31) / 32 * 32);
+            }
+            for (int64_t q = t.r0; q < t.r1; q += rows) nrow.push_back((int32_t)q);
+            r.g1 = (int32_t)nrow.size();
+            nranges.push_back(r);
+        }
+        nrow.push_back(n);
+        natural = spare(P, P.natural, [&]() { return wave_copy(P, P.natural, A, nullptr, nullptr, nrow, nranges, dict, host[1], s); });
+        P.natural.scattered = spread[0].scattered();
+    }
+    // What runs in plan order beside A's numbering (X inside Y, the resumable recurrence, a batch without
+    // every output) has the plan's own copy, not one more.
+    const Dict *plan_dict = natural ? nullptr : dict;
     const double plan_entry = plan_dict ? packed_entry : P.val_bytes + 4;
     std::vector<int32_t> vs;  // first slice of every group, and the end
     std::vector<WaveRange> ranges;
@@ -1061,8 +1092,10 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
         }
     }
     if (near) {
-        bool own = false;
-        if (P.padded <= P.nnz + P.nnz / 25) {
+        bool own = false;  // a copy of its own
+        if (natural) {
+            // the plan's
+        } else if (P.padded <= P.nnz + P.nnz / 25) {
             if (plan_dict) own = spare(P, P.wave, [&]() {
                     Tmp<int32_t> width(NS, s);
                     Tmp<int64_t> units((int64_t)NS + 1, s);
@@ -1085,34 +1118,6 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
         }
         P.wave.scattered = spread[1].scattered();
     }
-    if (!natural) return;
-    std::vector<int32_t> nrow;
-    ranges.clear();
-    for (const Inst &t : in) {
-        WaveRange r{(int32_t)nrow.size(), 0, t.p, t.bytes};
-        int64_t rows = t.r1 - t.r0;
-        if (!t.one) {
-            // A default budget of 5/4 of L2 where that is a good part of the matrix and its vectors, 3/5 of
-            // L2 beyond 3 times L2, where its window no longer stays in L2 (p = 8, us, 5/4 / 3/5 of L2;
-            // packed 7-point: 131^3 258 / 269, 200^3 872 / 876, 230^3 1384 / 1318, 256^3 1946 / 1794, 290^3
-            // 3007 / 2801; 256^3 bfloat16, binary32 sums: 1457 / 1346; packed 5-point: 2000^2 376 / 382,
-            // 4000 x 4100 1513 / 1489)
-            const double a_row = entry_bytes * (double)(P.nnz / std::max(n, 1) + 1) + (double)row_bytes;
-            const bool large = default_budget && a_row * (double)rows > 3.0 * (double)device_l2_bytes();
-            const int64_t most = large ? device_l2_bytes() / 5 * 3 / (kSlotSkew * t.p + 1) : t.most;
-            rows = std::max<int64_t>(band, (int64_t)((double)most / a_row));
-            // equal shares for the blocks where a group has a few slices for each (27-point stencil on
-            // 150^3, p = 8, packed: 1349 -> 1261 us; below, a whole slice more for each would be too much)
-            const int64_t even = 32 * (int64_t)device_sms();
-            rows = rows >= 2 * even ? (rows + even - 1) / even * even : std::max<int64_t>(32, (rows + 31) / 32 * 32);
-        }
-        for (int64_t q = t.r0; q < t.r1; q += rows) nrow.push_back((int32_t)q);
-        r.g1 = (int32_t)nrow.size();
-        ranges.push_back(r);
-    }
-    nrow.push_back(n);
-    spare(P, P.natural, [&]() { return wave_copy(P, P.natural, A, nullptr, nullptr, nrow, ranges, dict, host[1], s); });
-    P.natural.scattered = spread[0].scattered();
 }
 
 Plan *build_plan(const mpk_csr *A, const Levels *L, const mpk_plan_opts *o, cudaStream_t s,

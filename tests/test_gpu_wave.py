@@ -333,3 +333,30 @@ def test_a_wait_that_expires_in_a_batch(mpk, order):
         status()
         for Y, w in zip(Ys, want):
             assert np.array_equal(Y.cpu().numpy().view(np.uint64), w.view(np.uint64))
+
+
+def test_one_more_copy_beside_the_plans_own(mpk):
+    """Rows of very different lengths in a narrow band, original order: the plan's sliced copy and one in
+    A's numbering, not a third one in plan order with its rows sorted by length."""
+    A = _widths_matrix(40000, (1, 30, 4, 17, 0, 9, 2), 930)
+    dA = mpk.CsrMatrix.from_host(A)
+    L = mpk.build_levels(dA, 0)
+    P = mpk.plan(dA, L, p_max=5)
+    vectors = 8 * A.n * 6  # the workspace
+    padded = 12 * P.describe()["padded_entries"]
+    own = 12 * A.nnz * 1.04 + 4 * A.n  # sorted rows, their map
+    fits = P.describe()["device_bytes"]
+    assert fits < vectors + padded + own + 60 * A.n + (1 << 20)  # (permutations, tables, records)
+    # with room for exactly that the plan is the same, and its resumable recurrence right
+    P = mpk.plan(dA, L, p_max=5, mem_budget=fits)
+    X = gen.vector(A.n, 1, stream=6)
+    Xd = torch.from_numpy(X).cuda()
+    c = np.linspace(1.0, -0.5, 12)
+    S = P.cheb_begin(Xd, P.cheb_state(), c[0])
+    P.cheb_advance(S, 0, 5, c, scale=9.0, shift=0.3)
+    P.cheb_advance(S, 5, 11, c, scale=9.0, shift=0.3)
+    out = P.cheb_finish(S).cpu().numpy()
+    P.sync_status()
+    want = oracle.cheb(A, X, 11, c, scale=9.0, shift=0.3)
+    assert np.array_equal(out.view(np.uint64), want.view(np.uint64))
+    assert P.describe()["device_bytes"] == fits

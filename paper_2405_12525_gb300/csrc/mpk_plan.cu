@@ -707,29 +707,38 @@ struct Spread {
         return lines > 0.62 && bytes > 47e3 && (lead ? fresh > 0.5 : fresh > 0.3 || (fresh > 0.22 && bytes > 96e3));
     }
 };
-// in A's numbering (at[0], if asked for) and in plan order (at[1])
-static void gather_spread(const Plan &P, const mpk_csr *A, bool natural, Spread (&at)[2], cudaStream_t s) {
-    Tmp<GatherSpread> d(2, s);
-    MPK_CUDA(cudaMemsetAsync(d.p, 0, 2 * sizeof(GatherSpread), s));
-    const int per = (int)std::max<int64_t>(1, std::min<int64_t>(kSpreadSlices, kSpreadEntries / (32 * (P.nnz / P.n + 1))));
-    const int xbytes = (P.accum == MPK_F32 ? 4 : 8) * P.m;
-    auto samples = [&](int64_t nslices) { return (int)std::max<int64_t>(1, std::min<int64_t>(kSpreadSamples, nslices / per)); };
-    const int64_t ns = ((int64_t)P.n + 31) / 32;
-    const int nat = natural ? samples(ns) : 0, plan = samples(P.num_slices);
-    k_gather_spread<<<nat + plan, 1024, 0, s>>>(nat, ns, CsrSlices{A->row_ptr, A->col, P.n}, P.num_slices,
-                                                PlanSlices{P.slice_ptr, P.col}, per, P.m, xbytes, d.p);
-    MPK_LAUNCHED();
-    GatherSpread h[2];
-    MPK_CUDA(cudaMemcpyAsync(h, d.p, sizeof(h), cudaMemcpyDeviceToHost, s));
-    MPK_CUDA(cudaStreamSynchronize(s));
-    for (int q = 0; q < 2; ++q) {
-        const double rows = (double)std::max<unsigned long long>(h[q].rows, 1);
-        at[q].lines = (double)h[q].lines / rows;
-        at[q].bytes = (double)h[q].bytes / std::max(1, q ? plan : nat);
-        at[q].fresh = (double)h[q].bytes / (rows * xbytes);
-        at[q].lead = P.val_bytes == 8 && P.m == 4;
+// Of A's numbering (at[0], if asked for) and of the plan order (at[1]): measured on the stream by the
+// constructor, read by read(), which waits for it.
+struct SpreadSample {
+    const Plan &P;
+    cudaStream_t s;
+    Tmp<GatherSpread> d;
+    int per, xbytes, nat = 0, plan = 0;
+    SpreadSample(const Plan &plan_, const mpk_csr *A, bool natural, cudaStream_t s_) : P(plan_), s(s_), d(2, s_) {
+        per = (int)std::max<int64_t>(1, std::min<int64_t>(kSpreadSlices, kSpreadEntries / (32 * (P.nnz / P.n + 1))));
+        xbytes = (P.accum == MPK_F32 ? 4 : 8) * P.m;
+        auto samples = [&](int64_t nslices) { return (int)std::max<int64_t>(1, std::min<int64_t>(kSpreadSamples, nslices / per)); };
+        const int64_t ns = ((int64_t)P.n + 31) / 32;
+        nat = natural ? samples(ns) : 0;
+        plan = samples(P.num_slices);
+        MPK_CUDA(cudaMemsetAsync(d.p, 0, 2 * sizeof(GatherSpread), s));
+        k_gather_spread<<<nat + plan, 1024, 0, s>>>(nat, ns, CsrSlices{A->row_ptr, A->col, P.n}, P.num_slices,
+                                                    PlanSlices{P.slice_ptr, P.col}, per, P.m, xbytes, d.p);
+        MPK_LAUNCHED();
     }
-}
+    void read(Spread (&at)[2]) {
+        GatherSpread h[2];
+        MPK_CUDA(cudaMemcpyAsync(h, d.p, sizeof(h), cudaMemcpyDeviceToHost, s));
+        MPK_CUDA(cudaStreamSynchronize(s));
+        for (int q = 0; q < 2; ++q) {
+            const double rows = (double)std::max<unsigned long long>(h[q].rows, 1);
+            at[q].lines = (double)h[q].lines / rows;
+            at[q].bytes = (double)h[q].bytes / std::max(1, q ? plan : nat);
+            at[q].fresh = (double)h[q].bytes / (rows * xbytes);
+            at[q].lead = P.val_bytes == 8 && P.m == 4;
+        }
+    }
+};
 
 // A run of groups whose powers are computed together: a whole plan, or an instance of a batch plan
 struct WaveRange {
@@ -1007,8 +1016,22 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
                    std::min<int64_t>(n, 2 * (int64_t)band + 32) * 8 * P.m <= device_l2_bytes() / 4;
     // (not looked at where the large buffer is as good: 8 and 16 columns within 3 %, up to 32768 rows of
     // one column the same)
+    std::unique_ptr<SpreadSample> sample;
+    std::unique_ptr<Tmp<Dict>> table;
+    bool packed = false;
+    try {
+        if (P.m <= 4 && (int64_t)n * P.m > 32768) sample.reset(new SpreadSample(P, A, natural, s));
+        if (pack) {
+            table.reset(new Tmp<Dict>(1, s));
+            packed = find_values(P, A, table->p, s);
+        }
+    } catch (const Fail &f) {  // no memory for them: the plan does without
+        if (f.status != MPK_ERR_OOM) throw;
+        cudaGetLastError();
+    }
+    const Dict *dict = packed ? table->p : nullptr;
     Spread spread[2];
-    if (P.m <= 4 && (int64_t)n * P.m > 32768) gather_spread(P, A, natural, spread, s);
+    if (sample) sample->read(spread);
     // A numbering whose gathers are scattered where the levels' are not is left to the plan order: one
     // column, more rows than the gather and scatter of the vectors make up for.  Time of k_mpk, as it was
     // before this kernel, over A's numbering / plan order (96 KB buffers), apply p = 8 and a recurrence of
@@ -1018,16 +1041,6 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
     // gathers spread alike in both, are better off in A's numbering at every size (1M rows, binary32: 1.00
     // 1.04 / 0.96 1.03), two columns of anything too (126^3 permuted: 1.52 1.15 / 1.29 1.22).
     if (!batch && P.m == 1 && n > 1 << 18 && spread[0].lines > 0.5 && spread[0].bytes > 1.4 * spread[1].bytes) natural = false;
-    std::unique_ptr<Tmp<Dict>> table;
-    bool packed = false;
-    if (pack) try {
-            table.reset(new Tmp<Dict>(1, s));
-            packed = find_values(P, A, table->p, s);
-        } catch (const Fail &f) {  // no memory for the table
-            if (f.status != MPK_ERR_OOM) throw;
-            cudaGetLastError();
-        }
-    const Dict *dict = packed ? table->p : nullptr;
     const double packed_entry = 3.2, entry_bytes = packed ? packed_entry : P.val_bytes + 4;
     if (natural) {
         std::vector<int32_t> nrow;

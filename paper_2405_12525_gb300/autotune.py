@@ -1,5 +1,5 @@
-"""Autotuner for plan parameters: the group budget C (cache_bytes), the rows per chunk, the
-kernel's block shape and, for single plans, the unblocked sweep engine as one more candidate.
+"""Autotuner for plan parameters: the group budget C (cache_bytes), the rows per chunk (of the ticketed
+kernel only), the kernel's block shape and, for single plans, the unblocked sweep engine as one more candidate.
 
 The paper studies p and C by hand (Sec. 6, the p x C parameter scan); here each candidate
 plan is built, timed on the device with CUDA events over a few applies of the caller's
@@ -26,10 +26,11 @@ def _time(fn, reps: int):
 
 
 def default_candidates():
-    """Group budgets of 1/4, 1/2, 1 and 2 times the L2 size; the default chunk and 960 rows; the
-    planner's block shape, shape 0 and the unstaged shape (plan option shape = 0, 1, 3)."""
+    """The planner's own group budget (0), and 1/4, 1/2, 1 and 2 times the L2 size; the default chunk
+    and 960 rows; the planner's block shape, shape 1 and the unstaged shape (plan option shape = 0, 1,
+    3).  The untuned plan is among them, so the tuned one is never slower."""
     _, l2 = device_info()
-    return {"cache_bytes": [l2 // 4, l2 // 2, l2, 2 * l2], "chunk_rows": [0, 960], "shape": [0, 1, 3]}
+    return {"cache_bytes": [0, l2 // 4, l2 // 2, l2, 2 * l2], "chunk_rows": [0, 960], "shape": [0, 1, 3]}
 
 
 def _grid(cands):

@@ -113,3 +113,13 @@ def test_tune_batch_keeps_the_fastest_candidate(monkeypatch):
     assert best.opts["cache_bytes"] == 4 and [ms for ms, _ in report] == [2.5, 5.0, 10.0]
     with pytest.raises(ValueError):
         autotune.tune_batch([Mat()], [3], [None], candidates={"cache_bytes": [], "chunk_rows": [0]})
+
+
+def test_the_untuned_plan_is_a_candidate(monkeypatch):
+    """cache_bytes 0 keeps the planner's own budgets, which no other value gives."""
+    monkeypatch.setattr(autotune, "device_info", lambda: (152, 1 << 27))
+    grid = list(autotune._grid(autotune.default_candidates()))
+    assert {"cache_bytes": 0, "chunk_rows": 0, "shape": 0} in grid
+    _fake_device(monkeypatch, lambda o: 1.0 if o.get("cache_bytes") == 0 and o["shape"] == 0 else 2.0)
+    best, report = autotune.tune_plan(Mat(), None, 4, torch.zeros(5, 1, dtype=torch.float64))
+    assert best.opts["cache_bytes"] == 0 and best.opts["shape"] == 0 and report[0][0] == 1.0

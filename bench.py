@@ -1087,7 +1087,9 @@ def main():
                              f"{roofs['l2_bytes'] / 1e6:.0f} MB)",
                        "levels": desc["num_levels"], "groups": desc["num_groups"], "chunks": desc["num_chunks"],
                        "shape": desc["shape"], "chunk_rows": desc["chunk_rows"], "split_levels": args.split,
-                       "cache_bytes": desc["cache_bytes"], "window": desc["window"]},
+                       "cache_bytes": desc["cache_bytes"], "window": desc["window"],
+                       "schedule": "groups, chunks, shape, cache_bytes and window are the plan's row-chunk schedule; "
+                                   "the timed kernel runs cells of whole groups of it, sized for its own budget"},
             "roofline": roofline,
             "original_order": {"ms_per_step": ms_orig, "gflops": flops / (ms_orig * 1e-3) / 1e9,
                                "note": "level-blocked kernel on a copy of the matrix in its own numbering (no gather or scatter)",

@@ -131,12 +131,16 @@ typedef struct {
                                unstaged block shape (shape 0 or 3) of the staged or the sweep
                                engine, else MPK_ERR_UNSUPPORTED                              */
     int64_t cache_bytes;    /* C in bytes; 0 = three quarters of the device L2 (five
-                               quarters with two slices a warp, shape 5 below)               */
+                               quarters with two slices a warp, shape 5 below), and, for the
+                               schedule of shapes 0 and 3 (see mpk_apply), five quarters of
+                               it, or three fifths in A's numbering beyond three times L2    */
     int32_t order;          /* mpk_order of X, Y and the Chebyshev input/output             */
     int32_t chunk_rows;     /* rows per work unit (multiple of 32); 0 = 32 per compute warp
                                and slice of the block shape (512 for shape 2, 1024 for 5)     */
     int64_t wait_limit_ns;  /* bound on every device-side wait; 0 = 2 s                     */
-    int64_t mem_budget;     /* bytes the plan may allocate on the device; 0 = no limit     */
+    int64_t mem_budget;     /* bytes the plan may allocate on the device; 0 = no limit.  The
+                               plan leaves out its second copy of the matrix (see mpk_apply;
+                               up to (val_bytes + 4) * nnz + 4 n bytes) where it does not fit */
     int32_t trace;          /* 1: the level-blocked kernel accumulates timing counters      */
     int32_t level_capped;   /* 1: a row of BFS level L takes powers 1..min(L, p) only, the
                                local phase of DLB-MPK (Alg. 2) with the levels built from the
@@ -234,6 +238,9 @@ typedef struct {
                                      of each group's first row                             */
 } mpk_plan_desc;
 
+/* (The groups, their budget and window, the chunks and the block shape are those of the row-chunk
+ * schedule of mpk_apply.  Plans that run the schedule of shapes 0 and 3 keep it for the calls that
+ * need it; their own groups are runs of these, or runs of A's rows.) */
 mpk_status mpk_plan_describe(const mpk_plan_t *P, mpk_plan_desc *out);
 
 /* Writes the plan's permuted matrix P A P^T as CSR into caller buffers (device):
@@ -255,12 +262,19 @@ void mpk_plan_destroy(mpk_plan_t *P);
  * block per SM, and a cell waits on the counters of the cells it reads at power k-1; the other
  * shapes (and plans with trace, shuffle_seed, level_capped or split_levels, or whose tables do
  * not fit mem_budget) run row chunks that wait on the completion flags of the chunks they read.
- * With MPK_ORDER_ORIGINAL and a matrix of narrow band (the rows of X between a row's smallest
- * and largest column fit a quarter of L2) the plan keeps a second copy of the matrix in A's
- * own numbering, if mem_budget allows, and the kernel reads X and writes Y in place; else a
- * gather kernel first takes X into plan order in the plan's workspace, the kernel computes
+ * With MPK_ORDER_ORIGINAL the plan keeps a second copy of the matrix in A's own numbering, if
+ * mem_budget and device memory allow, and the kernel reads X and writes Y in place, where
+ *  - the rows of X between a row's smallest and largest column fit a quarter of L2 (all rows do, for
+ *    matrices of up to 4.2 M rows / nrhs), and
+ *  - for one right-hand side and more than 262144 rows, A's numbering does not scatter the reads of X
+ *    where the plan's keeps them together.
+ * Else a gather kernel first takes X into plan order in the plan's workspace, the kernel computes
  * every power there, and a last pass writes Y[1..p] through the permutation (one gather per
- * output row).  Results equal back-to-back SpMV bit for bit.  Not safe to run concurrently with another call on the same plan.
+ * output row).  Results equal back-to-back SpMV bit for bit.
+ * The launch of shapes 0 and 3 is a cooperative one that takes every SM: it starts when the kernels
+ * running on other streams leave room for one block on each, so a kernel that waits for this call's
+ * result on the device must not keep an SM to itself.
+ * Not safe to run concurrently with another call on the same plan.
  * ------------------------------------------------------------------------------------- */
 mpk_status mpk_apply(const mpk_plan_t *P, const double *X, int32_t p, double *Y, mpk_stream stream);
 
@@ -328,7 +342,8 @@ mpk_status mpk_cheb_filter(const mpk_plan_t *P, const double *X, int32_t degree,
  * mpk_cheb_state_bytes(P) bytes.  Blocks 0..2 are a ring holding v_j in block j % 3 (when the
  * state holds step k, v_k and v_{k-1} are live and the third block is scratch), block 3 is the
  * accumulator.  Save and restore all mpk_cheb_state_bytes(P) bytes.  Any split of the steps
- * gives the same bits as one mpk_cheb_filter call.
+ * gives the same bits as one mpk_cheb_filter call (which is faster where it runs in A's own
+ * numbering: the state is in plan order, and so are these steps).
  *   mpk_cheb_begin:   state <- v_0 = X, acc = c_0 X (c_0 = c0_re + i c0_im on (re, im) column
  *                     pairs when complex_coeff is 1); the state holds step 0.
  *   mpk_cheb_advance: steps k_begin+1 .. k_end with coefficients coeff_re[k] (and coeff_im[k]),
@@ -365,7 +380,7 @@ mpk_status mpk_read_trace(const mpk_plan_t *P, int64_t *counters, mpk_stream str
  * one persistent launch per apply.  The plan is that of the block-diagonal direct sum of the
  * matrices (Sec. 3's level blocking applies to it unchanged): block i keeps its own BFS
  * levels and row range, groups never span two blocks, and the blocks' Lp-diagram cells are
- * merged line by line into one ticket space, so that small blocks run side by side.
+ * merged line by line into one schedule, so that small blocks run side by side.
  * mats[i]: device CSR as for mpk_plan, all of one val_type; p_each[i] in [1, opts->p_max];
  * opts->nrhs applies to every block and opts->order to each block's own numbering (in plan
  * order block i uses the numbering of its own levels, mpk_build_levels(mats[i], 0)).
@@ -378,7 +393,10 @@ mpk_status mpk_batch_plan(const mpk_csr *mats, int32_t count, const int32_t *p_e
 /* X[i], Y[i]: host arrays of `count` device pointers; X[i] is n_i x nrhs and Y[i] receives
  * (p_each[i] + 1) x n_i x nrhs, powers 0..p_each[i] of block i (row-major, float64).
  * Y[i] = NULL leaves block i's powers in the plan's workspace only (see mpk_batch_workspace),
- * which saves their copy.  Asynchronous on `stream` (capturable in a CUDA graph); errors as
+ * which saves their copy.  The launch reads every X[i] and writes every Y[i] in place when the plan
+ * has at most 64 blocks, every Y[i] is given and no X or Y shares memory with another (but X[i] ==
+ * Y[i]); else the whole batch goes through the workspace, with a gather before and copies after.  Of outputs that share memory, powers 1 .. p of
+ * the last one stand.  Asynchronous on `stream` (capturable in a CUDA graph); errors as
  * for mpk_apply. */
 mpk_status mpk_batch_apply(const mpk_plan_t *P, const double *const *X, double *const *Y, mpk_stream stream);
 

@@ -405,7 +405,7 @@ struct Plan {
     int32_t *w_slice_chunk = nullptr;   // chunk of every slice (device)
     int32_t *w_chunk_nsl = nullptr;     // slices of every chunk (device)
     // wave kernel (single plans of the staged engine at the planner's own block shape): in plan
-    // order, and, for original-order plans whose matrix has a narrow band, in the matrix's own
+    // order, and, for original-order plans whose numbering serves (plan_wave), in the matrix's own
     WaveSet wave, natural;
     int32_t drop_unit = -1;  // armed by mpk_debug_drop_release for the next launch
     unsigned long long *trace = nullptr;  // counters when built with opts.trace

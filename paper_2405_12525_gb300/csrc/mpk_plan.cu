@@ -338,6 +338,7 @@ void export_csr(const Plan &P, int32_t *rp, int32_t *ci, double *va, cudaStream_
 // ----------------------------------------------------------------------------- wave kernel's tables
 // width of every slice (its longest row) and, if map is given, its rows sorted by length: blocks of
 // kSortSlices slices, longest first, stable, so that the 32 rows of a slice are about equally long
+// (the sorting window of SELL-C-sigma: Kreutzer et al., SIAM J. Sci. Comput. 36(5), 2014)
 // (longer blocks pad less but spread a slice's gathers: 2 / 4 / 8 / 32 slices, XXZ L = 24 recurrence 15.1 /
 // 15.0 / 15.4 / 15.6 ms, banded graph of 300k rows 271 / 249 / 240 / 238 us)
 // (slice s holds the rows [slice_row[s], slice_row[s + 1]) of its block's sorted list).  A block never
@@ -971,7 +972,7 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
     if (P.padded / 32 >= INT32_MAX) return;
     // the kernel's cells pay for a larger budget than k_mpk's, since a block's share of a cell is what
     // hides the cell's hand-over to the next power (256^3, p = 8: 97 / 130 / 160 / 200 MB took 2.18 /
-    // 2.09 / 2.09 / 2.14 ms)
+    // 2.09 / 2.09 / 2.14 ms; binary32 sums 100 / 130 / 160 / 200 MB 1.40 / 1.34 / 1.36 / 1.40 ms: one rule for both)
     const int64_t wave_cache = default_budget ? device_l2_bytes() / 4 * 5 : P.cache_bytes;
     const bool batch = !P.inst_p.empty();
     const int64_t row_bytes = 4 + 16 * (int64_t)P.m, vec_bytes = 32 * (int64_t)P.m;

@@ -596,11 +596,12 @@ __global__ void k_pack_fill(int32_t nslices, R rows, const T *va, const int32_t 
 }
 
 // How the gathers of x spread, from samples of up to 2048 rows (64 slices; of fewer when they hold over
-// 64 K entries): `lines` / `rows`, the 128-byte lines that a gather of one entry of a unit's rows touches,
-// per row, and `bytes`, those of the different 32-byte sectors that a sample's entries read (counted in
-// a bitmap of hashes, by the bits left free).
+// 64 K entries): `lines` / `looked`, the 128-byte lines that a gather of one entry of a unit's rows touches,
+// per row (looked at for one entry in four: comparing lanes takes most of the kernel's time), and `bytes`,
+// those of the different 32-byte sectors that a sample's entries read (counted in a bitmap of hashes, by the
+// bits left free), of `rows` gathered rows.
 struct GatherSpread {
-    unsigned long long lines, rows;
+    unsigned long long lines, looked, rows;
     float bytes;  // of all samples
 };
 constexpr int kSpreadSlices = 64, kSpreadEntries = 1 << 16, kSpreadSamples = 64, kSpreadBits = 1 << 18;
@@ -608,7 +609,8 @@ constexpr int kSpreadSlices = 64, kSpreadEntries = 1 << 16, kSpreadSamples = 64,
 struct CsrSlices {
     const int32_t *rp, *ci;
     int32_t n;
-    // calls f with the columns of the slice's first entries (-1: a row has fewer), four at a time
+    // calls f with the number (mod 4) and the columns of the slice's first entries (-1: a row has fewer),
+    // four at a time
     template <class F> __device__ __forceinline__ void visit(int64_t s, int most, int lane, F f) const {
         const int64_t r = 32 * s + lane;
         const int32_t e0 = r < n ? rp[r] : 0, len = r < n ? rp[r + 1] - e0 : 0;
@@ -618,7 +620,7 @@ struct CsrSlices {
 #pragma unroll
             for (int t = 0; t < 4; ++t) c[t] = j + t < len ? ci[e0 + j + t] : -1;
 #pragma unroll
-            for (int t = 0; t < 4; ++t) f(c[t]);
+            for (int t = 0; t < 4; ++t) f(t, c[t]);
         }
     }
 };
@@ -634,7 +636,7 @@ struct PlanSlices {
 #pragma unroll
             for (int t = 0; t < 4; ++t) c[t] = j + t < w ? col[e0 + 32 * (int64_t)(j + t) + lane] : -1;
 #pragma unroll
-            for (int t = 0; t < 4; ++t) f(c[t]);
+            for (int t = 0; t < 4; ++t) f(t, c[t]);
         }
     }
 };
@@ -643,29 +645,35 @@ template <class R>
 __device__ __forceinline__ void spread_sample(int64_t nslices, int per, const R &rows, int m, int xbytes, int block, int blocks,
                                               GatherSpread *out) {
     __shared__ uint32_t seen[kSpreadBits / 32];
-    __shared__ int s_lines, s_rows, s_set;
+    __shared__ int s_lines, s_looked, s_rows, s_set;
     for (int i = threadIdx.x; i < kSpreadBits / 32; i += blockDim.x) seen[i] = 0;
-    if (threadIdx.x == 0) s_lines = s_rows = s_set = 0;
+    if (threadIdx.x == 0) s_lines = s_looked = s_rows = s_set = 0;
     __syncthreads();
-    const int lane = threadIdx.x & 31, sector = max(32, xbytes);
+    const int lane = threadIdx.x & 31, sector = max(32, xbytes), shift = 31 - __clz(sector);  // (a power of two)
     const int64_t s0 = blocks > 1 ? (nslices - per) * block / (blocks - 1) : 0;
-    int lines = 0, taken = 0;
+    int lines = 0, looked = 0, taken = 0;
     for (int q = threadIdx.x >> 5; q < per && s0 + q < nslices; q += blockDim.x >> 5) {
-        rows.visit(s0 + q, kSpreadEntries / 32, lane, [&](int32_t c) {
+        rows.visit(s0 + q, kSpreadEntries / 32, lane, [&](int t, int32_t c) {
             const unsigned int on = __ballot_sync(0xffffffffu, c >= 0);
+            const bool look = t == ((q ^ (q >> 5)) & 3);  // (every entry of the rows in some slice)
+            const unsigned long long at = (unsigned long long)max(c, 0) * xbytes;
             bool first = false;
-            if (c >= 0) {  // (a unit: 32 / m rows)
-                const unsigned long long at = (unsigned long long)c * xbytes;
+            if (look && c >= 0)  // (a unit: 32 / m rows)
                 first = lane == __ffs(__match_any_sync(on, (uint32_t)(at >> 7) << 5 | (unsigned)(lane * m >> 5))) - 1;
-                const uint32_t h = ((uint32_t)(at / sector) * 0x9e3779b1u) >> 14;  // (18 bits: kSpreadBits)
+            if (c >= 0) {
+                const uint32_t h = ((uint32_t)(at >> shift) * 0x9e3779b1u) >> 14;  // (18 bits: kSpreadBits)
                 if (!((*(volatile uint32_t *)&seen[h >> 5] >> (h & 31)) & 1u)) atomicOr(&seen[h >> 5], 1u << (h & 31));
             }
-            lines += __popc(__ballot_sync(0xffffffffu, first));
+            if (look) {
+                lines += __popc(__ballot_sync(0xffffffffu, first));
+                looked += __popc(on);
+            }
             taken += __popc(on);
         });
     }
     if (lane == 0) {
         atomicAdd(&s_lines, lines);
+        atomicAdd(&s_looked, looked);
         atomicAdd(&s_rows, taken);
     }
     __syncthreads();
@@ -676,6 +684,7 @@ __device__ __forceinline__ void spread_sample(int64_t nslices, int per, const R 
     __syncthreads();
     if (threadIdx.x == 0) {
         atomicAdd(&out->lines, (unsigned long long)s_lines);
+        atomicAdd(&out->looked, (unsigned long long)s_looked);
         atomicAdd(&out->rows, (unsigned long long)s_rows);
         const float clear = fmaxf(1.0f, (float)(kSpreadBits - s_set)) / kSpreadBits;  // linear counting
         atomicAdd(&out->bytes, -logf(clear) * (float)kSpreadBits * (float)sector);
@@ -733,7 +742,7 @@ struct SpreadSample {
         MPK_CUDA(cudaStreamSynchronize(s));
         for (int q = 0; q < 2; ++q) {
             const double rows = (double)std::max<unsigned long long>(h[q].rows, 1);
-            at[q].lines = (double)h[q].lines / rows;
+            at[q].lines = (double)h[q].lines / (double)std::max<unsigned long long>(h[q].looked, 1);
             at[q].bytes = (double)h[q].bytes / std::max(1, q ? plan : nat);
             at[q].fresh = (double)h[q].bytes / (rows * xbytes);
             at[q].lead = P.val_bytes == 8 && P.m == 4;

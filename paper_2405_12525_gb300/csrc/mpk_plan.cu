@@ -710,11 +710,11 @@ struct Spread {
     // 1.0 (spin chain 0.25 lines: 0.58 to 0.74); above, up to 47 KB: 0.7 to 0.95 (banded graph of 100k rows, 31
     // KB; a permuted grid of 1400^2, 41 KB: 1.57); above, little of it fresh: 0.8 to 1.04 (the same, 2 columns, 62
     // KB, 0.13; of 300k rows, 60 KB, 0.25: 0.92); the rest 1.0 to 2.9, but for 63^3 in windows of 1000 rows (69 KB,
-    // 0.6): 0.92.  binary64 values with 4 columns need the lead more: banded graphs (0.23 to 0.45) 0.97, permuted
+    // 0.6): 0.92.  binary64 values with 4 columns need the lead more: banded graphs (0.23 to 0.54) 0.96, permuted
     // grids (above) 1.06 to 1.2.
     bool lead = false;
     bool scattered() const {
-        return lines > 0.62 && bytes > 47e3 && (lead ? fresh > 0.5 : fresh > 0.3 || (fresh > 0.22 && bytes > 96e3));
+        return lines > 0.62 && bytes > 47e3 && (lead ? fresh > 0.56 : fresh > 0.3 || (fresh > 0.22 && bytes > 96e3));
     }
 };
 // Of A's numbering (at[0], if asked for) and of the plan order (at[1]): measured on the stream by the

@@ -74,8 +74,8 @@ constexpr int kStagedWidth = 64;  // entries a row of the widest slice that the 
 // 200 KB let the copies run furthest ahead (96 KB: structured binary64 grids the same, others 5 to
 // 30 % slower), but leave 28 KB of L1, in whose lines the gathers in flight wait for L2.  Gathers that
 // touch a line a row then queue for lines: with 96 KB a grid of 126^3 with its rows shuffled, p = 8, plan
-// order, takes 409 in place of 889 us (binary64), 463 in place of 804 us (bfloat16; the ticketed kernel,
-// whose blocks stage less: 464).  A set of tables says which of the two its gathers need (WaveSet::scattered).
+// order, takes 381 in place of 839 us (binary64), 407 in place of 714 us (bfloat16; the ticketed kernel,
+// whose blocks stage less: 417).  A set of tables says which of the two its gathers need (WaveSet::scattered).
 constexpr int kWaveBytes = 200 * 1024, kWaveBytesScattered = 96 * 1024;
 template <class VT> struct WaveBuf {
     static constexpr int ENTRY = (int)sizeof(typename VT::T) + 4;

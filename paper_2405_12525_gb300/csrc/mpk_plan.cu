@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <cstddef>
 #include <memory>
 
 namespace mpk {
@@ -447,6 +448,16 @@ __global__ void k_slice_records(const int64_t *sptr, const int32_t *width, const
     }
 }
 
+// How the gathers of x spread, from samples of up to 2048 rows (64 slices; of fewer when they hold over
+// 64 K entries): `lines` / `looked`, the 128-byte lines that a gather of one entry of a unit's rows touches,
+// per row (looked at for one entry in four: comparing lanes takes most of the kernel's time), and `bytes`,
+// those of the different 32-byte sectors that a sample's entries read (counted in a bitmap of hashes, by the
+// bits left free), of `rows` gathered rows.
+struct GatherSpread {
+    unsigned long long lines, looked, rows;
+    float bytes;  // of all samples
+};
+
 // Different values of a matrix, as bit patterns in an open hash table; given up beyond kDictSize.
 constexpr int kDictSlots = 4 * kDictSize;
 constexpr unsigned long long kNoValue = 0x7ff8a5c3e1f00d01ULL;  // (a NaN; a matrix holding it is given up)
@@ -454,7 +465,8 @@ struct Dict {
     unsigned long long key[kDictSlots];
     int32_t index[kDictSlots];  // number of the slot's value
     double value[kDictSize];
-    int32_t count, over;
+    int32_t count, over;     // (read back together with what follows)
+    GatherSpread spread[2];  // of A's numbering and of the plan order
 };
 __device__ __forceinline__ unsigned long long value_bits(double v) { return (unsigned long long)__double_as_longlong(v); }
 __device__ __forceinline__ unsigned long long value_bits(float v) { return __float_as_uint(v); }
@@ -464,6 +476,7 @@ __global__ void k_dict_init(Dict *d) {
     for (int i = threadIdx.x; i < kDictSlots; i += blockDim.x) d->key[i] = kNoValue;
     for (int i = threadIdx.x; i < kDictSize; i += blockDim.x) d->value[i] = 0.0;
     if (threadIdx.x == 0) d->count = d->over = 0;
+    if (threadIdx.x < 2) d->spread[threadIdx.x] = GatherSpread{0, 0, 0, 0.0f};
 }
 template <class T> __global__ void k_dict(int64_t nnz, const T *va, Dict *d) {
     __shared__ unsigned long long seen[kDictSlots];  // the block's own table: most entries end here
@@ -595,15 +608,6 @@ __global__ void k_pack_fill(int32_t nslices, R rows, const T *va, const int32_t 
     }
 }
 
-// How the gathers of x spread, from samples of up to 2048 rows (64 slices; of fewer when they hold over
-// 64 K entries): `lines` / `looked`, the 128-byte lines that a gather of one entry of a unit's rows touches,
-// per row (looked at for one entry in four: comparing lanes takes most of the kernel's time), and `bytes`,
-// those of the different 32-byte sectors that a sample's entries read (counted in a bitmap of hashes, by the
-// bits left free), of `rows` gathered rows.
-struct GatherSpread {
-    unsigned long long lines, looked, rows;
-    float bytes;  // of all samples
-};
 constexpr int kSpreadSlices = 64, kSpreadEntries = 1 << 16, kSpreadSamples = 64, kSpreadBits = 1 << 18;
 // rows of A (32 consecutive ones a slice)
 struct CsrSlices {
@@ -717,39 +721,6 @@ struct Spread {
         return lines > 0.62 && bytes > 47e3 && (lead ? fresh > 0.56 : fresh > 0.3 || (fresh > 0.22 && bytes > 96e3));
     }
 };
-// Of A's numbering (at[0], if asked for) and of the plan order (at[1]): measured on the stream by the
-// constructor, read by read(), which waits for it.
-struct SpreadSample {
-    const Plan &P;
-    cudaStream_t s;
-    Tmp<GatherSpread> d;
-    int per, xbytes, nat = 0, plan = 0;
-    SpreadSample(const Plan &plan_, const mpk_csr *A, bool natural, cudaStream_t s_) : P(plan_), s(s_), d(2, s_) {
-        per = (int)std::max<int64_t>(1, std::min<int64_t>(kSpreadSlices, kSpreadEntries / (32 * (P.nnz / P.n + 1))));
-        xbytes = (P.accum == MPK_F32 ? 4 : 8) * P.m;
-        auto samples = [&](int64_t nslices) { return (int)std::max<int64_t>(1, std::min<int64_t>(kSpreadSamples, nslices / per)); };
-        const int64_t ns = ((int64_t)P.n + 31) / 32;
-        nat = natural ? samples(ns) : 0;
-        plan = samples(P.num_slices);
-        MPK_CUDA(cudaMemsetAsync(d.p, 0, 2 * sizeof(GatherSpread), s));
-        k_gather_spread<<<nat + plan, 1024, 0, s>>>(nat, ns, CsrSlices{A->row_ptr, A->col, P.n}, P.num_slices,
-                                                    PlanSlices{P.slice_ptr, P.col}, per, P.m, xbytes, d.p);
-        MPK_LAUNCHED();
-    }
-    void read(Spread (&at)[2]) {
-        GatherSpread h[2];
-        MPK_CUDA(cudaMemcpyAsync(h, d.p, sizeof(h), cudaMemcpyDeviceToHost, s));
-        MPK_CUDA(cudaStreamSynchronize(s));
-        for (int q = 0; q < 2; ++q) {
-            const double rows = (double)std::max<unsigned long long>(h[q].rows, 1);
-            at[q].lines = (double)h[q].lines / (double)std::max<unsigned long long>(h[q].looked, 1);
-            at[q].bytes = (double)h[q].bytes / std::max(1, q ? plan : nat);
-            at[q].fresh = (double)h[q].bytes / (rows * xbytes);
-            at[q].lead = P.val_bytes == 8 && P.m == 4;
-        }
-    }
-};
-
 // A run of groups whose powers are computed together: a whole plan, or an instance of a batch plan
 struct WaveRange {
     int32_t g0, g1;  // groups
@@ -821,25 +792,51 @@ static bool wave_tables(Plan &P, WaveSet &w, const std::vector<int32_t> &vs, con
     return true;
 }
 
-// The table of A's values; false if there are more than kDictSize (a matrix of random values is given
-// up after its first entries).  The set-up takes as long with packed copies as without: what the
-// table costs, the smaller copy saves (131 x 127 x 113: 5.29 against 5.35 ms).
-static bool find_values(const Plan &P, const mpk_csr *A, Dict *d, cudaStream_t s) {
+// What the choice of copies and buffers rests on, with one wait for the device: the spread of the gathers in
+// A's numbering (at[0], if `natural`) and in plan order (at[1]), if `spread`; and, if `values`, the table of
+// A's values in d, false if there are more than kDictSize (a matrix of random values is given up after its
+// first entries).  The set-up takes as long with packed copies as without: what the table costs, the smaller
+// copy saves (131 x 127 x 113: 5.29 against 5.35 ms).
+static bool look_over(const Plan &P, const mpk_csr *A, bool spread, bool natural, Spread (&at)[2], bool values, Dict *d,
+                      cudaStream_t s) {
     k_dict_init<<<1, 1024, 0, s>>>(d);
     MPK_LAUNCHED();
-    if (P.val_type == MPK_F64)
-        k_dict<<<grid_n(A->nnz), 256, 0, s>>>(A->nnz, static_cast<const double *>(A->val), d);
-    else if (P.val_type == MPK_F32)
-        k_dict<<<grid_n(A->nnz), 256, 0, s>>>(A->nnz, static_cast<const float *>(A->val), d);
-    else
-        k_dict<<<grid_n(A->nnz), 256, 0, s>>>(A->nnz, static_cast<const uint16_t *>(A->val), d);
-    MPK_LAUNCHED();
-    k_dict_number<<<1, 1024, 0, s>>>(d, P.val_type);
-    MPK_LAUNCHED();
-    int32_t found[2];  // number, given up
-    MPK_CUDA(cudaMemcpyAsync(found, &d->count, sizeof(found), cudaMemcpyDeviceToHost, s));
+    const int per = (int)std::max<int64_t>(1, std::min<int64_t>(kSpreadSlices, kSpreadEntries / (32 * (P.nnz / P.n + 1))));
+    const int xbytes = (P.accum == MPK_F32 ? 4 : 8) * P.m;
+    auto samples = [&](int64_t nslices) { return (int)std::max<int64_t>(1, std::min<int64_t>(kSpreadSamples, nslices / per)); };
+    const int64_t ns = ((int64_t)P.n + 31) / 32;
+    const int nat = natural ? samples(ns) : 0, plan = samples(P.num_slices);
+    if (spread) {
+        k_gather_spread<<<nat + plan, 1024, 0, s>>>(nat, ns, CsrSlices{A->row_ptr, A->col, P.n}, P.num_slices,
+                                                    PlanSlices{P.slice_ptr, P.col}, per, P.m, xbytes, d->spread);
+        MPK_LAUNCHED();
+    }
+    if (values) {
+        if (P.val_type == MPK_F64)
+            k_dict<<<grid_n(A->nnz), 256, 0, s>>>(A->nnz, static_cast<const double *>(A->val), d);
+        else if (P.val_type == MPK_F32)
+            k_dict<<<grid_n(A->nnz), 256, 0, s>>>(A->nnz, static_cast<const float *>(A->val), d);
+        else
+            k_dict<<<grid_n(A->nnz), 256, 0, s>>>(A->nnz, static_cast<const uint16_t *>(A->val), d);
+        MPK_LAUNCHED();
+        k_dict_number<<<1, 1024, 0, s>>>(d, P.val_type);
+        MPK_LAUNCHED();
+    }
+    struct {
+        int32_t count, over;
+        GatherSpread spread[2];
+    } h;
+    static_assert(sizeof(h) == sizeof(Dict) - offsetof(Dict, count), "the end of the table");
+    MPK_CUDA(cudaMemcpyAsync(&h, &d->count, sizeof(h), cudaMemcpyDeviceToHost, s));
     MPK_CUDA(cudaStreamSynchronize(s));
-    return !found[1] && found[0] <= kDictSize;
+    for (int q = 0; q < 2; ++q) {
+        const double rows = (double)std::max<unsigned long long>(h.spread[q].rows, 1);
+        at[q].lines = (double)h.spread[q].lines / (double)std::max<unsigned long long>(h.spread[q].looked, 1);
+        at[q].bytes = (double)h.spread[q].bytes / std::max(1, q ? plan : nat);
+        at[q].fresh = (double)h.spread[q].bytes / (rows * xbytes);
+        at[q].lead = P.val_bytes == 8 && P.m == 4;
+    }
+    return values && !h.over && h.count <= kDictSize;
 }
 
 // The packed copy of the slices `rows` (values at `val`); width and units: scratch of a word a slice.
@@ -1026,22 +1023,18 @@ static void plan_wave(Plan &P, const mpk_csr *A, int32_t band, const std::vector
                    std::min<int64_t>(n, 2 * (int64_t)band + 32) * 8 * P.m <= device_l2_bytes() / 4;
     // (not looked at where the large buffer is as good: 8 and 16 columns within 3 %, up to 32768 rows of
     // one column the same)
-    std::unique_ptr<SpreadSample> sample;
+    const bool look = P.m <= 4 && (int64_t)n * P.m > 32768;
+    Spread spread[2];
     std::unique_ptr<Tmp<Dict>> table;
     bool packed = false;
-    try {
-        if (P.m <= 4 && (int64_t)n * P.m > 32768) sample.reset(new SpreadSample(P, A, natural, s));
-        if (pack) {
+    if (look || pack) try {
             table.reset(new Tmp<Dict>(1, s));
-            packed = find_values(P, A, table->p, s);
+            packed = look_over(P, A, look, natural, spread, pack, table->p, s);
+        } catch (const Fail &f) {  // no memory for the table: the plan does without
+            if (f.status != MPK_ERR_OOM) throw;
+            cudaGetLastError();
         }
-    } catch (const Fail &f) {  // no memory for them: the plan does without
-        if (f.status != MPK_ERR_OOM) throw;
-        cudaGetLastError();
-    }
     const Dict *dict = packed ? table->p : nullptr;
-    Spread spread[2];
-    if (sample) sample->read(spread);
     // A numbering whose gathers are scattered where the levels' are not is left to the plan order: one
     // column, more rows than the gather and scatter of the vectors make up for.  Time of k_mpk, as it was
     // before this kernel, over A's numbering / plan order (96 KB buffers), apply p = 8 and a recurrence of

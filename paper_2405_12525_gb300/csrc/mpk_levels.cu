@@ -80,8 +80,9 @@ __global__ void k_tfill(int32_t n, const int32_t *rp, const int32_t *ci, int32_t
 // (Claims without a look at the level first, and prefetches of the winners' columns: slower.)
 // A graph whose search runs dry before every vertex is reached continues from the smallest
 // untouched vertex, which opens the next level: block 0 looks for it beside the narrow levels
-// (20000 vertices without edges: 27 ms; by the grid alone 166 to 187), the grid when it is not among the next kBfsNear *
-// kBfsBS (a grid-wide minimum, one barrier, and one more to publish it); the minima rotate through three slots, so that a slot is reset only
+// (20000 vertices without edges: 27 ms; by the grid alone 166 to 187), the grid when it is not among
+// the next kBfsNear * kBfsBS (a grid-wide minimum, one barrier, and one more to publish it); the
+// minima rotate through three slots, so that a slot is reset only
 // after its last readers passed the next barrier.  Every barrier wait is bounded; on expiry the
 // kernel records the failure and all blocks leave.
 constexpr int64_t kBfsWaitNs = 2000000000LL;  // bound of one grid-barrier wait (2 s)

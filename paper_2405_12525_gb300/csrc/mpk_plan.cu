@@ -644,11 +644,11 @@ struct PlanSlices {
         }
     }
 };
-// Sample `block` of `blocks`, of `per` slices; xbytes: of a row of x (all its columns)
+// Sample `block` of `blocks`, of `per` slices; xbytes: of a row of x (all its columns); seen: the bitmap, in
+// shared memory
 template <class R>
 __device__ __forceinline__ void spread_sample(int64_t nslices, int per, const R &rows, int m, int xbytes, int block, int blocks,
-                                              GatherSpread *out) {
-    __shared__ uint32_t seen[kSpreadBits / 32];
+                                              uint32_t *seen, GatherSpread *out) {
     __shared__ int s_lines, s_looked, s_rows, s_set;
     for (int i = threadIdx.x; i < kSpreadBits / 32; i += blockDim.x) seen[i] = 0;
     if (threadIdx.x == 0) s_lines = s_looked = s_rows = s_set = 0;
@@ -697,10 +697,11 @@ __device__ __forceinline__ void spread_sample(int64_t nslices, int per, const R 
 // samples in A's numbering into out[0], then of the plan's slices into out[1]
 __global__ void __launch_bounds__(1024) k_gather_spread(int nat_samples, int64_t nat_slices, CsrSlices nat, int64_t nslices,
                                                         PlanSlices plan, int per, int m, int xbytes, GatherSpread *out) {
+    __shared__ uint32_t seen[kSpreadBits / 32];
     if ((int)blockIdx.x < nat_samples)
-        spread_sample(nat_slices, per, nat, m, xbytes, blockIdx.x, nat_samples, out);
+        spread_sample(nat_slices, per, nat, m, xbytes, blockIdx.x, nat_samples, seen, out);
     else
-        spread_sample(nslices, per, plan, m, xbytes, blockIdx.x - nat_samples, gridDim.x - nat_samples, out + 1);
+        spread_sample(nslices, per, plan, m, xbytes, blockIdx.x - nat_samples, gridDim.x - nat_samples, seen, out + 1);
 }
 
 // The spread of an order, per row and sample: lines a row, bytes of a sample, and those as a part of the

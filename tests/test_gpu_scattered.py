@@ -191,3 +191,36 @@ def test_a_numbering_without_locality_is_left_to_the_levels(mpk, dtype, accum):
         P = mpk.plan(A, L, p_max=8, shape=shape, accum=accum)
         t[shape] = _time(lambda: P.cheb_filter(X, 32, c, scale=13.0, shift=6.0, out=out))
     assert t[0] < 1.25 * min(t[1], t[2]), t
+
+
+@pytest.mark.parametrize("cache_bytes", [0, 4000000])
+@pytest.mark.parametrize("val,accum", [("f64", 0), ("bf16", 1)])
+def test_original_order_through_the_levels(mpk, cache_bytes, val, accum):
+    """70^3 (343000 rows) shuffled in windows of 10 000: gathered into the levels' order, computed there
+    and scattered, bit for bit: powers, into host memory too, the recurrence, whole and in pieces."""
+    A = _shuffled_grid(mpk, 70, 10000, torch.float64 if val == "f64" else torch.bfloat16)
+    host = gen.CSR(A.row_ptr.cpu().numpy(), A.col.cpu().numpy(), A.val.double().cpu().numpy())
+    L = mpk.build_levels(A, 0)
+    P = mpk.plan(A, L, p_max=5, accum=accum, cache_bytes=cache_bytes)
+    X = gen.vector(A.n, 1, stream=9)
+    Xd = torch.from_numpy(X).cuda()
+    want = oracle.mpk_acc32(host, X, 5) if accum else oracle.mpk(host, X, 5)
+    Y = torch.full((6, A.n, 1), float("nan"), dtype=torch.float64, device="cuda")
+    for p in (5, 1):
+        Y.fill_(float("nan"))
+        P.apply(Xd, p, Y=Y)
+        P.sync_status()
+        _same(Y[:p + 1].cpu().numpy(), want[:p + 1])
+    Yh = P.apply_host(torch.from_numpy(X).pin_memory(), 5)
+    torch.cuda.synchronize()
+    P.sync_status()
+    _same(Yh.numpy(), want)
+    if not accum:
+        c = np.linspace(1.0, -0.5, 9)
+        ref = oracle.cheb(host, X, 8, c, scale=13.0, shift=6.0)
+        _same(P.cheb_filter(Xd, 8, c, scale=13.0, shift=6.0).cpu().numpy(), ref)
+        S = P.cheb_begin(Xd, P.cheb_state(), c[0])
+        P.cheb_advance(S, 0, 3, c, scale=13.0, shift=6.0)
+        P.cheb_advance(S, 3, 8, c, scale=13.0, shift=6.0)
+        _same(P.cheb_finish(S).cpu().numpy(), ref)
+        P.sync_status()
